@@ -78,13 +78,13 @@ enum { VQMC_PREC_FP32 = 0, VQMC_PREC_BF16 = 1 };
 /* Sampler implementation (vqmc_config.sampler).  All draw the same exact
  * samples of the model (Algorithm 1) from the same uniforms.
  *   AUTO: TENSOR_CORE where it applies, else CUDA_CORE.
- *   CUDA_CORE: one step at a time, FP32 FMAs on the CUDA cores; any model
- *     with h <= 5120 (BF16 weights) or h <= 2816 (FP32 weights).  Up to
- *     h = 2048 a CTA carries 16 samples; beyond, 4.
- *   CUDA_CORE_WIDE: the CUDA-core sampler with the layout it uses beyond
- *     h = 2048 (groups of four warps split the hidden units, 4 samples per
- *     CTA) at any h: four times the CTAs, fewer registers per sample; the
- *     batch autotuner chooses between the two per member.
+ *   CUDA_CORE: FP32 FMAs on the CUDA cores, in blocks of up to 16 steps; any
+ *     model with h <= 5120 (BF16 weights) or h <= 2816 (FP32 weights).  A CTA
+ *     carries 8 samples.
+ *   CUDA_CORE_WIDE: the CUDA-core sampler with the summation order it uses
+ *     beyond h = 2048 (four runs of 64 units instead of two or one: the FP32
+ *     rounding of a logit differs) at any h; the batch autotuner chooses
+ *     between the two per member.
  *   TENSOR_CORE: blocks of 64 or 128 steps whose bulk work (the logits from
  *     hidden units completed before the block, and the update of hidden
  *     units by the block's spins) runs as tcgen05 GEMMs, with a sequential
@@ -412,8 +412,8 @@ vqmc_status vqmc_batch_graph_launch(vqmc_batch* batch, vqmc_stream stream, vqmc_
 
 /* Autotuner of the batch's schedule.  First it measures one iteration of
  * each member alone; a member on the CUDA-core sampler with at most 2048
- * hidden units is timed in both of its layouts (16 samples per CTA, and the
- * wide one of VQMC_SAMPLER_CUDA_CORE_WIDE) and keeps the faster.  Then it
+ * hidden units is timed in both of its summation orders (its own, and that of
+ * VQMC_SAMPLER_CUDA_CORE_WIDE) and keeps the faster.  Then it
  * times one captured batched iteration (graph replays) under each candidate
  * schedule -- 1, 2, 4, ... up to the batch's internal streams, with members
  * assigned round-robin in index order or longest first onto the

@@ -35,10 +35,11 @@ __host__ __device__ inline int count_deg_le(int x, int n, int h) {
   return c > h ? h : (int)c;
 }
 
-// The sampler streams SPS consecutive rows per copy; its weight copies have
-// this many rows (wt_s row j = input j with row 0 zero, v_s row i = output i+1).
+// The samplers read rows in groups: their weight copies have zero rows past the
+// model's (wt_s row j = input j with row 0 zero, v_s row i = output i+1), up to
+// three rows past the last one they need, in multiples of 8.
 constexpr int kSamplerRowsPad = 8;
-inline int sampler_rows(int n) { return (n + 1 + kSamplerRowsPad - 1) / kSamplerRowsPad * kSamplerRowsPad; }
+inline int sampler_rows(int n) { return (n + 3 + kSamplerRowsPad - 1) / kSamplerRowsPad * kSamplerRowsPad; }
 
 // Device error word bits mirror VQMC_DEVERR_*.
 constexpr uint32_t kErrTimeout = VQMC_DEVERR_TIMEOUT;
@@ -88,7 +89,7 @@ struct vqmc_ctx {
   int act, prec;   // VQMC_ACT_*, VQMC_PREC_*
   int ham;         // VQMC_HAM_*
   int sampler;     // VQMC_SAMPLER_CUDA_CORE or _TENSOR_CORE (resolved at create)
-  int sampler_wide = 0;  // CUDA-core sampler in its four-warp-group layout
+  int sampler_wide = 0;  // CUDA-core sampler in its summation order of hp > 2048
   int nnz;
   int64_t d;
   uint64_t inst_hash = 0;
@@ -195,8 +196,8 @@ struct vqmc_ctx {
 namespace vqmc {
 
 // ---- sampler_bf16.cu / sampler_f32.cu: whether the CUDA-core sampler runs
-// models with hp padded hidden units and weights of type WT (its register
-// layout and shared-memory ring bound hp), in its default or wide layout
+// models with hp padded hidden units and weights of type WT, in its default
+// or wide summation order
 template <typename WT>
 bool sampler_wt_supports(int hp, bool wide);
 // ---- sampler.cu

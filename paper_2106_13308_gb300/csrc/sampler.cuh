@@ -9,8 +9,7 @@ namespace vqmc {
 struct SamplerArgs {
   int n, h, hp, B;
   int act;          // VQMC_ACT_*
-  int nst;          // ring stages
-  int wide;         // 1: the four-warp-group layout (4 samples per CTA) at any hp
+  int wide;         // 1: the summation order of hp > 2048 at any hp
   const void* wt;   // [n][hp]
   const void* v;    // [n][hp]
   const float* b1;  // [h]

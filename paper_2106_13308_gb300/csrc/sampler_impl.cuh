@@ -1,5 +1,42 @@
-// Implementation of the persistent sampler kernel, included by one
+// Blocked autoregressive sampler on the CUDA cores, included by one
 // translation unit per weight type (sampler_bf16.cu, sampler_f32.cu).
+//
+// Algorithm 1 with the incremental forward pass (Sec. 2.3): the logit of step
+// e (0-based) is
+//     z_e = b2_e + sum_{k complete} W2_ek g1_k,   g1_k = act(b1_k + sum_{j<m(k)} W1_kj s_j),
+// and with sorted degrees the complete units are a prefix.  A CTA draws 8
+// samples.  The hidden units go in groups of 16 in degree order; the steps
+// whose newest complete unit lies in group g ("the group's steps") are taken
+// in blocks of at most 16, each in three phases:
+//   Z  the terms of every unit before group g in the block's logits, a small
+//      GEMM (steps x samples over the complete units) on all warps;
+//   solve  two warps draw the block's spins one after another, carrying the
+//      pre-activations of group g's 16 units (the only ones that complete
+//      inside the block), 8 lanes per sample; the other warps meanwhile stage
+//      the next block's tables and write the previous block's outputs;
+//   U  the block's spins into the pre-activations of the units after group g,
+//      a second small GEMM on all warps.
+// All pre-activations (g1 once complete) of the CTA's samples stay in shared
+// memory; the weights are read once per CTA from L2.
+//
+// The order of every FP32 operation is fixed by h alone.  A
+// pre-activation is summed over the inputs in order.  A logit is summed as
+// GW*64 chains over the units k = c, c + GW*64, c + 2 GW*64, ... (c the
+// class of a unit), the chains of classes 2l and 2l + 1 added, then for each
+// run of 32 such pairs ("virtual warp") a binary tree over l that joins l
+// with l ^ 16 first, then ^ 8, 4, 2, 1, and the GW results added to b2 in
+// order.  GW is 1 up to hp = 64, 2 up to 2048 and 4 beyond.  Group g holds 8
+// neighbouring pairs (one octet) of one virtual warp, so the solver finishes
+// the tree from its 8 leaves and the partial sums of the other octets.
+//
+// What bounds it: the chain from one draw to the next (about 250 cycles, on two
+// of the CTA's eight warps) up to about 1000 hidden units, beyond it the issue
+// slots and shared-memory reads of the Z and U phases (2 bytes per multiply-add);
+// two CTAs on an SM overlap one's draws with the other's GEMMs.  Measured
+// (GB300), against one step at a time with a reduction over the CTA's lanes for
+// every draw: n = h = 1000, 1024 samples (BF16) 1440 -> 320 us; n = h = 2000,
+// 8192 samples 8580 -> 3990 us; n = 10000, h = 2000, 2048 samples (FP32) 7780 ->
+// 5600 us (15 TFLOP/s).
 #pragma once
 
 #include "sampler.cuh"
@@ -8,68 +45,15 @@ namespace vqmc {
 
 namespace {
 
-
-// ------------------------------------------------------- PTX: mbarrier/bulk
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait: false (and the timeout bit set) if the phase never completed.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t* err) {
-  for (long long it = 0; it < kSpinLimit; ++it)
-    if (mbar_try_wait(bar, parity)) return true;
-  atomicOr(err, kErrTimeout);
-  return false;
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-
-// ------------------------------------------------------------------ helpers
-
-template <typename T>
-__device__ __forceinline__ T from_f(float x);
-template <>
-__device__ __forceinline__ float from_f<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ bf16 from_f<bf16>(float x) { return __float2bfloat16_rn(x); }
-
-constexpr int kBig = 0x3fffffff;
-
+constexpr int kSamples = 8;      // samples per CTA
+constexpr int kSteps = 16;       // steps per block
+constexpr int kGroup = 16;       // hidden units per group
+constexpr int kLeaves = kGroup / 2;
+constexpr int kTI = 4;           // steps per Z task
+constexpr int kWarps = 8;
+constexpr int kSolvers = 2;      // warps that draw, 4 samples each: the last ones
+constexpr int kThreads = 32 * kWarps;
+constexpr int kChunk = 64;       // units per chunk of the state
 
 // ---- packed FP32 pairs (fma.rn.f32x2: two IEEE FP32 FMAs in one instruction)
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
@@ -80,544 +64,642 @@ __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
 __device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
+__device__ __forceinline__ float sum2(uint64_t v) {
+  float lo, hi;
+  unpack2(v, lo, hi);
+  return lo + hi;
+}
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-
-// Weights of units (2q, 2q+1) of a staged row: raw (as stored) and as an
-// FP32 pair.  BF16 widens exactly by a shift.
-template <typename T>
-struct Pair;
-template <>
-struct Pair<bf16> {
-  using raw = uint32_t;
-  static __device__ __forceinline__ raw ld(const bf16* row, int q) { return reinterpret_cast<const uint32_t*>(row)[q]; }
-  static __device__ __forceinline__ uint64_t f32(raw x) {
-    return pack2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
-  }
-};
-template <>
-struct Pair<float> {
-  using raw = uint64_t;
-  static __device__ __forceinline__ raw ld(const float* row, int q) { return reinterpret_cast<const uint64_t*>(row)[q]; }
-  static __device__ __forceinline__ uint64_t f32(raw x) { return x; }
-};
-template <typename T>
-__device__ __forceinline__ uint64_t ld_pair(const T* row, int q) {
-  return Pair<T>::f32(Pair<T>::ld(row, q));
+// 16 bytes from global to shared memory (zeros if !in), asynchronously
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {  // all but the last N groups have landed
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// lane 0's value, which the compiler then knows to be the same in all lanes: it
+// keeps the control flow that depends on it free of the reconvergence code
+// that a shuffle behind a possibly divergent branch costs (some 8 instructions)
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
+// 16 bytes to shared memory if in: one predicated store (a divergent branch
+// around it costs about 70 cycles)
+__device__ __forceinline__ void st16_if(uint32_t dst, uint64_t x, uint64_t y, bool in) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %3, 0;\n\t@q st.shared.v2.b64 [%0], {%1, %2};\n\t}" ::"r"(dst), "l"(x),
+               "l"(y), "r"((int)in)
+               : "memory");
+}
 
-// A CTA = NGRP groups of GW warps.  Group g owns
-// SL samples; its GW*32 lanes split the hidden units: lane L of the group
-// holds unit pairs q = r*GW*32 + L (units 2q, 2q+1), r = 0..U2-1, for all SL
-// samples.  Per step a group reduces its partial sums with shuffles and one
-// named barrier of its own warps; groups never wait for each other.  Lane 0
-// of the last warp also keeps the weight ring filled: whenever every warp
-// has released a stage it issues the copies for the block a full ring ahead.
-template <typename WT, int GW, int NGRP, int U2, int SL>
-struct Sampler {
-  static constexpr int NCW = GW * NGRP;      // warps
-  static constexpr int NT = NCW * 32;        // threads
-  static constexpr int S = SL * NGRP;        // samples per CTA
-  static constexpr int GL = GW * 32;         // lanes per group
-  static constexpr int RL = GL * 2 * U2;     // units covered (row length in smem)
-  static constexpr int SPS = 4;              // steps per ring stage (rows per copy)
-  static constexpr int UWIN = 128 / SL;      // steps per uniform window (32 lanes x 4 words)
-  static_assert(SL >= 1 && SL <= 16 && (SL & (SL - 1)) == 0, "SL must be a power of two <= 16");
+// Weights as stored: those of one pair of units (2q, 2q + 1), and of four
+// consecutive units (two pairs); widened to FP32 pairs (BF16 by a shift).
+template <typename T>
+struct Raw;
+template <>
+struct Raw<bf16> {
+  using two = uint32_t;
+  using four = unsigned long long;
+  static __device__ __forceinline__ uint64_t f32(two x) {
+    return pack2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
+  }
+  static __device__ __forceinline__ uint64_t lo(const four& x) { return f32((uint32_t)x); }
+  static __device__ __forceinline__ uint64_t hi(const four& x) { return f32((uint32_t)(x >> 32)); }
+};
+template <>
+struct Raw<float> {
+  using two = uint64_t;
+  using four = ulonglong2;
+  static __device__ __forceinline__ uint64_t f32(two x) { return x; }
+  static __device__ __forceinline__ uint64_t lo(const four& x) { return x.x; }
+  static __device__ __forceinline__ uint64_t hi(const four& x) { return x.y; }
+};
 
-  struct State {
-    uint64_t a[U2][SL];  // pre-activations of units (2q, 2q+1), or act() once complete
-    uint64_t acc[SL];    // dot accumulators (even / odd units)
-    uint64_t sg[SL];     // {s_{i-1}, s_{i-1}}
+// The tables of one block that the solver reads, staged during the previous
+// block's draws.
+struct Leaf {       // one pair of the group's units at one step
+  uint64_t v, w;    // W2 (this step's output) and W1 (this step's input)
+};
+struct LeafSum {    // one leaf of one sample at one step
+  uint64_t pre;     // the pair's two chains over the units before the group
+  uint64_t join;    // {the sum that joins the leaf on the tree's first level, on the second}
+};
+struct Tables {
+  Leaf leaf[kSteps][kLeaves];
+  float logit[kSteps][kSamples];        // logit(u)
+  float b2[kSteps];
+  int done[kSteps];                     // units of the group complete at the step
+};
+// What a block's draws leave for the outputs: bit t of bits[s]: spin of step
+// e0 + t is +1; s_e z_e for log pi.
+struct Drawn {
+  float x[kSteps * kSamples];
+  uint32_t bits[kSamples];
+};
+
+// Steps [e0, e1) of group grp.
+struct Block {
+  int e0, e1, grp, pad;
+};
+
+// count_deg_le and degree in 32 bits: n h < 2^32 for every model whose
+// weights fit the GPU (h <= 5120).
+__device__ __forceinline__ int complete_before(int e, int n, int h) {  // units with m(k) <= e
+  if (e < 1) return 0;
+  if (n <= 1) return h;
+  return min((int)(((unsigned)e * (unsigned)h + (unsigned)(n - 2)) / (unsigned)(n - 1)), h);
+}
+__device__ __forceinline__ Block next_block(int e0, int n, int h) {
+  Block b;
+  b.e0 = e0;
+  b.grp = complete_before(e0, n, h) / kGroup;
+  const int last = kGroup * b.grp + kGroup - 1;  // the group's last unit is complete from step degree(last) on
+  const int e1 = last < h ? 1 + (int)((unsigned)last * (unsigned)(n - 1) / (unsigned)h) : n;
+  b.e1 = min(min(e1, n), e0 + kSteps);
+  b.pad = 0;
+  return b;
+}
+
+template <typename WT, int GW, bool RELU>
+struct BlockSampler {
+  static constexpr int GL = GW * 32;  // pair classes
+  static constexpr int RL = GW * 64;  // classes
+  // a logit is ((zb + the group's tree) + post[0]) + ...
+  struct Post {
+    float zb, lg, post[GW == 4 ? 6 : 2];
   };
 
-  static __device__ __forceinline__ int deg(int k, int n, int h) { return k < h ? degree(k, n, h) : kBig; }
+  // The weights reach shared memory through a ring per warp (cp.async, no
+  // other warp involved): a stage holds 4 rows x 64 units of W2 (one round of
+  // Z) or 2 rows x 128 units of W1 (2 steps of a round of U).
+  static constexpr int kStageBytes = 256 * (int)sizeof(WT);
+  static constexpr int kDepth = sizeof(WT) == 2 ? 4 : 2;
+  static constexpr int kRingBytes = kDepth * kStageBytes;
+
+  // shared memory (bytes).  State: chunks of 64 units x 8 samples,
+  // [chunk][sample][64], the one past hp for a group that starts at hp; a
+  // chunk of zeros stands for pairs that are not complete.
+  static constexpr int kStateChunk = kSamples * kChunk;                   // floats
+  static constexpr int kOffZ = 0;                                         // leaf records [16][8][8] (LeafSum)
+  static constexpr int kOffR = kOffZ + kSteps * kSamples * kLeaves * 16;  // ring of each warp
+  static constexpr int kOffT = kOffR + kWarps * kRingBytes;               // trees of the other virtual warps [GW][16][8]
+  static constexpr int kOffS = kOffT + GW * kSteps * kSamples * 4;        // spins {s, s} [16][8]
+  static constexpr int kOffP = kOffS + kSteps * kSamples * 8;             // what the solver adds to a tree [16][8] (Post)
+  static constexpr int kOffTab = kOffP + kSteps * kSamples * (int)sizeof(Post);  // Tables [2]
+  static constexpr int kOffDrawn = kOffTab + 2 * (int)sizeof(Tables);     // Drawn [2]
+  static constexpr int kOffNext = kOffDrawn + 2 * (int)sizeof(Drawn);     // Block [2]
+  static constexpr int kOffZero = kOffNext + 2 * (int)sizeof(Block);      // a zero chunk
+  static constexpr int kOffA = kOffZero + 4 * kStateChunk;                // state
+  static_assert(kOffTab % 16 == 0 && sizeof(Tables) % 16 == 0 && kOffNext % 16 == 0 && kOffA % 16 == 0, "alignment");
+  static size_t smem_bytes(int hp) { return kOffA + (size_t)(hp / kChunk + 1) * kStateChunk * 4; }
 
   // hidden activation as the output layer sees it: rounded to bfloat16 in
   // the BF16 model (as the BF16 forward GEMM stores it), exact in FP32
-  static __device__ __forceinline__ float g1(int g_act, float a) {
-    const float g = act_f(g_act, a);
+  static __device__ __forceinline__ float g1(float a) {
+    const float g = RELU ? fmaxf(a, 0.0f) : 1.0f / (1.0f + expf(-a));
     if constexpr (sizeof(WT) == 2) return __bfloat162float(__float2bfloat16_rn(g));
     else return g;
   }
-
-  // Mixed slot: the lane's two units may be in different roles.  Weights of
-  // units that must not take part are zeroed, so the pair still runs as f32x2.
-  // (At i = 1 the spins are still zero, so the update adds nothing.)
-  static __device__ __forceinline__ void mixed(State& st, uint64_t wpair, uint64_t vpair, int r, int i, int m0,
-                                               int m1, int g_act) {
-    if (m0 >= i - 1 || m1 >= i - 1) {
-      float w0, w1;
-      unpack2(wpair, w0, w1);
-      const uint64_t w = pack2(m0 >= i - 1 ? w0 : 0.0f, m1 >= i - 1 ? w1 : 0.0f);
-#pragma unroll
-      for (int s = 0; s < SL; ++s) st.a[r][s] = fma2(w, st.sg[s], st.a[r][s]);
-    }
-    if (m0 == i - 1 || m1 == i - 1) {
-#pragma unroll
-      for (int s = 0; s < SL; ++s) {
-        float a0, a1;
-        unpack2(st.a[r][s], a0, a1);
-        if (m0 == i - 1) a0 = g1(g_act, a0);
-        if (m1 == i - 1) a1 = g1(g_act, a1);
-        st.a[r][s] = pack2(a0, a1);
-      }
-    }
-    if (m0 <= i - 1) {
-      float v0, v1;
-      unpack2(vpair, v0, v1);
-      const uint64_t v = pack2(v0, m1 <= i - 1 ? v1 : 0.0f);
-#pragma unroll
-      for (int s = 0; s < SL; ++s) st.acc[s] = fma2(v, st.a[r][s], st.acc[s]);
-    }
+  static __device__ __forceinline__ uint64_t g1_pair(uint64_t a) {
+    float lo, hi;
+    unpack2(a, lo, hi);
+    return pack2(g1(lo), g1(hi));
   }
 
-  // Slots r < ND: every unit complete -> dot.  MIX: slot ND is mixed.
-  // Remaining slots: every unit still accumulating -> update.  wp[r] holds
-  // the W2 pair of a dot slot and the W1 pair of the others; wq the W2 pair
-  // of the mixed slot.
-  using PR = typename Pair<WT>::raw;
-  template <int ND, bool MIX>
-  static __device__ __forceinline__ void body(State& st, const PR (&wp)[U2], PR wq, int i, int m0, int m1,
-                                              int g_act) {
-#pragma unroll
-    for (int r = 0; r < ND && r < U2; ++r) {
-      const uint64_t w = Pair<WT>::f32(wp[r]);
-#pragma unroll
-      for (int s = 0; s < SL; ++s) st.acc[s] = fma2(w, st.a[r][s], st.acc[s]);
-    }
-    constexpr int FIRST_UPD = MIX ? ND + 1 : ND;
-    if constexpr (MIX && ND < U2) mixed(st, Pair<WT>::f32(wp[ND]), Pair<WT>::f32(wq), ND, i, m0, m1, g_act);
-#pragma unroll
-    for (int r = FIRST_UPD; r < U2; ++r) {
-      const uint64_t w = Pair<WT>::f32(wp[r]);
-#pragma unroll
-      for (int s = 0; s < SL; ++s) st.a[r][s] = fma2(w, st.sg[s], st.a[r][s]);
-    }
-  }
-
-  // the pairs body<ND, MIX> reads, from the staged rows of its step
-  template <int ND, bool MIX>
-  static __device__ __forceinline__ void load(PR (&wp)[U2], PR& wq, const WT* wrow, const WT* vrow, int lq) {
-#pragma unroll
-    for (int r = 0; r < U2; ++r) wp[r] = Pair<WT>::ld(r < ND ? vrow : wrow, lq + r * GL);
-    if constexpr (MIX && ND < U2) wq = Pair<WT>::ld(vrow, lq + ND * GL);
-  }
-
-  // every slot treated as mixed (small n or h >> n)
-  static __device__ __forceinline__ void body_general(State& st, const WT* wrow, const WT* vrow, int lq, int i,
-                                                      int n, int h, int g_act) {
-#pragma unroll
-    for (int r = 0; r < U2; ++r) {
-      const int q = lq + r * GL;
-      mixed(st, ld_pair(wrow, q), ld_pair(vrow, q), r, i, deg(2 * q, n, h), deg(2 * q + 1, n, h), g_act);
-    }
-  }
-
-  // Reduce SL values over the 32 lanes: afterwards lane l holds the warp sum
-  // of sample q(l); lanes with (l & (32/SL - 1)) == 0 hold distinct samples.
-  static __device__ __forceinline__ float reduce_scatter(float (&v)[SL], int lane, int& q) {
-    q = 0;
-    int cnt = SL;
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-      if (cnt > 1) {
-        const bool up = (lane & o) != 0;
-        const int half = cnt / 2;
-#pragma unroll
-        for (int e = 0; e < SL / 2; ++e) {
-          if (e < half) {
-            const float keep = up ? v[e + half] : v[e];
-            const float send = up ? v[e] : v[e + half];
-            v[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-          }
-        }
-        q = 2 * q + (up ? 1 : 0);
-        cnt = half;
-      } else {
-        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-      }
-    }
-    return v[0];
-  }
-
-  // ring stages (each: SPS rows of W1^T and SPS rows of W2) that fit the
-  // shared-memory budget, at most 8
-  static int stages_for(int hp) {
-    const size_t stage = (size_t)2 * SPS * hp * sizeof(WT);
-    const size_t fixed = (size_t)RL * sizeof(WT) + 2 * 8 * 8 + (size_t)2 * NGRP * GW * SL * sizeof(float) + 256;
-    int nst = (int)((200 * 1024 - fixed) / stage);
-    return nst > 8 ? 8 : nst;
-  }
-  static size_t smem_bytes(int hp, int nst) {
-    return (size_t)nst * 2 * SPS * hp * sizeof(WT) + (size_t)RL * sizeof(WT) + 2 * 8 * 8 +
-           (size_t)2 * NGRP * GW * SL * sizeof(float) + 64;
-  }
-};
-
-// The per-warp step loop.  Slot roles (how many slots are complete, whether
-// one is mixed) change only every few hundred steps, so the kernel runs the
-// steps of one phase in a loop specialised for that phase, and re-dispatches
-// between phases.
-template <typename WT, int GW, int NGRP, int U2, int SL>
-struct Run {
-  using K = Sampler<WT, GW, NGRP, U2, SL>;
-  static constexpr int SPS = K::SPS, UWIN = K::UWIN, GL = K::GL, NCW = K::NCW;
-
-  const SamplerArgs& g;
-  typename K::State st;
-  WT* stages;
-  uint64_t* full;
-  int* relcnt;
-  int* fills;
-  float* gred;
-  const WT* gwt;
-  const WT* gv;
-  int stage_elems, hp, n, h, nst, nblocks;
-  uint32_t block_bytes;
-  int L, lane, wg, grp, b0, my_b, ub, ug;
-  bool writer, uvalid, ok;
-  float uw[4], unx[4];  // logits of this window / uniforms of the next (explicit mode)
-  float cw, cnx;        // b2 of this / the next 32 steps, lane l holds step win+l
-  float lp;
-  uint32_t bits;        // drawn spins of the current 32-step window (writer lanes)
-  int cs;               // ring stage holding the current step's rows
-  uint32_t cpar;        // its fill parity
-  int i;                // next step (1-based)
-  int m0, m1;           // degrees of this lane's units in the mixed slot
-  typename K::PR wp[U2], wq;  // this step's weight pairs, loaded one step ahead
-
-  uint32_t it0, it1;    // Philox iteration words
-
-  __device__ __forceinline__ Run(const SamplerArgs& a) : g(a) {
-    const unsigned long long it = a.it_dev ? *a.it_dev : ((unsigned long long)a.it1 << 32 | a.it0);
-    it0 = (uint32_t)it, it1 = (uint32_t)(it >> 32);
-  }
-
-  __device__ __forceinline__ void issue(int q) {
-    const int s = q % nst;
-    const uint32_t bar = smem_u32(&full[s]);
-    WT* dst = stages + (size_t)s * stage_elems;
-    fills[s] += 1;
-    mbar_expect_tx(bar, 2 * block_bytes);
-    bulk_g2s(smem_u32(dst), gwt + (size_t)q * SPS * hp, block_bytes, bar);
-    bulk_g2s(smem_u32(dst + SPS * hp), gv + (size_t)q * SPS * hp, block_bytes, bar);
-  }
-
-  __device__ __forceinline__ const WT* wrow_of(int t) const { return stages + (size_t)cs * stage_elems + (t & (SPS - 1)) * hp; }
-
-  // bounded wait for the current stage's copies
-  __device__ __forceinline__ void wait_stage() {
-    const uint32_t fb = smem_u32(&full[cs]);
-    bool got = !ok;
-    for (long long it = 0; it < kSpinLimit && !got; ++it) got = mbar_try_wait(fb, cpar);
-    if (!got) {
-      atomicOr(g.err, kErrTimeout);
-      ok = false;  // run on without waiting: every warp still reaches every named barrier
-    }
-  }
-
-  __device__ __forceinline__ void load_u(int win, float (&dst)[4]) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int t = win + 4 * ug + e;
-      dst[e] = (uvalid && t < n) ? __ldg(g.u + (size_t)ub * n + t) : 0.5f;
-    }
-  }
-
-  // writes the spins of the window ending at step t (0-based) as int8 +-1
-  __device__ __forceinline__ void flush(int t) {
-    const int w0 = t & ~31, len = t - w0 + 1;
-    int8_t* dst = g.s_out + (size_t)my_b * n + w0;
-    if (len == 32 && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-      uint32_t wd[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        // byte e of word k = +1 if bit 4k+e is set, else -1 (0xFF)
-        const uint32_t spread = (((bits >> (4 * k)) & 0xFu) * 0x00204081u) & 0x01010101u;
-        wd[k] = 0xFFFFFFFFu - 0xFEu * spread;
-      }
-      reinterpret_cast<uint4*>(dst)[0] = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-      reinterpret_cast<uint4*>(dst)[1] = make_uint4(wd[4], wd[5], wd[6], wd[7]);
+  // What a warp streams through its ring: the W1 rows of its rounds of U of
+  // one block, then the W2 rows of its first Z task of the next block (of
+  // every further task by itself).
+  struct Stream {
+    const WT* p;     // this lane's source of the next stage
+    int left, inc;   // stages left of this run, elements from one to the next
+    int half;        // FP32: elements from a stage's first copy to its second
+    int r, rows;     // the lane's first row of the stage, and the rows there are (beyond: zeros)
+    int k, steps;    // U: first unit of the warp's run, steps of the block
+    const WT* u;     // U: first row, at the lane's place in a stage
+    const WT* z;     // Z: the run that follows U
+    int zn;
+    uint32_t slot;   // byte offset of the next stage in the ring
+  };
+  static constexpr int kCol = 16 / (int)sizeof(WT);  // weights per lane and copy
+  static constexpr int kZLanes = 64 / kCol;          // lanes per row of a Z stage
+  static constexpr int kULanes = 128 / kCol;         // and of a U stage
+  static constexpr int kCopies = kStageBytes / 512;  // per lane and stage
+  static __device__ __forceinline__ void next_run(Stream& x, int hp, int lane) {
+    if (x.k < hp) {
+      const bool in = x.k + (lane % kULanes) * kCol < hp;
+      x.p = in ? x.u + x.k : x.u;
+      x.r = in ? lane / kULanes : kSteps, x.rows = x.steps;
+      x.left = (x.steps + 1) / 2, x.inc = 2 * hp, x.half = hp;
+      x.k += 128 * kWarps;
     } else {
-      for (int e = 0; e < len; ++e) dst[e] = ((bits >> e) & 1u) ? (int8_t)1 : (int8_t)-1;
+      x.p = x.z, x.left = x.zn, x.inc = RL, x.half = 2 * hp;
+      x.r = 0, x.rows = 1 << 30;
+      x.zn = 0;
     }
   }
-
-  // One step.  The weights of step i were loaded during step i-1; this step
-  // loads those of step i+1 right after its own FMAs, so the shared-memory
-  // latency hides behind the reduction and the draw.
-  template <int ND, bool MIX, bool GEN>
-  __device__ __forceinline__ void step() {
-    const int t = i - 1;
-    if ((t & (UWIN - 1)) == 0) {
-      if (g.u) {
+  static __device__ __forceinline__ void issue(Stream& x, uint32_t ring, int hp, int lane) {
+    if (x.left == 0) next_run(x, hp, lane);
+    if (x.left > 0) {
+      const uint32_t dst = ring + x.slot + 16 * lane;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) uw[e] = logit(unx[e]);
-        if (t + UWIN < n) load_u(t + UWIN, unx);
-      } else {
-        const uint4 r = philox4x32_10(make_uint4((uint32_t)((t + 4 * ug) >> 2), (uint32_t)ub + g.boff, it0, it1), g.key0,
-                                      g.key1);
-        uw[0] = logit(to_unit(r.x)), uw[1] = logit(to_unit(r.y));
-        uw[2] = logit(to_unit(r.z)), uw[3] = logit(to_unit(r.w));
+      for (int j = 0; j < kCopies; ++j) {
+        const bool in = x.r + j < x.rows;  // (a second copy: the next row of U; of Z all rows are there)
+        cp16(dst + 512 * j, in ? x.p + j * x.half : x.p, in);
       }
+      x.p += x.inc, x.r += 2, --x.left;
     }
-    if ((t & 31) == 0 && t > 0) {
-      cw = cnx;
-      cnx = (t + 32 + lane < n) ? __ldg(g.b2 + t + 32 + lane) : 0.0f;
-    }
-    const int ro = t & (SPS - 1);
+    cp_commit();
+    x.slot = (x.slot + kStageBytes) & (kRingBytes - 1);
+  }
+  static __device__ __forceinline__ int rounds(int vw, int pairs) {  // in which some lane's pair is complete
+    return pairs > vw * 32 ? (pairs - vw * 32 + GL - 1) / GL : 0;
+  }
+  // the run of Z task (vw, 4 steps from e); sampler_rows() leaves room past the last step
+  static __device__ __forceinline__ void add_z(Stream& x, const WT* v, int hp, int e, int vw, int lane, int pairs) {
+    x.z = v + (unsigned)((e + lane / kZLanes) * hp + 64 * vw + (lane % kZLanes) * kCol);
+    x.zn = rounds(vw, pairs);
+  }
+  static __device__ __forceinline__ void start(Stream& x, uint32_t ring, int hp, int lane) {
+    x.slot = 0, x.left = 0;
+#pragma unroll 1
+    for (int d = 0; d < kDepth; ++d) issue(x, ring, hp, lane);
+  }
+
+  // Z task: virtual warp vw, 4 steps from block step t0.  Lane (i, g), i < 16,
+  // sums the chains of pair classes i and i + 16 over the complete units (pairs
+  // below `pairs`) for samples 4g .. 4g + 3: the tree's first level joins the
+  // two on the lane itself.  32 accumulator pairs per lane, each weight pair
+  // serving 4 FMAs and each state pair 4.
+  static __device__ __forceinline__ void z_task(Stream& x, const unsigned char* ring, uint32_t ring_s, int hp,
+                                                const float* A, const float* zero, int t0, int vw, int lane, int pairs,
+                                                bool leaves, int octet, LeafSum* Z, float* T) {
+    uint64_t acc[2][kTI][4];
 #pragma unroll
-    for (int q = 0; q < SL; ++q) st.acc[q] = pack2(0.0f, 0.0f);
-    if constexpr (GEN) {
-      const WT* wrow = wrow_of(t);
-      K::body_general(st, wrow, wrow + SPS * hp, L, i, n, h, g.act);
-    } else {
-      K::template body<ND, MIX>(st, wp, wq, i, m0, m1, g.act);
-    }
-    if (ro == SPS - 1 || i == n) {
-      // done with the stage; the last warp to release it refills it
+    for (int i = 0; i < 2 * kTI * 4; ++i) acc[i / 16][i / 4 % 4][i % 4] = 0ull;
+    const int nr = rounds(vw, pairs), i16 = lane & 15, sg = lane >> 4;
+    int q = vw * 32 + i16;
+    const float* a = A + vw * kStateChunk + 4 * sg * kChunk + 2 * i16;
+#pragma unroll 1
+    for (int r = 0; r < nr; ++r) {
+      uint64_t xs[2][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint64_t* xp = reinterpret_cast<const uint64_t*>(q + 16 * h < pairs ? a + 32 * h : zero);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) xs[h][s] = xp[s * kChunk / 2];
+      }
+      cp_wait<kDepth - 1>();
       __syncwarp();
-      if (lane == 0) {
-        __threadfence_block();
-        if (atomicAdd(&relcnt[cs], 1) == NCW - 1) {
-          __threadfence_block();
-          relcnt[cs] = 0;
-          const int q = t / SPS + nst;
-          if (q < nblocks) issue(q);
+      const typename Raw<WT>::two* w = reinterpret_cast<const typename Raw<WT>::two*>(ring + x.slot) + i16;
+#pragma unroll
+      for (int t = 0; t < kTI; ++t)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint64_t wf = Raw<WT>::f32(w[32 * t + 16 * h]);
+#pragma unroll
+          for (int s = 0; s < 4; ++s) acc[h][t][s] = fma2(wf, xs[h][s], acc[h][t][s]);
+        }
+      __syncwarp();
+      issue(x, ring_s, hp, lane);
+      q += GL;
+      a += GW * kStateChunk;
+    }
+    if (leaves) {
+      // the group's own octet keeps its pairs, each with the sums that join
+      // it on the tree's first two levels
+      const bool own = (i16 >> 3) == (octet & 1), upper = octet >= 2;
+      const uint32_t rec =
+          (uint32_t)__cvta_generic_to_shared(Z + (t0 * kSamples + 4 * sg) * kLeaves + (lane & 7));
+#pragma unroll
+      for (int t = 0; t < kTI; ++t)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const float v0 = sum2(acc[0][t][s]), v1 = sum2(acc[1][t][s]);
+          const float d = __shfl_xor_sync(0xffffffffu, v0 + v1, 8);
+          st16_if(rec + (t * kSamples + s) * kLeaves * 16, upper ? acc[1][t][s] : acc[0][t][s], pack2(upper ? v0 : v1, d),
+                  own);
+        }
+    } else {
+      // the rest of the tree: 16 values over 16 lanes, halving the values
+      // held at every level; lane i ends with value i
+      float v[kTI * 4];
+#pragma unroll
+      for (int i = 0; i < kTI * 4; ++i) v[i] = sum2(acc[0][i / 4][i % 4]) + sum2(acc[1][i / 4][i % 4]);
+#pragma unroll
+      for (int o = 8; o >= 1; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+          const float keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
       }
+      T[(vw * kSteps + t0 + (i16 >> 2)) * kSamples + 4 * sg + (i16 & 3)] = v[0];
     }
-    if (i < n) {
-      if (ro == SPS - 1) {
-        if (++cs == nst) cs = 0, cpar ^= 1u;
-        wait_stage();
-      }
-      if constexpr (!GEN) {
-        // next step's pairs, with this phase's roles (a new phase reloads)
-        const WT* wrow = wrow_of(t + 1);
-        K::template load<ND, MIX>(wp, wq, wrow, wrow + SPS * hp, L);
-      }
-    }
-    // z_i: lanes -> warp (shuffles) -> group (shared memory + named barrier)
-    float v[SL];
-#pragma unroll
-    for (int q = 0; q < SL; ++q) {
-      float lo, hi;
-      unpack2(st.acc[q], lo, hi);
-      v[q] = lo + hi;
-    }
-    int qs;
-    const float ws = K::reduce_scatter(v, lane, qs);
-    float* rb = gred + (size_t)(t & 1) * NGRP * GW * SL;
-    if ((lane & (32 / SL - 1)) == 0) rb[wg * SL + qs] = ws;
-    const int e = t & 3;
-    const float lsel = e == 0 ? uw[0] : e == 1 ? uw[1] : e == 2 ? uw[2] : uw[3];
-    const float lg = __shfl_sync(0xffffffffu, lsel, ((t & (UWIN - 1)) >> 2) * SL + (lane & (SL - 1)));
-    float z = __shfl_sync(0xffffffffu, cw, t & 31);
-    if constexpr (GW > 1) asm volatile("barrier.sync %0, %1;" ::"r"(1 + grp), "r"(GW * 32) : "memory");
-    else __syncwarp();
-    // lanes >= SL compute a copy of lane (lane % SL)'s value; only bits < SL are used
-#pragma unroll
-    for (int w = 0; w < GW; ++w) z += rb[w * SL + (lane & (SL - 1))];
-    const bool up = z > lg;  // u < sigma(z)
-    const uint32_t mask = __ballot_sync(0xffffffffu, up);
-#pragma unroll
-    for (int q = 0; q < SL; ++q) {
-      const float sv = ((mask >> q) & 1u) ? 1.0f : -1.0f;
-      st.sg[q] = pack2(sv, sv);
-    }
-    bits |= (up ? 1u : 0u) << (t & 31);
-    if (g.logp && writer) lp += log_sigmoid(up ? z : -z);
-    if ((t & 31) == 31 || i == n) {
-      if (writer) flush(t);
-      bits = 0;
-    }
-    ++i;
   }
 
-  template <int ND, bool MIX, bool GEN>
-  __device__ __forceinline__ void steps(int i_end) {
-    if constexpr (!GEN) {
-      const WT* wrow = wrow_of(i - 1);
-      K::template load<ND, MIX>(wp, wq, wrow, wrow + SPS * hp, L);
+  // The draws of one block for 4 samples by one warp, 8 lanes per sample: lane
+  // l of a sample holds leaf l of the group's octet.  The chain from one draw
+  // to the next (the newest unit's pre-activation and act, its leaf's FMA, four
+  // levels of sums, three shuffles, b2, the other virtual warps' trees, the
+  // compare) is about 200 cycles; a spin has two values, so both logits of step
+  // t + 1 are begun before spin t is known, and each iteration finishes the two
+  // logits of step t beside the first half of step t + 1's.  Only the units
+  // that complete with spin t differ between the two.  Stores are made by all
+  // of a sample's lanes alike (a divergent store costs about 70 cycles).
+  // A: the group's units of sample 0 in the state; over: the group's steps end
+  // with this block.
+  static __device__ __forceinline__ void solve(const Tables& tb, Drawn& out, const LeafSum* Z, const float* T, Post* P,
+                                               uint64_t* SP, float* A, int steps, int wg, int sw, int lane, bool over) {
+    const int s = 4 * sw + (lane >> 3), l = lane & 7;
+    // what joins the group's tree to a logit: one (step, sample) per lane and turn
+#pragma unroll 1
+    for (int i = lane; i < 4 * kSteps; i += 32) {
+      const int t = i >> 2, sq = 4 * sw + (i & 3);
+      Post x{};
+      x.zb = tb.b2[t], x.lg = tb.logit[t][sq];
+      if constexpr (GW > 1) {
+#pragma unroll
+        for (int q = 0; q < GW; ++q) {
+          const float y = T[(q * kSteps + t) * kSamples + sq];
+          x.zb = q < wg ? x.zb + y : x.zb;
+          if (q > 0) x.post[q - 1] = q > wg ? y : 0.0f;
+        }
+      }
+      P[t * kSamples + sq] = x;
     }
-    while (i < i_end) step<ND, MIX, GEN>();
-  }
-
-  // code = 2*nd + mixed, nd in [0, U2]
-  template <int LO, int HI>
-  __device__ __forceinline__ void dispatch(int code, int i_end) {
-    if constexpr (LO == HI) {
-      steps<LO / 2, (LO & 1) != 0, false>(i_end);
-    } else {
-      constexpr int MID = (LO + HI) / 2;
-      if (code <= MID) dispatch<LO, MID>(code, i_end);
-      else dispatch<MID + 1, HI>(code, i_end);
+    __syncwarp();
+    uint64_t* row = reinterpret_cast<uint64_t*>(A + s * kChunk) + l;
+    const LeafSum* zr = Z + s * kLeaves + l;
+    float a0, a1, g0 = 0.0f, g1_ = 0.0f;  // this leaf's units: pre-activations, activations (zero until complete)
+    unpack2(*row, a0, a1);
+    const int first = uniform(tb.done[0]);
+    int u = 0;  // units done so far
+#pragma unroll 1
+    for (; u < first; ++u) {
+      const float f = g1(u & 1 ? a1 : a0);
+      const bool mine = (u >> 1) == l;
+      g0 = mine && !(u & 1) ? f : g0;
+      g1_ = mine && (u & 1) ? f : g1_;
     }
+    auto leaf_sum = [&](const ulonglong2& r, uint64_t v, float x0, float x1) {
+      float c, d;
+      unpack2(r.y, c, d);
+      return (sum2(fma2(v, pack2(x0, x1), r.x)) + c) + d;
+    };
+    ulonglong2 vw = *reinterpret_cast<const ulonglong2*>(&tb.leaf[0][l]);
+    // the candidates after spin t - 1 = -1 (m) and +1 (p)
+    float ym = leaf_sum(*reinterpret_cast<const ulonglong2*>(zr), vw.x, g0, g1_), yp = ym;
+    float m0 = g0, m1 = g1_, p0 = g0, p1 = g1_;
+    uint64_t w = 0ull;  // W1 of spin t - 1
+    bool up = true;
+    uint32_t bits = 0;
+#pragma unroll 1
+    for (int t = 0; t < steps; ++t) {
+      const int tn = min(t + 1, steps - 1);
+      const ulonglong2 rn = *reinterpret_cast<const ulonglong2*>(zr + tn * kSamples * kLeaves);
+      const ulonglong2 vwn = *reinterpret_cast<const ulonglong2*>(&tb.leaf[tn][l]);
+      const float4 pz = *reinterpret_cast<const float4*>(P + t * kSamples + s);
+      const int dn = t + 1 < steps ? uniform(tb.done[tn]) : u;
+      // spin t - 1 is known: its pre-activations and activations
+      const float sv = up ? 1.0f : -1.0f;
+      unpack2(fma2(w, pack2(sv, sv), pack2(a0, a1)), a0, a1);
+      w = vw.y;
+      g0 = up ? p0 : m0, g1_ = up ? p1 : m1;
+      m0 = p0 = g0, m1 = p1 = g1_;
+      // the units that complete with spin t, for both of its values: all but
+      // the last (there is rarely more than one) in a loop, so that the rest
+      // of the iteration is straight code
+      float w0, w1;
+      unpack2(w, w0, w1);
+      auto complete = [&](bool any) {
+        const float xa = u & 1 ? a1 : a0, xw = u & 1 ? w1 : w0;
+        const float fm = g1(xa - xw), fp = g1(xa + xw);
+        const bool mine = any && (u >> 1) == l;
+        const bool lo = mine && !(u & 1), hi = mine && (u & 1);
+        m0 = lo ? fm : m0, p0 = lo ? fp : p0;
+        m1 = hi ? fm : m1, p1 = hi ? fp : p1;
+      };
+#pragma unroll 1
+      for (; u + 1 < dn; ++u) complete(true);
+      if constexpr (RELU) {
+        complete(u < dn);
+      } else {
+        if (u < dn) complete(true);
+      }
+      u = dn;
+      // the two logits of step t
+      float zm = ym + __shfl_xor_sync(0xffffffffu, ym, 4), zp = yp + __shfl_xor_sync(0xffffffffu, yp, 4);
+      zm += __shfl_xor_sync(0xffffffffu, zm, 2), zp += __shfl_xor_sync(0xffffffffu, zp, 2);
+      zm += __shfl_xor_sync(0xffffffffu, zm, 1), zp += __shfl_xor_sync(0xffffffffu, zp, 1);
+      zm = pz.x + zm, zp = pz.x + zp;
+      if constexpr (GW > 1) zm += pz.z, zp += pz.z;
+      if constexpr (GW == 4) {
+        const float q = P[t * kSamples + s].post[2];
+        zm = (zm + pz.w) + q, zp = (zp + pz.w) + q;
+      }
+      ym = leaf_sum(rn, vwn.x, m0, m1);
+      yp = leaf_sum(rn, vwn.x, p0, p1);
+      vw = vwn;
+      const float z = up ? zp : zm;
+      up = z > pz.y;  // u < sigma(z)
+      const float sn = up ? 1.0f : -1.0f;
+      SP[t * kSamples + s] = pack2(sn, sn);
+      out.x[t * kSamples + s] = up ? z : -z;
+      bits |= (up ? 1u : 0u) << t;
+    }
+    out.bits[s] = bits;
+    // the group's state back: g1 if its steps are over
+    const float sv = up ? 1.0f : -1.0f;
+    const uint64_t a = fma2(w, pack2(sv, sv), pack2(a0, a1));
+    *row = over ? g1_pair(a) : a;
   }
 };
 
-template <typename WT, int GW, int NGRP, int U2, int SL>
-__global__ void __launch_bounds__(GW * NGRP * 32, 1) sampler_kernel(const SamplerArgs g) {
-  using K = Sampler<WT, GW, NGRP, U2, SL>;
-  constexpr int RL = K::RL, SPS = K::SPS, GL = K::GL;
-  extern __shared__ __align__(128) unsigned char smem[];
-  const int nst = g.nst, hp = g.hp;
-  const int stage_elems = 2 * SPS * hp;  // W1^T rows then W2 rows
-  // ring, then RL elements of slack: lanes holding padding units (k >= hp)
-  // read past their row, never past the ring
-  const int ring_elems = nst * stage_elems + RL;
-  WT* stages = reinterpret_cast<WT*>(smem);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + ((size_t)ring_elems * sizeof(WT) + 7) / 8 * 8);
-  int* relcnt = reinterpret_cast<int*>(full + 8);     // [8] warps that released each stage
-  int* fills = relcnt + 8;                            // [8] copies issued into each stage
-  int* failed = fills + 8;                            // some warp gave up a wait
-  float* red = reinterpret_cast<float*>(fills + 12);  // [2][NGRP][GW][SL]
-
-  const int n = g.n, h = g.h;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-  // zero the ring once: every value a lane may read must be finite
-  for (int q = tid; q < ring_elems; q += K::NT) stages[q] = from_f<WT>(0.0f);
-  if (tid == 0) {
-    for (int s = 0; s < nst; ++s) {
-      mbar_init(smem_u32(&full[s]), 1);
-      relcnt[s] = 0;
-      fills[s] = 0;
-    }
-    *failed = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+// Fills the tables of block b; i: 0 .. 63
+template <typename WT>
+__device__ __forceinline__ void stage_tables(Tables* tb, const SamplerArgs& g, const Block& b, int b0, uint32_t it0,
+                                             uint32_t it1, int i) {
+  using R = Raw<WT>;
+  const int steps = b.e1 - b.e0, k0 = kGroup * b.grp;
+  const WT* wt = reinterpret_cast<const WT*>(g.wt);
+  const WT* v = reinterpret_cast<const WT*>(g.v);
+  const int t = i >> 2, c = i & 3;  // units 4c .. 4c + 3 of the group at step t
+  typename R::four wv{}, ww{};
+  if (t < steps && k0 + kGroup <= g.hp) {
+    wv = __ldg(reinterpret_cast<const typename R::four*>(v + (size_t)(b.e0 + t) * g.hp + k0 + 4 * c));
+    ww = __ldg(reinterpret_cast<const typename R::four*>(wt + (size_t)(b.e0 + 1 + t) * g.hp + k0 + 4 * c));
   }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncthreads();
-
-  Run<WT, GW, NGRP, U2, SL> R(g);
-  R.stages = stages, R.full = full, R.relcnt = relcnt, R.fills = fills;
-  R.gwt = reinterpret_cast<const WT*>(g.wt);
-  R.gv = reinterpret_cast<const WT*>(g.v);
-  R.stage_elems = stage_elems, R.hp = hp, R.n = n, R.h = h, R.nst = nst;
-  R.nblocks = (n + SPS - 1) / SPS;
-  R.block_bytes = (uint32_t)(SPS * hp * sizeof(WT));
-  // Stage q % nst holds block q: rows q*SPS.. of wt_s (row j = input j, row 0
-  // zero) and of v_s (row i = output i+1), copied whole.  The warp that
-  // releases a stage last issues the copies of the block a full ring ahead.
-  if (tid == 0)
-    for (int q = 0; q < nst && q < R.nblocks; ++q) R.issue(q);
-
-  const int grp = warp / GW, wg = warp % GW;
-  R.grp = grp, R.wg = wg, R.lane = lane;
-  R.L = wg * 32 + lane;
-  R.b0 = blockIdx.x * K::S + grp * SL;
-  R.gred = red + (size_t)grp * GW * SL;
-#pragma unroll
-  for (int r = 0; r < U2; ++r) {
-    const int k = 2 * (r * GL + R.L);
-    const float x0 = k < h ? __ldg(g.b1 + k) : 0.0f;
-    const float x1 = k + 1 < h ? __ldg(g.b1 + k + 1) : 0.0f;
-#pragma unroll
-    for (int s = 0; s < SL; ++s) R.st.a[r][s] = pack2(x0, x1);
-  }
-#pragma unroll
-  for (int s = 0; s < SL; ++s) R.st.sg[s] = pack2(0.0f, 0.0f);
-  // uniforms: lane l (< 32) holds 4 words for sample l % SL, steps
-  // win + 4*(l / SL) .. +3 of the current window
-  R.ug = lane / SL;
-  R.ub = R.b0 + lane % SL;
-  R.uvalid = R.ub < g.B;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) R.uw[e] = 0.0f, R.unx[e] = 0.5f;
-  if (g.u) R.load_u(0, R.unx);
-  R.cw = lane < n ? __ldg(g.b2 + lane) : 0.0f;
-  R.cnx = 32 + lane < n ? __ldg(g.b2 + 32 + lane) : 0.0f;
-  R.my_b = R.b0 + lane;
-  R.writer = wg == 0 && lane < SL && R.my_b < g.B;
-  R.ok = true;
-  R.lp = 0.0f;
-  R.bits = 0;
-  R.cs = 0, R.cpar = 0;
-  R.i = 1;
-  R.wait_stage();
-
-  // warp-uniform slot bookkeeping: nd = #slots complete before step i, nt =
-  // #slots with at least one unit complete at step i; thresholds are the
-  // degrees of the next slot's last / first unit
-  const int kw = 2 * wg * 32;  // first unit of the warp in slot 0
-  int nd = 0, nt = 0;
-  int thr_nd = K::deg(kw + 63, n, h), thr_nt = K::deg(kw, n, h);
-  while (R.i <= n) {
-    const int i = R.i;
-    while (nd < U2 && thr_nd <= i - 2) {
-      ++nd;
-      thr_nd = nd < U2 ? K::deg(kw + nd * 2 * GL + 63, n, h) : kBig;
+  const int e = b.e0 + t, done = complete_before(e, g.n, g.h) - k0 - 4 * c;
+  tb->leaf[t][2 * c] = Leaf{R::lo(wv), R::lo(ww)}, tb->leaf[t][2 * c + 1] = Leaf{R::hi(wv), R::hi(ww)};
+  if (c == 0) tb->b2[t] = e < b.e1 ? __ldg(g.b2 + e) : 0.0f, tb->done[t] = done;
+  // the uniforms: 4 steps of one sample per thread (a block touches at most 5 groups of 4 steps)
+  const int s = i & 7, c4 = 4 * ((b.e0 >> 2) + (i >> 3));
+  if (c4 < b.e1) {
+    uint32_t xw[4] = {0, 0, 0, 0};
+    if (!g.u) {
+      const uint4 r = philox4x32_10(make_uint4((uint32_t)c4 >> 2, (uint32_t)(b0 + s) + g.boff, it0, it1), g.key0, g.key1);
+      xw[0] = r.x, xw[1] = r.y, xw[2] = r.z, xw[3] = r.w;
     }
-    while (nt < U2 && thr_nt <= i - 1) {
-      ++nt;
-      thr_nt = nt < U2 ? K::deg(kw + nt * 2 * GL, n, h) : kBig;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      const int e4 = c4 + j;
+      const uint32_t w = j & 2 ? (j & 1 ? xw[3] : xw[2]) : (j & 1 ? xw[1] : xw[0]);
+      if (e4 < b.e0 || e4 >= b.e1) continue;
+      const float u = !g.u ? to_unit(w) : b0 + s < g.B ? __ldg(g.u + (size_t)(b0 + s) * g.n + e4) : 0.5f;
+      tb->logit[e4 - b.e0][s] = logit(u);
     }
-    // the phase lasts until nd or nt next changes
-    long long end = (long long)n + 1;
-    if (thr_nd < kBig && thr_nd + 2 < end) end = thr_nd + 2;
-    if (thr_nt < kBig && thr_nt + 1 < end) end = thr_nt + 1;
-    const int i_end = (int)end;
-    R.m0 = nd < U2 ? K::deg(2 * (R.L + nd * GL), n, h) : kBig;
-    R.m1 = nd < U2 ? K::deg(2 * (R.L + nd * GL) + 1, n, h) : kBig;
-    if (nt <= nd + 1) R.template dispatch<0, 2 * U2>(2 * nd + (nt - nd), i_end);
-    else R.template steps<0, false, true>(i_end);
   }
-
-  // Every warp runs all n steps, so this barrier is reached by all.  After a
-  // failed wait, copies may still be in flight: drain them before exiting.
-  if (!R.ok) *failed = 1;
-  __syncthreads();
-  if (tid == 0 && *failed)
-    for (int s = 0; s < nst; ++s)
-      if (fills[s] > 0 && !mbar_wait(smem_u32(&full[s]), (uint32_t)((fills[s] - 1) & 1), g.err)) break;
-  if (R.ok && R.writer && g.logp) g.logp[R.my_b] = R.lp;
 }
 
-template <typename WT, int GW, int NGRP, int U2, int SL>
+// The outputs of block b by one warp; lanes 0 .. 7 keep log pi of the samples.
+__device__ __forceinline__ void write_block(const SamplerArgs& g, const Block& b, Drawn* d, int b0, int lane,
+                                            float& lp) {
+  const int steps = b.e1 - b.e0, s = lane >> 2;
+  const uint32_t bits = d->bits[s];
+  if (b0 + s < g.B) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int t = 4 * (lane & 3) + j;
+      if (t < steps) g.s_out[(size_t)(b0 + s) * g.n + b.e0 + t] = (bits >> t) & 1u ? (int8_t)1 : (int8_t)-1;
+    }
+  }
+  if (g.logp) {
+#pragma unroll 1
+    for (int q = lane; q < steps * kSamples; q += 32) d->x[q] = log_sigmoid(d->x[q]);
+    __syncwarp();
+    if (lane < kSamples)
+#pragma unroll 1
+      for (int t = 0; t < steps; ++t) lp += d->x[t * kSamples + lane];
+  }
+}
+
+// The steady state of the kernel has to fit the instruction cache (the phases
+// alternate every few thousand cycles, and a miss costs several hundred): the
+// activation is a template parameter, and loops are unrolled no further than
+// their operands' latency asks for.
+template <typename WT, int GW, bool RELU>
+__global__ void __launch_bounds__(kThreads, 2) sampler_kernel(const SamplerArgs g) {
+  using K = BlockSampler<WT, GW, RELU>;
+  using R = Raw<WT>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  LeafSum* Z = reinterpret_cast<LeafSum*>(smem + K::kOffZ);
+  unsigned char* ring = smem + K::kOffR + uniform(threadIdx.x >> 5) * K::kRingBytes;
+  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+  float* T = reinterpret_cast<float*>(smem + K::kOffT);
+  uint64_t* SP = reinterpret_cast<uint64_t*>(smem + K::kOffS);
+  typename K::Post* P = reinterpret_cast<typename K::Post*>(smem + K::kOffP);
+  Tables* tables = reinterpret_cast<Tables*>(smem + K::kOffTab);
+  Drawn* drawn = reinterpret_cast<Drawn*>(smem + K::kOffDrawn);
+  Block* next = reinterpret_cast<Block*>(smem + K::kOffNext);
+  float* zero = reinterpret_cast<float*>(smem + K::kOffZero);
+  float* A = reinterpret_cast<float*>(smem + K::kOffA);
+
+  const int n = g.n, h = g.h, hp = g.hp;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
+  const int b0 = blockIdx.x * kSamples;
+  const WT* wt = reinterpret_cast<const WT*>(g.wt);
+  const WT* v = reinterpret_cast<const WT*>(g.v);
+  const unsigned long long it = g.it_dev ? *g.it_dev : ((unsigned long long)g.it1 << 32 | g.it0);
+  const uint32_t it0 = (uint32_t)it, it1 = (uint32_t)(it >> 32);
+
+#pragma unroll 1
+  for (int k = tid; k < hp + kChunk; k += kThreads) {
+    const float x = k < h ? __ldg(g.b1 + k) : 0.0f;
+#pragma unroll
+    for (int s = 0; s < kSamples; ++s) A[(k / kChunk) * K::kStateChunk + s * kChunk + k % kChunk] = x;
+  }
+#pragma unroll 1
+  for (int k = tid; k < K::kStateChunk; k += kThreads) zero[k] = 0.0f;
+  for (int k = tid; k < kSteps * kSamples; k += kThreads) SP[k] = 0ull;
+  __syncthreads();
+
+  // The blocks go through a pipeline, so that each part stands once in the
+  // code: turn i finds block i + 2, stages the tables of block i + 1, takes
+  // block i through Z, the draws and U, and writes the outputs of block i - 1.
+  Block b{0, 0, 0, 0}, nb{0, 0, 0, 0}, prev{0, 0, 0, 0};  // e0 == e1: none
+  float lp = 0.0f;
+  typename K::Stream st{};
+  st.k = hp;  // no U before the first block
+#pragma unroll 1
+  for (int turn = -2;; ++turn) {
+    const int par = turn & 1, steps = b.e1 - b.e0;
+    if (steps > 0) {
+      // ----------------------------------------------------------- Z
+      const int gs = b.grp % (4 * GW), pairs = kLeaves * b.grp;
+#pragma unroll 1
+      for (int task = warp; task < 4 * GW; task += kWarps) {
+        const int vw = task >> 2, t0 = kTI * (task & 3);
+        if (t0 >= steps) continue;
+        if (GW > 2 && task != warp) {
+          __syncwarp();
+          K::add_z(st, v, hp, b.e0 + t0, vw, lane, pairs);
+          K::start(st, ring_s, hp, lane);
+        }
+        K::z_task(st, ring, ring_s, hp, A, zero, t0, vw, lane, pairs, vw == gs >> 2, gs & 3, Z, T);
+      }
+    }
+    __syncthreads();  // Z and T complete
+    const bool more = nb.e1 > nb.e0;
+    if (steps > 0 && more) {
+      // U of this block, then the next block's Z
+      st.u = wt + (unsigned)((b.e0 + 1 + lane / K::kULanes) * hp + min((lane % K::kULanes) * K::kCol, hp - K::kCol));
+      st.k = kGroup * (b.grp + 1) + 128 * warp, st.steps = steps;
+      K::add_z(st, v, hp, nb.e0 + kTI * (warp & 3), warp >> 2, lane,
+               warp < 4 * GW && kTI * (warp & 3) < nb.e1 - nb.e0 ? kLeaves * nb.grp : 0);
+      K::start(st, ring_s, hp, lane);
+    }
+    if (warp >= kWarps - kSolvers) {
+      if (steps > 0) {
+        const int k0 = kGroup * b.grp, gs = b.grp % (4 * GW);
+        K::solve(tables[par], drawn[par], Z, T, P, SP, A + k0 / kChunk * K::kStateChunk + k0 % kChunk, steps, gs >> 2,
+                 warp - (kWarps - kSolvers), lane, nb.grp != b.grp);
+      }
+    } else if (warp == 2) {
+      if (lane == 0) {
+        Block x{0, 0, 0, 0};
+        const int e = turn == -2 ? 0 : nb.e1;
+        if (e < n && (turn == -2 || more)) x = next_block(e, n, h);
+        next[par] = x;
+      }
+      if (prev.e1 > prev.e0) write_block(g, prev, drawn + (par ^ 1), b0, lane, lp);
+    } else if (more && warp < 2) {
+      stage_tables<WT>(tables + (par ^ 1), g, nb, b0, it0, it1, tid);
+    }
+    __syncthreads();  // the block's spins are drawn
+    prev = b;
+    b = nb;
+    nb = next[par];
+    nb = Block{uniform(nb.e0), uniform(nb.e1), uniform(nb.grp), 0};
+    if (steps == 0 || !more) {
+      if (turn >= 0 && steps == 0) break;  // the last block's outputs are written
+      continue;
+    }
+    // ------------------------------------------------------------- U
+    // 128 units per warp and round, four consecutive ones per lane
+#pragma unroll 1
+    for (int k = kGroup * (prev.grp + 1) + 128 * warp; k < hp; k += 128 * kWarps) {
+      const int kl = k + 4 * lane;
+      const bool in = kl < hp;
+      float* a = A + kl / kChunk * K::kStateChunk + kl % kChunk;
+      uint64_t a0[kSamples], a1[kSamples];
+#pragma unroll
+      for (int s = 0; s < kSamples; ++s) {
+        ulonglong2 x = make_ulonglong2(0ull, 0ull);
+        if (in) x = *reinterpret_cast<const ulonglong2*>(a + s * kChunk);
+        a0[s] = x.x, a1[s] = x.y;
+      }
+#pragma unroll 1
+      for (int t = 0; t < steps; t += 2) {
+        cp_wait<K::kDepth - 1>();
+        __syncwarp();
+        const typename R::four* w = reinterpret_cast<const typename R::four*>(ring + st.slot) + lane;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {  // past the last step the weights are zero
+          const uint64_t u0 = R::lo(w[32 * j]), u1 = R::hi(w[32 * j]);
+          const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(SP + (t + j) * kSamples);
+#pragma unroll
+          for (int s = 0; s < kSamples; s += 2) {
+            const ulonglong2 x = sp[s / 2];
+            a0[s] = fma2(u0, x.x, a0[s]);
+            a1[s] = fma2(u1, x.x, a1[s]);
+            a0[s + 1] = fma2(u0, x.y, a0[s + 1]);
+            a1[s + 1] = fma2(u1, x.y, a1[s + 1]);
+          }
+        }
+        __syncwarp();
+        K::issue(st, ring_s, hp, lane);
+      }
+      if (in)
+#pragma unroll
+        for (int s = 0; s < kSamples; ++s)
+          *reinterpret_cast<ulonglong2*>(a + s * kChunk) = make_ulonglong2(a0[s], a1[s]);
+      if (kl < kGroup * b.grp && in)  // units of a group that has no steps of its own are complete now
+#pragma unroll 1
+        for (int i = 0; i < 2 * kSamples; ++i) {
+          uint64_t* x = reinterpret_cast<uint64_t*>(a + (i >> 1) * kChunk) + (i & 1);
+          *x = K::g1_pair(*x);
+        }
+    }
+    // the next Z reads the units below group b.grp: group prev.grp (written
+    // by the solver) and, if there are any, the groups completed just now
+    if (b.grp > prev.grp + 1) __syncthreads();
+  }
+  if (warp == 2 && lane < kSamples && g.logp && b0 + lane < g.B) g.logp[b0 + lane] = lp;
+}
+
+template <typename WT, int GW>
 cudaError_t launch_cfg(const SamplerArgs& a, cudaStream_t st) {
-  using K = Sampler<WT, GW, NGRP, U2, SL>;
-  SamplerArgs b = a;
-  b.nst = K::stages_for(a.hp);
-  if (b.nst < 2) return cudaErrorNotSupported;
-  const size_t smem = K::smem_bytes(a.hp, b.nst);
-  auto kern = sampler_kernel<WT, GW, NGRP, U2, SL>;
+  const bool relu = a.act == VQMC_ACT_RELU;
+  auto kern = relu ? sampler_kernel<WT, GW, true> : sampler_kernel<WT, GW, false>;
+  const size_t smem = BlockSampler<WT, GW, true>::smem_bytes(a.hp);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int grid = (a.B + K::S - 1) / K::S;
-  kern<<<grid, K::NT, smem, st>>>(b);
+  kern<<<(a.B + kSamples - 1) / kSamples, kThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-// Shapes: a group covers GW*32 lanes x 2*U2 units >= hp; 16 samples per CTA
-// up to hp = 2048.  Beyond, four warps per group and 2 samples per group (4
-// per CTA) keep the pre-activations in about 140 registers per thread; the
-// ring then holds two stages of SPS rows when they fit the shared memory
-// (BF16 up to hp = 5120, FP32 up to hp = 2816).
+// The summation order (GW) by hp; `wide` asks for the order of hp > 2048 at any hp.
 template <typename WT>
 cudaError_t launch_sampler_wt(const SamplerArgs& a, cudaStream_t st) {
-  if (a.wide && a.hp <= 5120) return launch_cfg<WT, 4, 2, 20, 2>(a, st);
-  if (a.hp <= 64) return launch_cfg<WT, 1, 2, 1, 8>(a, st);
-  if (a.hp <= 1024) return launch_cfg<WT, 2, 2, 8, 8>(a, st);
-  if (a.hp <= 2048) return launch_cfg<WT, 2, 4, 16, 4>(a, st);
-  if (a.hp <= 5120) return launch_cfg<WT, 4, 2, 20, 2>(a, st);
-  return cudaErrorNotSupported;
+  if (!sampler_wt_supports<WT>(a.hp, a.wide)) return cudaErrorNotSupported;
+  if (a.wide || a.hp > 2048) return launch_cfg<WT, 4>(a, st);
+  if (a.hp <= 64) return launch_cfg<WT, 1>(a, st);
+  return launch_cfg<WT, 2>(a, st);
 }
 
 // Whether launch_sampler_wt<WT> runs models with hp padded hidden units.
 template <typename WT>
 bool sampler_wt_supports(int hp, bool wide) {
-  if (hp <= 2048 && !wide) return true;
-  if (hp <= 5120) return Sampler<WT, 4, 2, 20, 2>::stages_for(hp) >= 2;
-  return false;
+  (void)wide;
+  return hp <= (sizeof(WT) == 2 ? 5120 : 2816);
 }
 
 }  // namespace vqmc

@@ -1148,8 +1148,7 @@ vqmc_status vqmc_batch_autotune(vqmc_batch* b, const int32_t* B, vqmc_stream str
   const size_t m = b->members.size();
   // 1. cost of one iteration of each member alone (after one warm-up step),
   // and for a member on the CUDA-core sampler up to 2048 hidden units the
-  // faster of its two layouts (16 samples per CTA, or the wide one: groups of
-  // four warps, 4 samples per CTA)
+  // faster of its two summation orders
   std::vector<double> cost(m, 0.0);
   {
     cudaEvent_t e0 = nullptr, e1 = nullptr;

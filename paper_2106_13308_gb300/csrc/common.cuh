@@ -168,11 +168,12 @@ struct vqmc_ctx {
   void* D = nullptr;       // [Bmax][np] output adjoint delta
   void* Dt = nullptr;      // [n][Bp]
   void* GAt = nullptr;     // [h][Bp] hidden pre-activation adjoint, transposed
+  float* GA = nullptr;     // FP32: the same, [Bmax][hp]
   float* logp = nullptr;   // [Bmax]
   float* coef = nullptr;   // [Bmax]
   double* stats = nullptr; // [4]
   float* row_part = nullptr;  // [ceil(max(n,h)/128)][Bmax] partial row sums
-  float* col_part = nullptr;  // [ceil(Bmax/128)][max(np,hp)] partial column sums
+  float* col_part = nullptr;  // [ceil(Bmax/64)][max(np,hp)] partial column sums
   int row_part_ld = 0, col_part_ld = 0, row_part_tiles = 0, col_part_tiles = 0;
   uint32_t* err = nullptr;   // sticky device error word
   // per-part step timing (vqmc_timing_*): events[step][part boundary]

@@ -2,8 +2,9 @@
 // passes (Sec. 2.3; gradient of Sec. 2.1), used by the CUDA-core and the
 // tcgen05 implementations.
 //
-// All GEMMs are C[m][n] = sum_k A[m][k] * Bm[n][k] with both operands stored
-// K-contiguous ("TN").  With sorted MADE degrees the weight matrices are block
+// All GEMMs are C[m][n] = sum_k A[m][k] * B[n][k].  The tcgen05 implementation
+// takes both operands K-contiguous ("TN"); the CUDA-core one takes A
+// K-contiguous and B as Bm[k][n].  With sorted MADE degrees the weight matrices are block
 // staircases, so each N-tile only visits the K-range where its weights can be
 // non-zero, and fully masked output tiles of the weight gradients are written
 // as zeros without a main loop.
@@ -51,6 +52,9 @@ struct GemmArgs {
   float* col_part;     // [M-tile][ldc]
   int ldc;
   uint32_t* err;       // device error word (bounded waits)
+  int sms;             // SMs of the device (FP32: choice of the tile)
+  float* part;         // FP32 weight gradients, optional: scratch for the parts
+  size_t part_cap;     // of a split K, part_cap floats
   // Adam step fused into the weight-gradient epilogue (tensor-core path,
   // kOpDV / kOpDW with theta set; gout unused): theta, adam_m and adam_v
   // point at the weight block, [M][ldg]; the refreshed weights also go to
@@ -93,13 +97,9 @@ __host__ __device__ inline bool gemm_tile_masked(int op, int m0, int m1, int n0,
   return false;
 }
 
-__host__ __device__ inline bool gemm_out_kept(int op, int m, int k, int n, int h) {
-  if (op == kOpDV) return degree(k, n, h) <= m;
-  if (op == kOpDW) return m < degree(k, n, h);
-  return true;
-}
-
 cudaError_t launch_gemm_simt_f32(const GemmArgs<float>& a, cudaStream_t st);
+// rows per tile (and per column partial) of that launch
+int gemm_simt_rows(int op, int M, int N, int sms);
 // tcgen05 path (BF16 operands, FP32 accumulation in tensor memory).
 cudaError_t launch_gemm_tc_bf16(const GemmArgs<bf16>& a, cudaStream_t st);
 bool gemm_tc_available();

@@ -2,280 +2,411 @@
 // the plain FP32 precision (FP32 operands, FP32 accumulation).  The BF16
 // precision runs the same GEMMs on the tcgen05 tensor cores (gemm_tc.cu).
 //
-// Tile 128 x 128 x 16, 256 threads, 8 x 8 outputs per thread (rows
-// m0 + 8*ty + i, columns n0 + 8*tx + j), register-staged double buffering.
+// 256 threads, TM x TN outputs per thread (rows m0 + TM ty + i, columns
+// n0 + 64 q + 4 tx + j, j < 4), K in steps of 16 through a ring of stages filled
+// by 16-byte cp.async copies.  A is K-contiguous and stays so in shared memory
+// (rows of 16 floats, padded to 20); B comes from its [K][N] form, which every
+// operand here has beside the other, so that neighbouring columns are pairs for
+// the packed multiply-adds (fma.rn.f32x2: half the issue slots of scalar ones).
+// Per four K values a thread reads TM + TN times 16 bytes for 2 TM TN packed
+// multiply-adds.  Every output is one chain over K in order (a split K: one
+// chain per part, the parts added in order).
+//
+// What bounds it: the FP32 pipe and, at 128 x 128, the registers that two CTAs
+// per SM leave (128 a thread).  Measured (GB300) at n = 10000, h = 2000, 2048
+// samples, where a GEMM's 2.05e10 multiply-adds take 509 us at the derived peak
+// of 80 TFLOP/s, against 128 x 128 x 16 tiles transposed through registers with
+// scalar multiply-adds: hidden 1830 -> 956 us, output 1313 -> 862, hidden adjoint
+// 1746 -> 914, weight gradients 1270 -> 990.  (4-byte copies that transposed both
+// operands on the way cost more than they saved below 128 x 128: hidden 1445 us.)
+// Small models: the weight gradients of n = 20, h = 40, 1024 samples, one tile,
+// 144 -> 12 us with the batch split.
+#include <algorithm>
+
 #include "gemm.cuh"
 
 namespace vqmc {
 namespace {
 
-constexpr int BM = 128, BN = 128, BK = 16;
+constexpr int BK = 16, kThreads = 256;
 
-template <typename T>
-struct Vec8;
-template <>
-struct Vec8<float> {
-  static __device__ __forceinline__ void load(const float* p, float* v) {
-    const float4 a = *reinterpret_cast<const float4*>(p);
-    const float4 b = *reinterpret_cast<const float4*>(p + 4);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-  }
-};
-template <>
-struct Vec8<bf16> {
-  static __device__ __forceinline__ void load(const bf16* p, float* v) {
-    const uint4 q = *reinterpret_cast<const uint4*>(p);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      v[2 * e] = __uint_as_float(w[e] << 16);
-      v[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-    }
-  }
+template <int TM, int TN>
+struct Tile {
+  static constexpr int BM = 16 * TM, BN = 16 * TN;
+  static constexpr int kStages = TM * TN >= 64 ? 3 : 4;
+  // A rows TM ty + i of 20 floats, 4 floats more every TM rows: the two ty of
+  // a warp on different banks
+  static constexpr int kLdA = 20, kA = BM * kLdA + 16 * 4;
+  static constexpr int kStage = kA + BK * BN;
+  static constexpr int kSmem = kStages * kStage * 4;
 };
 
-template <typename T>
-__device__ __forceinline__ float to_f(T x);
-template <>
-__device__ __forceinline__ float to_f<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ float to_f<bf16>(bf16 x) { return __bfloat162float(x); }
-template <typename T>
-__device__ __forceinline__ T of_f(float x);
-template <>
-__device__ __forceinline__ float of_f<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ bf16 of_f<bf16>(float x) { return __float2bfloat16_rn(x); }
-
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + expf(-x)); }
-// log sigma(x) and sigma(-x) of an output element from one exponential,
-// e = exp(-|x|): log sigma(x) = min(x, 0) - log(1 + e), sigma(-x) =
-// (x >= 0 ? e : 1) / (1 + e), on the hardware exp2/log2 approximations and
-// the approximate division (absolute error of the log term below 4e-7 for
-// 1 + e in (1, 2], relative error of sigma a few 2^-23: far inside the FP32
-// model's tolerances on log pi and the gradient)
-__device__ __forceinline__ void log_sigmoid_pair(float x, float& ls, float& sm) {
-  const float e = __expf(-fabsf(x));
-  ls = fminf(x, 0.0f) - __logf(1.0f + e);
-  sm = __fdividef(x >= 0.0f ? e : 1.0f, 1.0f + e);
+
+__device__ __forceinline__ uint64_t dup2(float x) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+// 16 bytes to shared memory, the first `bytes` of them from src, zeros beyond
+__device__ __forceinline__ void cp16(uint32_t dst, const float* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 
-// 8 consecutive K-elements of row r starting at k (zeros outside [.., khi) or r >= R)
-template <typename T>
-__device__ __forceinline__ void load8(const T* base, int ld, int r, int R, int k, int khi, float* v) {
-  if (r < R && k + 8 <= khi) {
-    Vec8<T>::load(base + (size_t)r * ld + k, v);
+// four consecutive floats; one 16-byte access where the address allows it and
+// all four are inside
+__device__ __forceinline__ void store4(float* p, const float (&x)[4], int valid) {
+  if (valid >= 4 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
   } else {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = (r < R && k + e < khi) ? to_f(base[(size_t)r * ld + k + e]) : 0.0f;
+    for (int j = 0; j < 4; ++j)
+      if (j < valid) p[j] = x[j];
   }
 }
+// signs of four consecutive spins (the first `valid`; +1 beyond)
+__device__ __forceinline__ void spins4(const int8_t* p, int valid, float (&s)[4]) {
+  uint32_t w = 0x01010101u;
+  if (valid >= 4 && (reinterpret_cast<uintptr_t>(p) & 3) == 0) {
+    w = __ldg(reinterpret_cast<const uint32_t*>(p));
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < valid && p[j] < 0) w |= 0x80u << (8 * j);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) s[j] = (w >> (8 * j + 7)) & 1u ? -1.0f : 1.0f;
+}
 
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const GemmArgs<T> g) {
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN + 4];
-  __shared__ float colbuf[16][BN];
-
+template <int OP, int TM, int TN>
+__global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<float> g, int kpart) {
+  using T = Tile<TM, TN>;
+  constexpr int BM = T::BM, BN = T::BN, kStages = T::kStages;
+  extern __shared__ __align__(16) float sm[];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  constexpr int op = OP;
+  // Tiles in launch order, heaviest K range first where the masks make the
+  // ranges uneven (as in gemm_tc.cu)
+  int tm = blockIdx.y, tn = blockIdx.x;
+  if (op == kOpHidden || op == kOpGA || op == kOpOut) {
+    const int L = blockIdx.y * gridDim.x + blockIdx.x;
+    tm = L % gridDim.y;
+    tn = op == kOpGA ? L / (int)gridDim.y : (int)gridDim.x - 1 - L / (int)gridDim.y;
+  }
+  const int m0 = tm * BM, n0 = tn * BN;
   const int m1 = min(m0 + BM, g.M), n1 = min(n0 + BN, g.N);
-  const int op = g.op;
-
-  if (op == kOpDV || op == kOpDW) {
-    if (gemm_tile_masked(op, m0, m1, n0, n1, g.n, g.h)) {
-      for (int q = tid; q < BM * BN; q += 256) {
+  constexpr bool wgrad = op == kOpDV || op == kOpDW;
+  if (wgrad && gemm_tile_masked(op, m0, m1, n0, n1, g.n, g.h)) {
+    if (gridDim.z == 1)
+      for (int q = tid; q < BM * BN; q += kThreads) {
         const int m = m0 + q / BN, nn = n0 + q % BN;
         if (m < g.M && nn < g.N) g.gout[(size_t)m * g.ldg + nn] = 0.0f;
       }
-      return;
-    }
+    return;
   }
   if (op == kOpOut && g.flip_rows) {
     // single-flip rows of the transverse field: a tile whose columns all
     // precede the flipped spin of each of its rows (one sample, no unflipped
     // row) contributes nothing the log-ratios read, so it is skipped
-    const long long ga = g.row0 + m0;
-    const int ia = (int)(ga % (g.n + 1));
-    const int last = m1 - 1 - m0;
-    if (ia + last < g.n && n0 + BN <= ia) return;
+    const int ia = (int)((g.row0 + m0) % (g.n + 1));
+    if (ia + m1 - 1 - m0 < g.n && n0 + BN <= ia) return;
   }
   int klo, khi;
   gemm_k_range(op, n0, n1, g.K, g.n, g.h, &klo, &khi);
   klo = klo / BK * BK;
+  if (gridDim.z > 1) klo = blockIdx.z * kpart, khi = min(khi, klo + kpart);
+  const int nk = khi > klo ? (khi - klo + BK - 1) / BK : 0;
 
-  float acc[8][8];
+  // A: a thread copies the 16 bytes tid % 4 of rows tid / 4, + 64, ...; B: 16
+  // bytes of the stage's 16 rows of BN floats
+  const int cr = tid >> 2, ck = 4 * (tid & 3);
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
+  auto issue = [&](int it) {
+    if (it < nk) {
+      const int k0 = klo + it * BK;
+      const uint32_t dst = base + (it % kStages) * T::kStage * 4;
+      const int bytes = max(0, min(16, 4 * (khi - k0 - ck)));
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+      for (int r = 0; r < BM; r += 64) {
+        const int m = m0 + cr + r;
+        const bool in = m < g.M && bytes > 0;
+        cp16(dst + 4 * ((cr + r) * T::kLdA + (cr + r) / TM * 4 + ck), g.A + (in ? (size_t)m * g.lda + k0 + ck : 0),
+             in ? bytes : 0);
+      }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+      for (int q = 0; q < BK * BN / 4; q += kThreads) {
+        const int r = (q + tid) / (BN / 4), c = (q + tid) % (BN / 4) * 4;
+        const bool in = k0 + r < khi && n0 + c < g.ldb;  // ldb: N padded to a multiple of 64
+        cp16(dst + 4 * (T::kA + r * BN + c), g.Bm + (in ? (size_t)(k0 + r) * g.ldb + n0 + c : 0), in ? 16 : 0);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
 
-  const int lr = tid >> 1, lk = (tid & 1) * 8;
-  const int passes = g.Bm2 ? 2 : 1;
-  for (int pass = 0; pass < passes; ++pass) {
-    const T* Bmat = pass == 0 ? g.Bm : g.Bm2;
-    float ra[8], rb[8];
-    int k0 = klo;
-    if (k0 < khi) {
-      load8(g.A, g.lda, m0 + lr, g.M, k0 + lk, khi, ra);
-      load8(Bmat, g.ldb, n0 + lr, g.N, k0 + lk, khi, rb);
+  uint64_t acc2[TM][TN / 2];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j) acc2[i][j] = 0ull;
+#pragma unroll
+  for (int s = 0; s < kStages - 1; ++s) issue(s);
+  for (int it = 0; it < nk; ++it) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();  // stage it has landed for all; stage it - 1 is free
+    issue(it + kStages - 1);
+    const float* as = sm + (it % kStages) * T::kStage + TM * ty * T::kLdA + 4 * ty;
+    const float* bs = sm + (it % kStages) * T::kStage + T::kA + 4 * tx;
+#pragma unroll
+    for (int k4 = 0; k4 < BK; k4 += 4) {
+      float4 a[TM];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(as + i * T::kLdA + k4);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        uint64_t b[TN / 2];
+#pragma unroll
+        for (int q = 0; q < TN / 4; ++q) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(bs + (k4 + kk) * BN + 64 * q);
+          b[2 * q] = v.x, b[2 * q + 1] = v.y;
+        }
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const uint64_t ai = dup2(kk == 0 ? a[i].x : kk == 1 ? a[i].y : kk == 2 ? a[i].z : a[i].w);
+#pragma unroll
+          for (int j = 0; j < TN / 2; ++j) acc2[i][j] = fma2(ai, b[j], acc2[i][j]);
+        }
+      }
     }
-    int buf = 0;
-    for (; k0 < khi; k0 += BK) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        As[buf][lk + e][lr] = ra[e];
-        Bs[buf][lk + e][lr] = rb[e];
-      }
-      __syncthreads();
-      if (k0 + BK < khi) {
-        load8(g.A, g.lda, m0 + lr, g.M, k0 + BK + lk, khi, ra);
-        load8(Bmat, g.ldb, n0 + lr, g.N, k0 + BK + lk, khi, rb);
-      }
-#pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 8]);
-        const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 8 + 4]);
-        const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 8]);
-        const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 8 + 4]);
-        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-      }
-      buf ^= 1;
-    }
-    __syncthreads();
   }
 
   // ---------------------------------------------------------------- epilogue
-  const int mb = m0 + ty * 8, nb = n0 + tx * 8;
-  float rowsum[8], colsum[8];
+  // columns in groups of four: group q starts at n0 + 64 q + 4 tx
+  const int mb = m0 + ty * TM;
+  float acc[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) rowsum[i] = 0.0f, colsum[i] = 0.0f;
-
-  if (op == kOpHidden) {
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int m = mb + i;
+    for (int j = 0; j < TN / 2; ++j) unpack2(acc2[i][j], acc[i][2 * j], acc[i][2 * j + 1]);
+  if constexpr (wgrad) {
+    const bool split = gridDim.z > 1;  // parts are stored as they are, the sum over them applies the mask
+    float* out = split ? g.part + (size_t)blockIdx.z * g.M * g.N : g.gout;
+    const int ld = split ? g.N : g.ldg;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int nn = nb + j;
-        if (m < g.M && nn < g.N) {
-          float v = acc[i][j] + g.bias[nn];
-          if (g.pre) g.pre[(size_t)m * g.ldpre + nn] = v;
-          v = g.act == VQMC_ACT_RELU ? fmaxf(v, 0.0f) : sigmoidf_(v);
-          const T tv = of_f<T>(v);
-          g.out[(size_t)m * g.ldo + nn] = tv;
-          if (g.out_t) g.out_t[(size_t)nn * g.ldt + m] = tv;
-        }
+    for (int i = 0; i < TM; ++i) {
+      if (mb + i >= g.M) continue;
+      const int cd = count_deg_le(mb + i, g.n, g.h);  // kept: W2 columns below it, W1^T columns from it on
+#pragma unroll
+      for (int q = 0; q < TN / 4; ++q) {
+        const int nn = n0 + 64 * q + 4 * tx;
+        float x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = split || (nn + j < cd) == (op == kOpDV) ? acc[i][4 * q + j] : 0.0f;
+        store4(out + (size_t)(mb + i) * ld + nn, x, g.N - nn);
       }
     }
-  } else if (op == kOpOut) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int m = mb + i;
-      const float cm = (g.coef && m < g.M) ? g.coef[m] : 0.0f;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int nn = nb + j;
-        if (m < g.M && nn < g.N) {
-          const float z = acc[i][j] + g.bias[nn];
-          const float s = g.S8[(size_t)m * g.lds8 + nn] > 0 ? 1.0f : -1.0f;
-          float ls, sm;
-          log_sigmoid_pair(s * z, ls, sm);
-          rowsum[i] += ls;
-          if (g.coef) {
-            const float d = cm * s * sm;
-            const T tv = of_f<T>(d);
-            g.out[(size_t)m * g.ldo + nn] = tv;
-            g.out_t[(size_t)nn * g.ldt + m] = tv;
-            colsum[j] += d;
-          }
-        }
-      }
-    }
-  } else if (op == kOpGA) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int m = mb + i;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int nn = nb + j;
-        if (m < g.M && nn < g.N) {
-          const float hv = to_f(g.aux[(size_t)m * g.ldaux + nn]);
-          const float dact = g.act == VQMC_ACT_RELU ? (hv > 0.0f ? 1.0f : 0.0f) : hv * (1.0f - hv);
-          const float v = acc[i][j] * dact;
-          g.out_t[(size_t)nn * g.ldt + m] = of_f<T>(v);
-          colsum[j] += v;
-        }
-      }
-    }
-  } else if (op == kOpDV || op == kOpDW) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int m = mb + i;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int nn = nb + j;
-        if (m < g.M && nn < g.N)
-          g.gout[(size_t)m * g.ldg + nn] = gemm_out_kept(op, m, nn, g.n, g.h) ? acc[i][j] : 0.0f;
-      }
-    }
-  } else if (op == kOpEloc) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int m = mb + i;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int nn = nb + j;
-        if (m < g.M && nn < g.N) {
-          const float s = g.S8[(size_t)m * g.lds8 + nn] > 0 ? 0.5f : -0.5f;
-          rowsum[i] = fmaf(s, acc[i][j], rowsum[i]);
-        }
-      }
-    }
+    return;
   }
+
+  float rowsum[TM], colsum[TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i) rowsum[i] = 0.0f;
+#pragma unroll
+  for (int j = 0; j < TN; ++j) colsum[j] = 0.0f;
+  // TM consecutive rows of column nn of the transposed output
+  auto store_t = [&](int nn, const float (&x)[TM]) {
+    if (nn >= g.N) return;
+    float* o = g.out_t + (size_t)nn * g.ldt + mb;  // ldt: a multiple of 64
+    if (mb + TM <= g.M) {
+#pragma unroll
+      for (int i = 0; i < TM; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+        if (mb + i < g.M) o[i] = x[i];
+    }
+  };
+  // prod: the logarithms of log sigma(x) = min(x, 0) - log(1 + e), e =
+  // exp(-|x|), are taken of the product of a row's TN factors 1 + e in (1, 2]
+  // (one rounding of 2^-24 each, where each logarithm has an absolute error
+  // of a few 2^-23)
+  float prod[TM];
+#pragma unroll
+  for (int i = 0; i < TM; ++i) prod[i] = 1.0f;
+#pragma unroll
+  for (int q = 0; q < TN / 4; ++q) {
+    const int nn = n0 + 64 * q + 4 * tx, valid = g.N - nn;
+    if (valid <= 0) continue;
+    float bias[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if constexpr (op == kOpHidden || op == kOpOut)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j < valid) bias[j] = g.bias[nn + j];
+    float t[4][TM];  // values for the transposed output
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const int m = mb + i;
+      float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      if (m < g.M) {
+        if constexpr (op == kOpHidden) {
+          float a[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            a[j] = acc[i][4 * q + j] + bias[j];
+            x[j] = g.act == VQMC_ACT_RELU ? fmaxf(a[j], 0.0f) : sigmoidf_(a[j]);
+          }
+          if (g.pre) store4(g.pre + (size_t)m * g.ldpre + nn, a, valid);
+          store4(g.out + (size_t)m * g.ldo + nn, x, valid);
+        } else if constexpr (op == kOpOut) {
+          // sigma(-x) = (x >= 0 ? e : 1) / (1 + e); hardware exp2 / log2
+          // approximations and the approximate division
+          float s[4];
+          spins4(g.S8 + (size_t)m * g.lds8 + nn, valid, s);
+          const float cm = g.coef ? g.coef[m] : 0.0f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float z = s[j] * (acc[i][4 * q + j] + bias[j]), e = __expf(-fabsf(z));
+            if (j < valid) rowsum[i] += fminf(z, 0.0f), prod[i] *= 1.0f + e;
+            if (g.coef && j < valid) {
+              x[j] = cm * s[j] * __fdividef(z >= 0.0f ? e : 1.0f, 1.0f + e);
+              colsum[4 * q + j] += x[j];
+            }
+          }
+          if (g.coef) store4(g.out + (size_t)m * g.ldo + nn, x, valid);
+        } else if constexpr (op == kOpGA) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (j < valid) {
+              const float hv = g.aux[(size_t)m * g.ldaux + nn + j];
+              x[j] = acc[i][4 * q + j] * (g.act == VQMC_ACT_RELU ? (hv > 0.0f ? 1.0f : 0.0f) : hv * (1.0f - hv));
+              colsum[4 * q + j] += x[j];
+            }
+          store4(g.out + (size_t)m * g.ldo + nn, x, valid);
+        } else {
+          float s[4];
+          spins4(g.S8 + (size_t)m * g.lds8 + nn, valid, s);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (j < valid) rowsum[i] = fmaf(0.5f * s[j], acc[i][4 * q + j], rowsum[i]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) t[j][i] = x[j];
+    }
+    if constexpr (op == kOpHidden || op == kOpOut || op == kOpGA)
+      if (op == kOpGA || (op == kOpHidden && g.out_t) || (op == kOpOut && g.coef))
+#pragma unroll
+        for (int j = 0; j < 4; ++j) store_t(nn + j, t[j]);
+  }
+  if constexpr (op == kOpOut)
+#pragma unroll
+    for (int i = 0; i < TM; ++i) rowsum[i] -= __logf(prod[i]);
 
   // row partials: reduce over the 16 tx lanes of each half-warp
   if (g.row_part && (op == kOpOut || op == kOpEloc)) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < TM; ++i) {
       float v = rowsum[i];
       v += __shfl_xor_sync(0xffffffffu, v, 1);
       v += __shfl_xor_sync(0xffffffffu, v, 2);
       v += __shfl_xor_sync(0xffffffffu, v, 4);
       v += __shfl_xor_sync(0xffffffffu, v, 8);
-      if (tx == 0 && mb + i < g.M) g.row_part[(size_t)blockIdx.x * g.ldr + mb + i] = v;
+      if (tx == 0 && mb + i < g.M) g.row_part[(size_t)tn * g.ldr + mb + i] = v;
     }
   }
   // column partials: reduce over the 16 ty rows in a fixed order
   if (g.col_part && ((op == kOpOut && g.coef) || op == kOpGA)) {
+    __syncthreads();  // the operand stages are consumed
+    float(*colbuf)[BN] = reinterpret_cast<float(*)[BN]>(sm);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) colbuf[ty][tx * 8 + j] = colsum[j];
+    for (int j = 0; j < TN; ++j) colbuf[ty][64 * (j / 4) + 4 * tx + j % 4] = colsum[j];
     __syncthreads();
     if (tid < BN) {
       float v = 0.0f;
 #pragma unroll
       for (int q = 0; q < 16; ++q) v += colbuf[q][tid];
-      if (n0 + tid < g.N) g.col_part[(size_t)blockIdx.y * g.ldc + n0 + tid] = v;
+      if (n0 + tid < g.N) g.col_part[(size_t)tm * g.ldc + n0 + tid] = v;
     }
   }
 }
 
-template <typename T>
-cudaError_t launch_simt(const GemmArgs<T>& a, cudaStream_t st) {
-  if (a.M <= 0 || a.N <= 0) return cudaSuccess;
-  dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM);
-  gemm_simt_kernel<T><<<grid, 256, 0, st>>>(a);
+// The parts of a split K, added in order; zero outside the mask.  One row per
+// blockIdx.y.
+__global__ void wgrad_sum_kernel(int op, int M, int N, int parts, const float* __restrict__ part, int n, int h,
+                                 float* __restrict__ gout, int ldg) {
+  const int m = blockIdx.y, nn = blockIdx.x * blockDim.x + threadIdx.x;
+  if (nn >= N) return;
+  float s = 0.0f;
+  if ((nn < count_deg_le(m, n, h)) == (op == kOpDV))
+    for (int z = 0; z < parts; ++z) s += part[((size_t)z * M + m) * N + nn];
+  gout[(size_t)m * ldg + nn] = s;
+}
+
+long long tiles(int M, int N, int BM, int BN) { return (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN); }
+
+template <int OP, int TM, int TN>
+cudaError_t launch_op(const GemmArgs<float>& a, int parts, int kpart, cudaStream_t st) {
+  using T = Tile<TM, TN>;
+  auto kern = gemm_simt_kernel<OP, TM, TN>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((a.N + T::BN - 1) / T::BN, (a.M + T::BM - 1) / T::BM, parts);
+  kern<<<grid, kThreads, T::kSmem, st>>>(a, kpart);
+  if (parts > 1)
+    wgrad_sum_kernel<<<dim3((a.N + 127) / 128, a.M), 128, 0, st>>>(a.op, a.M, a.N, parts, a.part, a.n, a.h, a.gout,
+                                                                   a.ldg);
   return cudaGetLastError();
+}
+
+template <int TM, int TN>
+cudaError_t launch_tile(const GemmArgs<float>& a, int parts, int kpart, cudaStream_t st) {
+  switch (a.op) {
+    case kOpHidden: return launch_op<kOpHidden, TM, TN>(a, 1, 0, st);
+    case kOpDV: return launch_op<kOpDV, TM, TN>(a, parts, kpart, st);
+    case kOpGA: return launch_op<kOpGA, TM, TN>(a, 1, 0, st);
+    case kOpDW: return launch_op<kOpDW, TM, TN>(a, parts, kpart, st);
+  }
+  if constexpr (TN == 8) {  // a row partial per 128 columns
+    if (a.op == kOpOut) return launch_op<kOpOut, TM, TN>(a, 1, 0, st);
+    if (a.op == kOpEloc) return launch_op<kOpEloc, TM, TN>(a, 1, 0, st);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t launch_gemm_simt_f32(const GemmArgs<float>& a, cudaStream_t st) { return launch_simt(a, st); }
+// Tile by the number of CTAs it gives: 128 x 128 from three CTAs per SM on
+// (below, the masks' uneven K ranges and the last wave cost more than its better
+// operand reuse gains: 256 tiles of the hidden GEMM above took 1103 us, 512 of 64
+// x 128 987), 64 x 128 from one and a half, else 64 x 64 (tim500's hidden GEMM,
+// 64 tiles: 70 -> 22 us); the ops with row partials keep 128 columns (a partial
+// per 128 columns).
+int gemm_simt_rows(int op, int M, int N, int sms) {
+  return tiles(M, N, 128, 128) >= 3ll * sms ? 128 : 64;
+}
+
+cudaError_t launch_gemm_simt_f32(const GemmArgs<float>& a, cudaStream_t st) {
+  if (a.M <= 0 || a.N <= 0) return cudaSuccess;
+  const int sms = a.sms > 0 ? a.sms : 1;
+  if (gemm_simt_rows(a.op, a.M, a.N, sms) == 128) return launch_tile<8, 8>(a, 1, 0, st);
+  if (a.op == kOpOut || a.op == kOpEloc || 2 * tiles(a.M, a.N, 64, 128) >= 3ll * sms) return launch_tile<4, 8>(a, 1, 0, st);
+  // few tiles: the weight gradients (K = the batch) also split K, as far as
+  // the scratch for the parts goes and with at least 64 samples each
+  int parts = 1, kpart = 0;
+  if ((a.op == kOpDV || a.op == kOpDW) && a.part) {
+    const long long want = 4ll * sms / tiles(a.M, a.N, 64, 64), cap = (long long)(a.part_cap / ((size_t)a.M * a.N));
+    parts = (int)std::max(1ll, std::min({want, cap, (long long)a.K / 64}));
+    kpart = ((a.K + parts - 1) / parts + BK - 1) / BK * BK;
+    parts = (a.K + kpart - 1) / kpart;
+  }
+  return launch_tile<4, 4>(a, parts, kpart, st);
+}
 
 }  // namespace vqmc

@@ -80,20 +80,22 @@ cudaError_t forward(const vqmc_ctx* c, int B, const int8_t* d_s, float* d_logp, 
   if (e != cudaSuccess) return e;
 
   GemmArgs<T> a{};
-  a.n = c->n, a.h = c->h, a.act = c->act, a.err = c->err;
+  a.n = c->n, a.h = c->h, a.act = c->act, a.err = c->err, a.sms = c->num_sms;
   a.op = kOpHidden;
   a.M = B, a.N = c->h, a.K = c->n;
   a.A = Sx, a.lda = c->np;
   a.Bm = reinterpret_cast<const T*>(c->w_s), a.ldb = c->np;
+  if constexpr (sizeof(T) == 4) a.Bm = reinterpret_cast<const T*>(c->wt_s) + c->hp, a.ldb = c->hp;  // [K][N] form
   a.bias = c->b1;
   a.out = H, a.ldo = c->hp;
   a.out_t = nullptr;  // the transposed activations feed only the adjoint, which this call does not run
   GemmArgs<T> z{};
-  z.n = c->n, z.h = c->h, z.act = c->act, z.err = c->err;
+  z.n = c->n, z.h = c->h, z.act = c->act, z.err = c->err, z.sms = c->num_sms;
   z.op = kOpOut;
   z.M = B, z.N = c->n, z.K = c->h;
   z.A = H, z.lda = c->hp;
   z.Bm = reinterpret_cast<const T*>(c->v_s), z.ldb = c->hp;
+  if constexpr (sizeof(T) == 4) z.Bm = reinterpret_cast<const T*>(c->vt_s), z.ldb = c->np;
   z.bias = c->b2;
   z.S8 = d_s, z.lds8 = c->n;
   z.row_part = part, z.ldr = ldb;

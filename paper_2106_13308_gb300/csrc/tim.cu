@@ -141,6 +141,7 @@ GemmArgs<T> chunk_args(const vqmc_ctx* c, GemmOp op, int rows) {
   a.h = c->h;
   a.act = c->act;
   a.err = c->err;
+  a.sms = c->num_sms;
   a.M = rows;
   if (op == kOpHidden) {
     a.N = c->h, a.K = c->n;
@@ -172,6 +173,9 @@ cudaError_t chunk_gemm<bf16>(const vqmc_ctx* c, GemmOp op, int rows, long long g
 template <>
 cudaError_t chunk_gemm<float>(const vqmc_ctx* c, GemmOp op, int rows, long long g0, cudaStream_t st) {
   GemmArgs<float> a = chunk_args<float>(c, op, rows);
+  // the CUDA-core GEMM reads its second operand in [K][N] form
+  if (op == kOpHidden) a.Bm = (const float*)c->wt_s + c->hp, a.ldb = c->hp;
+  else a.Bm = (const float*)c->vt_s, a.ldb = c->np;
   a.row_part = c->tim_row_part + g0, a.row0 = g0;
   return launch_gemm_simt_f32(a, st);
 }

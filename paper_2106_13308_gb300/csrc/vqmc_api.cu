@@ -77,6 +77,10 @@ GemmArgs<T> make_args(const vqmc_ctx* c, GemmOp op, int B, const int8_t* d_s, co
   a.ldr = c->row_part_ld;
   a.ldc = c->col_part_ld;
   a.err = c->err;
+  a.sms = c->num_sms;
+  // FP32: the output adjoint's row-major copy D is read by the hidden adjoint
+  // alone, so the weight gradients after it have it for the parts of a split K
+  if (c->prec == VQMC_PREC_FP32) a.part = (float*)c->D, a.part_cap = (size_t)c->Bmax * c->np;
   const int n = c->n, h = c->h;
   switch (op) {
     case kOpHidden:
@@ -159,7 +163,15 @@ cudaError_t launch_gemm(const vqmc_ctx* c, GemmOp op, int B, const int8_t* d_s, 
     return launch_gemm_tc_bf16(a, st);
   }
   GemmArgs<float> a = make_args<float>(c, op, B, d_s, coef, grad);
-  if (op == kOpEloc) a.Bm = c->J;
+  // the CUDA-core GEMM reads its second operand in [K][N] form
+  switch (op) {
+    case kOpHidden: a.Bm = (const float*)c->wt_s + c->hp, a.ldb = c->hp; break;  // row j = input j
+    case kOpOut: a.Bm = (const float*)c->vt_s, a.ldb = c->np; break;
+    case kOpDV: a.Bm = (const float*)c->H, a.ldb = c->hp; break;
+    case kOpGA: a.Bm = (const float*)c->v_s, a.ldb = c->hp, a.out = c->GA, a.ldo = c->hp; break;
+    case kOpDW: a.Bm = c->GA, a.ldb = c->hp; break;
+    case kOpEloc: a.Bm = c->J; break;  // symmetric
+  }
   return launch_gemm_simt_f32(a, st);
 }
 
@@ -177,12 +189,16 @@ namespace {
 vqmc_status backward_from_operands(vqmc_ctx* c, int B, const int8_t* d_s, const float* gout, float* grad,
                                    cudaStream_t st, const AdamStep* fuse = nullptr, bool hidden_done = false) {
   const int n = c->n, h = c->h;
-  const int mtiles = (B + 127) / 128;
+  // column partials: one per tile row
+  auto mtiles = [&](GemmOp op, int N) {
+    const int rows = c->prec == VQMC_PREC_FP32 ? gemm_simt_rows(op, B, N, c->num_sms) : 128;
+    return (B + rows - 1) / rows;
+  };
   if (!hidden_done) VQ_CUDA(launch_gemm(c, kOpHidden, B, d_s, nullptr, nullptr, st));
   VQ_CUDA(launch_gemm(c, kOpOut, B, d_s, gout, nullptr, st));
-  VQ_CUDA(launch_col_sum(c, n, mtiles, grad + (size_t)2 * n * h + h, st));  // db2
+  VQ_CUDA(launch_col_sum(c, n, mtiles(kOpOut, n), grad + (size_t)2 * n * h + h, st));  // db2
   VQ_CUDA(launch_gemm(c, kOpGA, B, d_s, nullptr, nullptr, st));
-  VQ_CUDA(launch_col_sum(c, h, mtiles, grad + (size_t)n * h, st));          // db1
+  VQ_CUDA(launch_col_sum(c, h, mtiles(kOpGA, h), grad + (size_t)n * h, st));          // db1
   VQ_CUDA(launch_gemm(c, kOpDV, B, d_s, nullptr, grad, st, fuse));          // dW2
   VQ_CUDA(launch_gemm(c, kOpDW, B, d_s, nullptr, grad, st, fuse));          // dW1^T
   return VQMC_OK;
@@ -287,6 +303,7 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
   VQ_ALLOC(c->D, (size_t)Bmax * c->np * es);
   VQ_ALLOC(c->Dt, (size_t)n * c->Bp * es);
   VQ_ALLOC(c->GAt, (size_t)h * c->Bp * es);
+  if (c->prec == VQMC_PREC_FP32) VQ_ALLOC(c->GA, (size_t)Bmax * c->hp * es);
   VQ_ALLOC(c->logp, (size_t)Bmax * 4);
   VQ_ALLOC(c->coef, (size_t)Bmax * 4);
   VQ_ALLOC(c->ones, (size_t)Bmax * 4);
@@ -299,7 +316,7 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
   c->row_part_tiles = (n + 127) / 128;
   c->row_part_ld = c->Bp;
   VQ_ALLOC(c->row_part, (size_t)c->row_part_tiles * c->row_part_ld * 4);
-  c->col_part_tiles = (Bmax + 127) / 128;
+  c->col_part_tiles = (Bmax + 63) / 64;
   c->col_part_ld = c->np > c->hp ? c->np : c->hp;
   VQ_ALLOC(c->col_part, (size_t)c->col_part_tiles * c->col_part_ld * 4);
   VQ_ALLOC(c->err, 16);
@@ -417,7 +434,7 @@ void vqmc_destroy(vqmc_ctx* c) {
   }
   void* ptrs[] = {c->theta, c->adam_m, c->adam_v, c->grad, c->wt_s, c->v_s, c->w_s, c->vt_s, c->row_ptr,
                   c->col, c->w, c->field, c->J, c->J_hi, c->J_lo, c->S, c->E, c->Sx, c->St, c->H, c->Ht,
-                  c->D, c->Dt, c->GAt, c->logp, c->coef, c->stats, c->row_part, c->col_part, c->err,
+                  c->D, c->Dt, c->GAt, c->GA, c->logp, c->coef, c->stats, c->row_part, c->col_part, c->err,
                   c->step_stats, c->Sbits, c->eloc_part, c->eloc_slice, c->erow, c->alpha, c->tim_A,
                   c->tim_S8, c->tim_H, c->tim_row_part, c->sr_A, c->sr_x, c->sr_ones, c->sr_xinv,
                   c->sr_events, c->dstate, c->ones};
@@ -645,7 +662,7 @@ vqmc_status vqmc_step(vqmc_ctx* c, int32_t B, vqmc_stream stream, vqmc_step_stat
     // sampler (+ operand layouts unless the tensor-core sampler writes them), energy (dense: GEMM +
     // finish; sparse: [pack,] slices [, slice sum]), stats (with the Adam step counter), 7 gradient
     // kernels, [Adam with the weight-copy refresh unless fused into the gradient GEMMs,] bias Adam,
-    // [2 L2 prefetches,] step stats
+    // [2 L2 prefetches,] step stats; the sums over a split batch of small FP32 models are not counted
     const int sampler = tc ? 1 : 2;
     const int energy = !sparse ? 2 : (tc ? 0 : 1) + 1 + (c->eloc_slices > 1 ? 1 : 0);
     c->launches += sampler + energy + tim_launches + 1 + 7 + (fuse ? 1 : 2) + (tc ? 2 : 0) + 1;

@@ -29,15 +29,22 @@
 // neighbouring pairs (one octet) of one virtual warp, so the solver finishes
 // the tree from its 8 leaves and the partial sums of the other octets.
 //
-// What bounds it: the chain from one draw to the next (about 250 cycles, on two
+// What bounds it: the chain from one draw to the next (about 220 cycles, on two
 // of the CTA's eight warps) up to about 1000 hidden units, beyond it the issue
-// slots and shared-memory reads of the Z and U phases (2 bytes per multiply-add);
+// slots and shared-memory reads of the Z and U phases (2 bytes per multiply-add;
+// at n = h = 2000 55% of the issue slots and 60% of the load/store pipe are busy);
 // two CTAs on an SM overlap one's draws with the other's GEMMs.  Measured
 // (GB300), against one step at a time with a reduction over the CTA's lanes for
-// every draw: n = h = 1000, 1024 samples (BF16) 1440 -> 320 us; n = h = 2000,
-// 8192 samples 8580 -> 3990 us; n = 10000, h = 2000, 2048 samples (FP32) 7780 ->
-// 5600 us (15 TFLOP/s).
+// every draw: a sampling and energy pass at n = h = 1000, 1024 samples (BF16)
+// 1457 -> 293 us; a training step at n = h = 2000, 8192 samples (BF16) 9194 ->
+// 4118 us; the draws alone at n = 10000, h = 2000, 2048 samples (FP32) 7780 ->
+// 5250 us (16 TFLOP/s).  The code stays near the instruction cache's 32 KB: at
+// 47 KB (loops peeled, branches not known to be uniform) it ran at 2.7 cycles per
+// instruction.  No per-step store in the solver (25 cycles each, 70 behind a
+// divergent branch): the spins are written after a block.
 #pragma once
+
+#include <type_traits>
 
 #include "sampler.cuh"
 
@@ -74,9 +81,9 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-// 16 bytes from global to shared memory (zeros if !in), asynchronously
-__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool in) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+// 16 bytes from global to shared memory, asynchronously
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -108,6 +115,14 @@ struct Raw<bf16> {
   static __device__ __forceinline__ uint64_t f32(two x) {
     return pack2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
   }
+  // zero if !in; volatile: issued where it stands (before the draws)
+  static __device__ __forceinline__ four ld4(const bf16* p, bool in) {
+    four v;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\tmov.b64 %0, 0;\n\t@q ld.global.nc.b64 %0, [%1];\n\t}"
+                 : "=l"(v)
+                 : "l"(p), "r"((int)in));
+    return v;
+  }
   static __device__ __forceinline__ uint64_t lo(const four& x) { return f32((uint32_t)x); }
   static __device__ __forceinline__ uint64_t hi(const four& x) { return f32((uint32_t)(x >> 32)); }
 };
@@ -116,6 +131,15 @@ struct Raw<float> {
   using two = uint64_t;
   using four = ulonglong2;
   static __device__ __forceinline__ uint64_t f32(two x) { return x; }
+  static __device__ __forceinline__ four ld4(const float* p, bool in) {
+    four v;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %3, 0;\n\tmov.b64 %0, 0;\n\tmov.b64 %1, 0;\n\t"
+        "@q ld.global.nc.v2.b64 {%0, %1}, [%2];\n\t}"
+        : "=l"(v.x), "=l"(v.y)
+        : "l"(p), "r"((int)in));
+    return v;
+  }
   static __device__ __forceinline__ uint64_t lo(const four& x) { return x.x; }
   static __device__ __forceinline__ uint64_t hi(const four& x) { return x.y; }
 };
@@ -174,9 +198,8 @@ struct BlockSampler {
     float zb, lg, post[GW == 4 ? 6 : 2];
   };
 
-  // The weights reach shared memory through a ring per warp (cp.async, no
-  // other warp involved): a stage holds 4 rows x 64 units of W2 (one round of
-  // Z) or 2 rows x 128 units of W1 (2 steps of a round of U).
+  // W2 reaches shared memory through a ring per warp (cp.async, no other warp
+  // involved): a stage holds 4 rows x 64 units, one round of Z.
   static constexpr int kStageBytes = 256 * (int)sizeof(WT);
   static constexpr int kDepth = sizeof(WT) == 2 ? 4 : 2;
   static constexpr int kRingBytes = kDepth * kStageBytes;
@@ -211,47 +234,21 @@ struct BlockSampler {
     return pack2(g1(lo), g1(hi));
   }
 
-  // What a warp streams through its ring: the W1 rows of its rounds of U of
-  // one block, then the W2 rows of its first Z task of the next block (of
-  // every further task by itself).
+  // What a warp streams through its ring: the W2 rows of its first Z task of
+  // the next block (of every further task by itself).
   struct Stream {
     const WT* p;     // this lane's source of the next stage
-    int left, inc;   // stages left of this run, elements from one to the next
-    int half;        // FP32: elements from a stage's first copy to its second
-    int r, rows;     // the lane's first row of the stage, and the rows there are (beyond: zeros)
-    int k, steps;    // U: first unit of the warp's run, steps of the block
-    const WT* u;     // U: first row, at the lane's place in a stage
-    const WT* z;     // Z: the run that follows U
-    int zn;
+    int left;        // stages left
     uint32_t slot;   // byte offset of the next stage in the ring
   };
   static constexpr int kCol = 16 / (int)sizeof(WT);  // weights per lane and copy
-  static constexpr int kZLanes = 64 / kCol;          // lanes per row of a Z stage
-  static constexpr int kULanes = 128 / kCol;         // and of a U stage
+  static constexpr int kZLanes = 64 / kCol;          // lanes per row of a stage
   static constexpr int kCopies = kStageBytes / 512;  // per lane and stage
-  static __device__ __forceinline__ void next_run(Stream& x, int hp, int lane) {
-    if (x.k < hp) {
-      const bool in = x.k + (lane % kULanes) * kCol < hp;
-      x.p = in ? x.u + x.k : x.u;
-      x.r = in ? lane / kULanes : kSteps, x.rows = x.steps;
-      x.left = (x.steps + 1) / 2, x.inc = 2 * hp, x.half = hp;
-      x.k += 128 * kWarps;
-    } else {
-      x.p = x.z, x.left = x.zn, x.inc = RL, x.half = 2 * hp;
-      x.r = 0, x.rows = 1 << 30;
-      x.zn = 0;
-    }
-  }
   static __device__ __forceinline__ void issue(Stream& x, uint32_t ring, int hp, int lane) {
-    if (x.left == 0) next_run(x, hp, lane);
     if (x.left > 0) {
-      const uint32_t dst = ring + x.slot + 16 * lane;
 #pragma unroll
-      for (int j = 0; j < kCopies; ++j) {
-        const bool in = x.r + j < x.rows;  // (a second copy: the next row of U; of Z all rows are there)
-        cp16(dst + 512 * j, in ? x.p + j * x.half : x.p, in);
-      }
-      x.p += x.inc, x.r += 2, --x.left;
+      for (int j = 0; j < kCopies; ++j) cp16(ring + x.slot + 16 * lane + 512 * j, x.p + j * (32 / kZLanes) * hp);
+      x.p += RL, --x.left;
     }
     cp_commit();
     x.slot = (x.slot + kStageBytes) & (kRingBytes - 1);
@@ -259,13 +256,11 @@ struct BlockSampler {
   static __device__ __forceinline__ int rounds(int vw, int pairs) {  // in which some lane's pair is complete
     return pairs > vw * 32 ? (pairs - vw * 32 + GL - 1) / GL : 0;
   }
-  // the run of Z task (vw, 4 steps from e); sampler_rows() leaves room past the last step
-  static __device__ __forceinline__ void add_z(Stream& x, const WT* v, int hp, int e, int vw, int lane, int pairs) {
-    x.z = v + (unsigned)((e + lane / kZLanes) * hp + 64 * vw + (lane % kZLanes) * kCol);
-    x.zn = rounds(vw, pairs);
-  }
-  static __device__ __forceinline__ void start(Stream& x, uint32_t ring, int hp, int lane) {
-    x.slot = 0, x.left = 0;
+  // starts the stream of Z task (vw, 4 steps from e); sampler_rows() leaves room past the last step
+  static __device__ __forceinline__ void start(Stream& x, uint32_t ring, const WT* v, int hp, int e, int vw, int lane,
+                                               int pairs) {
+    x.p = v + (unsigned)((e + lane / kZLanes) * hp + 64 * vw + (lane % kZLanes) * kCol);
+    x.left = rounds(vw, pairs), x.slot = 0;
 #pragma unroll 1
     for (int d = 0; d < kDepth; ++d) issue(x, ring, hp, lane);
   }
@@ -350,15 +345,16 @@ struct BlockSampler {
   // compare) is about 200 cycles; a spin has two values, so both logits of step
   // t + 1 are begun before spin t is known, and each iteration finishes the two
   // logits of step t beside the first half of step t + 1's.  Only the units
-  // that complete with spin t differ between the two.  Stores are made by all
-  // of a sample's lanes alike (a divergent store costs about 70 cycles).
-  // A: the group's units of sample 0 in the state; over: the group's steps end
-  // with this block.
+  // that complete with spin t differ between the two.  Nothing is stored per
+  // step (a store costs about 25 cycles there, a divergent one 70).
+  // A: the group's units of sample 0 in the state; multi: several units may
+  // complete with one spin; over: the group's steps end with this block.
   static __device__ __forceinline__ void solve(const Tables& tb, Drawn& out, const LeafSum* Z, const float* T, Post* P,
-                                               uint64_t* SP, float* A, int steps, int wg, int sw, int lane, bool over) {
+                                               uint64_t* SP, float* A, int steps, int wg, int sw, int lane, bool multi,
+                                               bool over) {
     const int s = 4 * sw + (lane >> 3), l = lane & 7;
     // what joins the group's tree to a logit: one (step, sample) per lane and turn
-#pragma unroll 1
+#pragma unroll
     for (int i = lane; i < 4 * kSteps; i += 32) {
       const int t = i >> 2, sq = 4 * sw + (i & 3);
       Post x{};
@@ -399,22 +395,23 @@ struct BlockSampler {
     uint64_t w = 0ull;  // W1 of spin t - 1
     bool up = true;
     uint32_t bits = 0;
-#pragma unroll 1
-    for (int t = 0; t < steps; ++t) {
+    float xlo = 0.0f, xhi = 0.0f;  // s z of steps l and l + 8
+    // one step; MULTI: several units may complete with one spin
+    auto step = [&](int t, auto multi) {
+      constexpr bool MULTI = decltype(multi)::value;
       const int tn = min(t + 1, steps - 1);
       const ulonglong2 rn = *reinterpret_cast<const ulonglong2*>(zr + tn * kSamples * kLeaves);
       const ulonglong2 vwn = *reinterpret_cast<const ulonglong2*>(&tb.leaf[tn][l]);
       const float4 pz = *reinterpret_cast<const float4*>(P + t * kSamples + s);
-      const int dn = t + 1 < steps ? uniform(tb.done[tn]) : u;
+      int dn = tb.done[tn];
+      if constexpr (MULTI || !RELU) dn = uniform(dn);
       // spin t - 1 is known: its pre-activations and activations
       const float sv = up ? 1.0f : -1.0f;
       unpack2(fma2(w, pack2(sv, sv), pack2(a0, a1)), a0, a1);
       w = vw.y;
       g0 = up ? p0 : m0, g1_ = up ? p1 : m1;
       m0 = p0 = g0, m1 = p1 = g1_;
-      // the units that complete with spin t, for both of its values: all but
-      // the last (there is rarely more than one) in a loop, so that the rest
-      // of the iteration is straight code
+      // the units that complete with spin t, for both of its values
       float w0, w1;
       unpack2(w, w0, w1);
       auto complete = [&](bool any) {
@@ -425,9 +422,10 @@ struct BlockSampler {
         m0 = lo ? fm : m0, p0 = lo ? fp : p0;
         m1 = hi ? fm : m1, p1 = hi ? fp : p1;
       };
+      if constexpr (MULTI) {
 #pragma unroll 1
-      for (; u + 1 < dn; ++u) complete(true);
-      if constexpr (RELU) {
+        for (; u < dn; ++u) complete(true);
+      } else if constexpr (RELU) {
         complete(u < dn);
       } else {
         if (u < dn) complete(true);
@@ -448,12 +446,27 @@ struct BlockSampler {
       vw = vwn;
       const float z = up ? zp : zm;
       up = z > pz.y;  // u < sigma(z)
-      const float sn = up ? 1.0f : -1.0f;
-      SP[t * kSamples + s] = pack2(sn, sn);
-      out.x[t * kSamples + s] = up ? z : -z;
+      const float x = up ? z : -z;
+      xlo = t == l ? x : xlo, xhi = t == l + 8 ? x : xhi;
       bits |= (up ? 1u : 0u) << t;
+    };
+    if (multi) {
+#pragma unroll 1
+      for (int t = 0; t < steps; ++t) step(t, std::true_type{});
+    } else {
+#pragma unroll 1
+      for (int t = 0; t < steps; t += 2) {
+        step(t, std::false_type{});
+        if (t + 1 < steps) step(t + 1, std::false_type{});
+      }
     }
     out.bits[s] = bits;
+    out.x[l * kSamples + s] = xlo, out.x[(l + 8) * kSamples + s] = xhi;
+#pragma unroll
+    for (int t = l; t < kSteps; t += 8) {
+      const float sn = (bits >> t) & 1u ? 1.0f : -1.0f;
+      SP[t * kSamples + s] = pack2(sn, sn);
+    }
     // the group's state back: g1 if its steps are over
     const float sv = up ? 1.0f : -1.0f;
     const uint64_t a = fma2(w, pack2(sv, sv), pack2(a0, a1));
@@ -565,7 +578,6 @@ __global__ void __launch_bounds__(kThreads, 2) sampler_kernel(const SamplerArgs 
   Block b{0, 0, 0, 0}, nb{0, 0, 0, 0}, prev{0, 0, 0, 0};  // e0 == e1: none
   float lp = 0.0f;
   typename K::Stream st{};
-  st.k = hp;  // no U before the first block
 #pragma unroll 1
   for (int turn = -2;; ++turn) {
     const int par = turn & 1, steps = b.e1 - b.e0;
@@ -578,27 +590,34 @@ __global__ void __launch_bounds__(kThreads, 2) sampler_kernel(const SamplerArgs 
         if (t0 >= steps) continue;
         if (GW > 2 && task != warp) {
           __syncwarp();
-          K::add_z(st, v, hp, b.e0 + t0, vw, lane, pairs);
-          K::start(st, ring_s, hp, lane);
+          K::start(st, ring_s, v, hp, b.e0 + t0, vw, lane, pairs);
         }
         K::z_task(st, ring, ring_s, hp, A, zero, t0, vw, lane, pairs, vw == gs >> 2, gs & 3, Z, T);
       }
     }
     __syncthreads();  // Z and T complete
     const bool more = nb.e1 > nb.e0;
-    if (steps > 0 && more) {
-      // U of this block, then the next block's Z
-      st.u = wt + (unsigned)((b.e0 + 1 + lane / K::kULanes) * hp + min((lane % K::kULanes) * K::kCol, hp - K::kCol));
-      st.k = kGroup * (b.grp + 1) + 128 * warp, st.steps = steps;
-      K::add_z(st, v, hp, nb.e0 + kTI * (warp & 3), warp >> 2, lane,
+    // requested before the draws: the weights of this warp's first round of U
+    // (128 units, four consecutive ones per lane) and of its next Z task
+    const bool u_todo = steps > 0 && more;
+    const int k1 = kGroup * (b.grp + 1) + 128 * warp;
+    const int ue = b.e0 + 1;  // W1 row of the block's first input
+    constexpr int kAhead = sizeof(WT) == 2 ? kSteps : kSteps / 2;
+    typename R::four w[kAhead];
+    auto load = [&](int t, int k) {
+      w[t % kAhead] = R::ld4(wt + (unsigned)((ue + t) * hp + k + 4 * lane), t < steps && k + 4 * lane < hp);
+    };
+    if (u_todo) {
+#pragma unroll
+      for (int t = 0; t < kAhead; ++t) load(t, k1);
+      K::start(st, ring_s, v, hp, nb.e0 + kTI * (warp & 3), warp >> 2, lane,
                warp < 4 * GW && kTI * (warp & 3) < nb.e1 - nb.e0 ? kLeaves * nb.grp : 0);
-      K::start(st, ring_s, hp, lane);
     }
     if (warp >= kWarps - kSolvers) {
       if (steps > 0) {
         const int k0 = kGroup * b.grp, gs = b.grp % (4 * GW);
         K::solve(tables[par], drawn[par], Z, T, P, SP, A + k0 / kChunk * K::kStateChunk + k0 % kChunk, steps, gs >> 2,
-                 warp - (kWarps - kSolvers), lane, nb.grp != b.grp);
+                 warp - (kWarps - kSolvers), lane, h > n || (h == n && b.e0 == 0), nb.grp != b.grp);
       }
     } else if (warp == 2) {
       if (lane == 0) {
@@ -621,9 +640,8 @@ __global__ void __launch_bounds__(kThreads, 2) sampler_kernel(const SamplerArgs 
       continue;
     }
     // ------------------------------------------------------------- U
-    // 128 units per warp and round, four consecutive ones per lane
 #pragma unroll 1
-    for (int k = kGroup * (prev.grp + 1) + 128 * warp; k < hp; k += 128 * kWarps) {
+    for (int k = k1; k < hp; k += 128 * kWarps) {
       const int kl = k + 4 * lane;
       const bool in = kl < hp;
       float* a = A + kl / kChunk * K::kStateChunk + kl % kChunk;
@@ -634,27 +652,26 @@ __global__ void __launch_bounds__(kThreads, 2) sampler_kernel(const SamplerArgs 
         if (in) x = *reinterpret_cast<const ulonglong2*>(a + s * kChunk);
         a0[s] = x.x, a1[s] = x.y;
       }
-#pragma unroll 1
-      for (int t = 0; t < steps; t += 2) {
-        cp_wait<K::kDepth - 1>();
-        __syncwarp();
-        const typename R::four* w = reinterpret_cast<const typename R::four*>(ring + st.slot) + lane;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {  // past the last step the weights are zero
-          const uint64_t u0 = R::lo(w[32 * j]), u1 = R::hi(w[32 * j]);
-          const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(SP + (t + j) * kSamples);
+      for (int t = 0; t < kSteps; ++t) {
+        if (t >= steps) break;
+        const uint64_t u0 = R::lo(w[t % kAhead]), u1 = R::hi(w[t % kAhead]);
+        const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(SP + t * kSamples);
 #pragma unroll
-          for (int s = 0; s < kSamples; s += 2) {
-            const ulonglong2 x = sp[s / 2];
-            a0[s] = fma2(u0, x.x, a0[s]);
-            a1[s] = fma2(u1, x.x, a1[s]);
-            a0[s + 1] = fma2(u0, x.y, a0[s + 1]);
-            a1[s + 1] = fma2(u1, x.y, a1[s + 1]);
-          }
+        for (int s = 0; s < kSamples; s += 2) {
+          const ulonglong2 x = sp[s / 2];
+          a0[s] = fma2(u0, x.x, a0[s]);
+          a1[s] = fma2(u1, x.x, a1[s]);
+          a0[s + 1] = fma2(u0, x.y, a0[s + 1]);
+          a1[s + 1] = fma2(u1, x.y, a1[s + 1]);
         }
-        __syncwarp();
-        K::issue(st, ring_s, hp, lane);
+        // 16 rows in registers: the next round's; 8 (FP32): this round's second half
+        if (kAhead == kSteps) load(t, k + 128 * kWarps);
+        else if (t + kAhead < kSteps) load(t + kAhead, k);
       }
+      if (kAhead < kSteps)
+#pragma unroll
+        for (int t = 0; t < kAhead; ++t) load(t, k + 128 * kWarps);
       if (in)
 #pragma unroll
         for (int s = 0; s < kSamples; ++s)

@@ -29,11 +29,22 @@
 // lanes per sample, each lane owning every 8th step of a segment and partial
 // sums of all the block's recent units) and then write the block's spins as
 // the update GEMM's operand; while they solve, warps 2-3 merge the previous
-// block's recent g1 into the Z operand, prepare the next block's logits and
-// recent-unit weights and write out the previous block's spins; warp 4 lane 0
-// streams 128 x 64 BF16 weight tiles with TMA into a ring of six tiles,
-// consumed in two slots of three; warp 5 lane 0 issues the MMAs.  Every wait is bounded; after a failed wait the CTA
-// raises the timeout bit and runs on without waiting, so it still finishes.
+// block's recent g1 into the Z operand, prepare the next block's schedule,
+// logits and recent-unit weights, write out the previous block's spins and add
+// up its log pi; one thread of warp 4 streams 128 x 64 BF16 weight tiles with
+// TMA into a ring of six tiles, consumed in two slots of three; one of warp 5
+// issues the MMAs.  Every wait is bounded; after a failed wait the CTA raises
+// the timeout bit and runs on without waiting, so it still finishes.
+//
+// What bounds it: the chain of the solver's segments, about 550 cycles each,
+// then warps 2-3 (models of few units per block), and some 3,300 cycles from one
+// block's last draw to the next one's first.  Measured (GB300, n = 10000, h =
+// 2000, 1024 samples with log pi): 1264 -> 742 us; n = 500, h = 193: 138 -> 92
+// us.  What that took, the arithmetic unchanged: warp-uniform control flow made
+// known to the compiler (the warp index, the segment bounds) and one elected
+// thread per issuing warp; one copy of each piece of code (280 -> 90 KB; the
+// instruction cache holds 32); predicated stores in place of branches; log pi
+// and the next block's schedule moved to warps 2-3.
 #include <algorithm>
 #include <type_traits>
 
@@ -51,12 +62,10 @@ constexpr int kRmax = 32;                  // recent units per block
 constexpr int kNStage = 6;                 // weight tiles in the ring
 constexpr int kTileBytes = 128 * 64 * 2;   // one 128 x 64 BF16 tile
 // The ring is consumed in slots of up to three tiles (48 KB): one
-// full-barrier wait and one commit per slot.  The single thread that issues
-// the MMAs pays a fixed cost for every wait and every commit, comparable to
-// the tensor work of an N = 16 tile, so grouping tiles cuts the time per
-// tile.  A slot's tiles that are consecutive 64-column chunks of the same
-// rows arrive in one copy: the copy engine's time goes by copies more than by
-// bytes (a 32 KB box streams about twice as fast as two 16 KB boxes).
+// full-barrier wait and one commit per slot.  A slot's tiles that are
+// consecutive 64-column chunks of the same rows arrive in one copy: the copy
+// engine's time goes by copies more than by bytes (a 32 KB box streams about
+// twice as fast as two 16 KB boxes).
 constexpr int kSlotTiles = 3;
 constexpr int kNSlot = kNStage / kSlotTiles;
 constexpr int kMaxHp = 2048;               // hidden units (padded) in TMEM
@@ -92,15 +101,15 @@ constexpr int kOffP = kOffLG + 2 * kDrows * kS * 4;            // recent pre-act
 constexpr int kOffWr = kOffP + kRmax * kS * 4;                 // W1 of recent units [kDrows][kLdW] bf16
 constexpr int kOffVr = kOffWr + kDrows * kLdW * 2;             // W2 of recent units [kDrows][kLdW] bf16
 constexpr int kOffPS = kOffVr + kDrows * kLdW * 2;             // solver: g1 of the recent units [16][kLdP]
-constexpr int kOffHF = kOffPS + kS * kLdP * 4;                 // (unused)
-constexpr int kOffSB = kOffHF + kS * kLdP * 4;                 // drawn spins, bit e%32 of word [2][16][e/32]
-constexpr int kOffCU = kOffSB + 2 * kS * (kDmax / 32) * 4;     // completion step of each recent unit, [kRmax] int
-constexpr int kOffBar = kOffCU + (kDmax + 8) * 4;              // mbarriers + slots
+constexpr int kOffSB = kOffPS + kS * kLdP * 4;                 // drawn spins, bit e%32 of word [2][16][e/32]
+constexpr int kBlkInts = kRmax + 4;                            // completion step of each recent unit, then klo, R, zvalid
+constexpr int kOffCU = kOffSB + 2 * kS * (kDmax / 32) * 4;     // [2][kBlkInts] int
+constexpr int kOffBar = kOffCU + 2 * kBlkInts * 4;              // mbarriers + slots
 constexpr int kSmemBytes = 1024 + kOffBar + 128;
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 
 struct TcArgs {
-  int n, h, hp, B, D, act;
+  int n, h, hp, B, D;
   const bf16* w;      // w_s [h][np]: row k = W1[k] (column j-1 = input j)
   int np;
   const bf16* v;      // v_s  [rows][hp]: row r = W2[r] (output r + 1)
@@ -142,34 +151,17 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 // the two BF16 weights of a word, widened (exactly) to an FP32 pair
 __device__ __forceinline__ uint64_t bf2(uint32_t w) { return pk2(bf_lo(w), bf_hi(w)); }
 
-// bounded wait that gives up at once after any failure in the CTA; with
-// backoff the polling thread sleeps between tries so that it takes no issue
-// slots from a busy warp on the same sub-partition
-// The same wait polling with mbarrier.test_wait, which returns at once: for
-// the MMA issuer's waits on landed tiles, which are usually already complete
-// (a try_wait there costs the issuing thread about 190 cycles even then),
-// and for the single threads of the producer and the MMA issuer on the
-// block hand-offs, where a try_wait's suspension delays the reaction.
-__device__ __forceinline__ bool test_or_abort(uint32_t bar, uint32_t parity, volatile int* abort, uint32_t* err) {
-  for (long long it = 0; it < kSpinLimit; ++it) {
-    if (mbar_test_wait(bar, parity)) return true;
-    if ((it & 255) == 255 && *abort) return false;
-  }
-  atomicOr(err, kErrTimeout);
-  *abort = 1;
-  return false;
+// *p = x where ok holds, as a predicated store (a branch around one costs the
+// warp some 70 cycles)
+__device__ __forceinline__ void store_if(bool ok, float* p, float x) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t@p st.shared.f32 [%1], %2;\n\t}" ::"r"((int)ok),
+               "r"(smem_u32(p)), "f"(x)
+               : "memory");
 }
-__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort, uint32_t* err,
-                                              bool backoff = false) {
-  if (*abort) return false;
-  for (long long it = 0; it < kSpinLimit; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255) == 255 && *abort) return false;
-    if (backoff) __nanosleep(64);
-  }
-  atomicOr(err, kErrTimeout);
-  *abort = 1;
-  return false;
+__device__ __forceinline__ void store_if(bool ok, void* p, bf16 x) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t@p st.shared.b16 [%1], %2;\n\t}" ::"r"((int)ok),
+               "r"(smem_u32(p)), "h"(__bfloat16_as_ushort(x))
+               : "memory");
 }
 
 template <int ACT>
@@ -202,8 +194,8 @@ __device__ __forceinline__ float g1f(float a) {
 // all the sample's lanes with the same value).
 template <int ACT, bool LP>
 __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf16* Wr, const float* Zs,
-                                      const float* LG, const int* TC, uint32_t* SB, float* HH, unsigned char* Hr,
-                                      int s_me, int q, int klo, int R, int steps, float& lp) {
+                                      float* LG, const int* TC, uint32_t* SB, float* HH, unsigned char* Hr,
+                                      int s_me, int q, int klo, int R, int steps) {
   float* hh = HH + s_me * kLdP;
   float P[kRmax];
 #pragma unroll
@@ -211,7 +203,7 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
   static_assert(kLanes == 8 && kRmax == 32, "hh is zeroed as one float4 per lane");
   reinterpret_cast<float4*>(hh)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncwarp();
-  uint32_t w0 = 0, w1 = 0, w2 = 0, w3 = 0;  // this lane's drawn spins: bit e % 32 of word e / 32
+  uint32_t bits = 0;  // this lane's drawn spins: bit i for step 8 i + q
   // The segments run in four phases by r / 8 (a template parameter PH of the
   // helpers below): in segment r only units 0 .. r-1 are complete (g1 != 0
   // in hh) and only units r .. 31 still need partial sums, so the logit's dot
@@ -261,13 +253,8 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
   // draw of step e from its logit, and the spin into this lane's partial sums
   auto draw = [&](auto ph, int e, float z) {
     const bool up = z > LG[e * kS + s_me];  // u < sigma(z)
-    const uint32_t m = up ? 1u << (e & 31) : 0u;
-    const int wd = e >> 5;
-    w0 |= wd == 0 ? m : 0u;
-    w1 |= wd == 1 ? m : 0u;
-    w2 |= wd == 2 ? m : 0u;
-    w3 |= wd == 3 ? m : 0u;
-    if constexpr (LP) lp += log_sigmoid(up ? z : -z);
+    bits |= (uint32_t)up << (e / kLanes);
+    if constexpr (LP) LG[e * kS + s_me] = up ? z : -z;
     wrow(ph, e, up ? 1.0f : -1.0f);
   };
   // the partial sum of unit k among this lane's units 8 PH .. 8 PH + 15
@@ -307,13 +294,13 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
   float g_last = 0.0f;  // g1 of the unit that completed last
   int lo = 0;
   int e = q;
-  int hi = R > 0 ? TC[0] : steps - 1;  // last step of the current segment
+  int hi = R > 0 ? uniform(TC[0]) : steps - 1;  // last step of the current segment
   float zp = 0.0f, vn = 0.0f, lgn = 0.0f, wn = 0.0f, xr = 0.0f;
   if (e <= hi) zp = zdot(Ph0{}, e), lgn = LG[e * kS + s_me], wn = wt(e, 0);
   xr = extract(Ph0{}, 0);
   // segment r: steps [lo, hi], units 0 .. r-1 complete; true after the last (r = R)
   auto segment = [&](auto ph, int r) -> bool {
-    const int nhi = r + 1 < R ? TC[r + 1] : steps - 1;  // last step of segment r + 1
+    const int nhi = r + 1 < R ? uniform(TC[r + 1]) : steps - 1;  // last step of segment r + 1
     hh[r > 0 ? r - 1 : 0] = g_last;                     // (unit 0's entry is still zero at r = 0)
     float x;
     if (hi - lo + 1 <= kLanes) {
@@ -324,17 +311,13 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
       const bool up = z > lgn;
       const float sv = own ? (up ? 1.0f : -1.0f) : 0.0f;
       x = allsum(fmaf(wn, sv, xr));
-      const uint32_t m = (own && up) ? 1u << (e & 31) : 0u;
-      const int wd = e >> 5;
-      w0 |= wd == 0 ? m : 0u;
-      w1 |= wd == 1 ? m : 0u;
-      w2 |= wd == 2 ? m : 0u;
-      w3 |= wd == 3 ? m : 0u;
-      if constexpr (LP) lp += own ? log_sigmoid(up ? z : -z) : 0.0f;
+      bits |= (uint32_t)(own && up) << ((uint32_t)e / kLanes);
+      if constexpr (LP) store_if(own, LG + el * kS + s_me, up ? z : -z);
       wrow(ph, el, sv);
     } else {
       // ---- a long segment: every step of the lane with its full logit,
       // then unit r's partial sums
+#pragma unroll 1
       for (int ee = lo + ((q - lo) & (kLanes - 1)); ee <= hi; ee += kLanes) draw(ph, ee, zdot(ph, ee));
       x = allsum(extract(ph, r < kRmax ? r : kRmax - 1));
     }
@@ -358,19 +341,27 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
   };
   bool last = false;
   int r = 0;
+#pragma unroll 1
   for (; r < 8 && !last; ++r) last = segment(Ph0{}, r);
+#pragma unroll 1
   for (; r < 16 && !last; ++r) last = segment(std::integral_constant<int, 1>{}, r);
+#pragma unroll 1
   for (; r < 24 && !last; ++r) last = segment(std::integral_constant<int, 2>{}, r);
+#pragma unroll 1
   for (; !last; ++r) last = segment(std::integral_constant<int, 3>{}, r);  // r <= R <= 32
-  // the sample's spins: its lanes' words combined; lane q < 4 stores word q
+  // the sample's spins: step e is bit e % 32 of word e / 32 = bit 8 (i % 4) + q
+  // of word i / 4, i = e / 8.  The lanes' bits are combined with shuffles;
+  // lane q < 4 stores word q.
+  static_assert(kLanes == 8 && kDmax == 128, "four words of four groups of 8 steps");
+  uint32_t wd[kDmax / 32];
 #pragma unroll
-  for (int d = 1; d < kLanes; d <<= 1) {
-    w0 |= __shfl_xor_sync(0xffffffffu, w0, d);
-    w1 |= __shfl_xor_sync(0xffffffffu, w1, d);
-    w2 |= __shfl_xor_sync(0xffffffffu, w2, d);
-    w3 |= __shfl_xor_sync(0xffffffffu, w3, d);
+  for (int t = 0; t < kDmax / 32; ++t) {
+    const uint32_t x = bits >> (4 * t);
+    wd[t] = ((x & 1u) | (x & 2u) << 7 | (x & 4u) << 14 | (x & 8u) << 21) << q;
+#pragma unroll
+    for (int d = 1; d < kLanes; d <<= 1) wd[t] |= __shfl_xor_sync(0xffffffffu, wd[t], d);
   }
-  if (q < kDmax / 32) SB[s_me * (kDmax / 32) + q] = q == 0 ? w0 : q == 1 ? w1 : q == 2 ? w2 : w3;
+  if (q < kDmax / 32) SB[s_me * (kDmax / 32) + q] = q == 0 ? wd[0] : q == 1 ? wd[1] : q == 2 ? wd[2] : wd[3];
   // every recent unit is complete: its g1 goes to the staging operand Hr
   // (2 chunks of 64 units from chunk klo / 64), once warps 2-3 have moved
   // the previous block's recent g1 out of it
@@ -378,11 +369,8 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
 #pragma unroll
   for (int j = 0; j < kRmax / kLanes; ++j) {
     const int r = q + kLanes * j;
-    if (r < R) {
-      const int k = klo + r;
-      *reinterpret_cast<bf16*>(Hr + ((k >> 6) - (klo >> 6)) * 2048 + sw128_offset(s_me, k & 63)) =
-          __float2bfloat16_rn(hh[r]);
-    }
+    const int k = klo + r;
+    store_if(r < R, Hr + ((k >> 6) - (klo >> 6)) * 2048 + sw128_offset(s_me, k & 63), __float2bfloat16_rn(hh[r]));
   }
 }
 
@@ -413,6 +401,16 @@ __device__ __forceinline__ Blk blk_of(int b, int n, int h, int D, int ntiles, in
   return r;
 }
 
+// The four phases of the weight tiles in a block: [i0, i1) of phase p.  Update
+// phases count tiles as unit tile * nkd + K-chunk (nkd = D / 64 is 1 or 2: a
+// shift by nkd - 1 divides by it, a mask of nkd - 1 gives the chunk).
+constexpr int kPhCrit = 0, kPhCor = 1, kPhBulk = 2, kPhZ = 3;
+__device__ __forceinline__ void phase_range(const Blk& B, int p, int nkd, int ntiles, int& i0, int& i1) {
+  i0 = p == kPhCrit ? B.crit0 * nkd : p == kPhCor ? B.cor0 : p == kPhBulk ? B.bulk0 * nkd : 0;
+  i1 = p == kPhCrit ? B.crit1 * nkd : p == kPhCor ? B.cor1 : p == kPhBulk ? ntiles * nkd : B.np;
+}
+
+template <int ACT, bool LP>
 __global__ void __launch_bounds__(kThreads, 1)
     sampler_tc_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapW,
                       const __grid_constant__ CUtensorMap mapV2, const __grid_constant__ CUtensorMap mapV3,
@@ -443,7 +441,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int n = g.n, h = g.h, D = g.D;
   const int nblk = (n + D - 1) / D;
   const int ntiles = (g.hp + 127) / 128;
@@ -471,9 +469,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = (uint32_t)uniform((int)*tmem_slot);
   // A = b1 for every sample
   if (warp < 4) {
+#pragma unroll 1
     for (int t = 0; t < ntiles; ++t) {
       const int k = 128 * t + 32 * warp + lane;
       const float x = k < h ? g.b1[k] : 0.0f;
@@ -494,52 +493,51 @@ __global__ void __launch_bounds__(kThreads, 1)
     // recent units (W2, block b's rows), the remaining update tiles, then the
     // Z GEMM of block b+1 over the units complete before block b (W2, block
     // b+1's rows).
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;  // slots issued
-      // the tiles [i0, i1) of one phase, kSlotTiles per slot; yc(i, y, c)
-      // gives tile i's first row and 64-column chunk.  A run of tiles with
-      // the same rows and consecutive chunks (at most `most`) is one copy
-      // through the chunked map of its length (m2: 2, m3: 3).
-      auto load_phase = [&](const CUtensorMap* m1, const CUtensorMap* m2, const CUtensorMap* m3, int most, int i0,
-                            int i1, auto yc) -> bool {
-        for (int i = i0; i < i1; i += kSlotTiles) {
-          const int cnt = min(kSlotTiles, i1 - i);
-          const int s = it % kNSlot;
-          if (it >= kNSlot &&
-              !test_or_abort(smem_u32(&empty[s]), (uint32_t)((it / kNSlot - 1) & 1), abort, g.err))
-            return false;
-          const uint32_t bar = smem_u32(&full[s]);
-          mbar_expect_tx(bar, (uint32_t)(cnt * kTileBytes));
-          for (int j = 0; j < cnt;) {
-            int y, c;
-            yc(i + j, y, c);
-            int run = 1;
-            while (j + run < cnt && run < most) {
-              int y2, c2;
-              yc(i + j + run, y2, c2);
-              if (y2 != y || c2 != c + run) break;
-              ++run;
-            }
-            const uint32_t dst = base + kOffRing + (s * kSlotTiles + j) * kTileBytes;
-            if (run == 1) tma_load_2d(dst, m1, 64 * c, y, bar);
-            else tma_load_3d(dst, run == 2 ? m2 : m3, 0, y, c, bar);
-            j += run;
-          }
-          ++it;
-        }
-        return true;
-      };
       bool ok = true;
+#pragma unroll 1
       for (int b = 0; b < nblk && ok; ++b) {
         const Blk B = blk_of(b, n, h, D, ntiles, nblk);
-        // update tiles: index q -> unit tile q / nkd, K-chunk q % nkd of block b-1's inputs
-        auto upd = [&](int q, int& y, int& c) { y = 128 * (q / nkd), c = (b - 1) * (D / 64) + q % nkd; };
-        ok = load_phase(&mapW, &mapW2, &mapW2, 2, B.crit0 * nkd, B.crit1 * nkd, upd);
-        if (ok)
-          ok = load_phase(&mapV, &mapV2, &mapV3, 3, B.cor0, B.cor1, [&](int c, int& y, int& cc) { y = b * D, cc = c; });
-        if (ok) ok = load_phase(&mapW, &mapW2, &mapW2, 2, B.bulk0 * nkd, ntiles * nkd, upd);
-        if (ok)
-          ok = load_phase(&mapV, &mapV2, &mapV3, 3, 0, B.np, [&](int c, int& y, int& cc) { y = (b + 1) * D, cc = c; });
+#pragma unroll 1
+        for (int p = 0; p < 4 && ok; ++p) {
+          // the tiles [i0, i1) of phase p, kSlotTiles per slot.  An update
+          // phase's index i is unit tile i / nkd, K-chunk i % nkd of block
+          // b-1's inputs; a Z phase's is the 64-unit chunk.  A run of tiles
+          // with the same rows and consecutive chunks (at most `most`) is one
+          // copy through the chunked map of its length.
+          const bool upd = p == kPhCrit || p == kPhBulk;
+          int i0, i1;
+          phase_range(B, p, nkd, ntiles, i0, i1);
+          const CUtensorMap* m1 = upd ? &mapW : &mapV;
+          const CUtensorMap* m2 = upd ? &mapW2 : &mapV2;
+          const int most = upd ? 2 : 3;
+          const int sh = upd ? nkd - 1 : 31, msk = upd ? nkd - 1 : -1;
+          const int y0 = upd ? 0 : (p == kPhZ ? b + 1 : b) * D, c0 = upd ? (b - 1) * nkd : 0;
+#pragma unroll 1
+          for (int i = i0; i < i1; i += kSlotTiles) {
+            const int cnt = min(kSlotTiles, i1 - i);
+            const int s = it % kNSlot;
+            if (it >= kNSlot &&
+                !test_or_abort(smem_u32(&empty[s]), (uint32_t)((it / kNSlot - 1) & 1), abort, g.err)) {
+              ok = false;
+              break;
+            }
+            const uint32_t bar = smem_u32(&full[s]);
+            mbar_expect_tx(bar, (uint32_t)(cnt * kTileBytes));
+#pragma unroll 1
+            for (int j = 0; j < cnt;) {
+              const int t = (i + j) >> sh, k = (i + j) & msk;
+              // chunks that follow in the same rows: all of a Z phase's, up to the last of an update tile's
+              const int run = min(min(most, cnt - j), upd ? nkd - k : kSlotTiles);
+              const uint32_t dst = base + kOffRing + (s * kSlotTiles + j) * kTileBytes;
+              if (run == 1) tma_load_2d(dst, m1, 64 * (c0 + k), y0 + 128 * t, bar);
+              else tma_load_3d(dst, run == 2 ? m2 : &mapV3, 0, y0 + 128 * t, c0 + k, bar);
+              j += run;
+            }
+            ++it;
+          }
+        }
       }
       // no copy may still be landing when the CTA exits (after a failure
       // some loaded tiles are never consumed)
@@ -553,64 +551,62 @@ __global__ void __launch_bounds__(kThreads, 1)
     // block b (commit -> zfull); then, while block b's solver runs, the rest
     // of the update and, once block b-1's recent g1 are in the operand, the Z
     // GEMM of block b+1 into the other Z buffer.
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;  // slots consumed
       bool ok = true, any = false;
-      // the tiles [i0, i1) of one phase in the producer's slots; op(i, dcol,
-      // bop, acc) gives tile i's accumulator column, B operand and whether it
-      // accumulates.  Each 128 x 64 weight tile against a 16 x 64 operand is
-      // 4 MMAs of K = 16; one commit releases the slot.
-      auto mma_phase = [&](int i0, int i1, auto op) -> bool {
-        for (int i = i0; i < i1; i += kSlotTiles) {
-          const int cnt = min(kSlotTiles, i1 - i);
-          const int s = it % kNSlot;
-          if (!test_or_abort(smem_u32(&full[s]), (uint32_t)((it / kNSlot) & 1), abort, g.err)) return false;
-          fence_after();
-          for (int j = 0; j < cnt; ++j) {
-            uint32_t dcol, bop;
-            bool acc;
-            op(i + j, dcol, bop, acc);
-            const uint64_t da = smem_desc_sw128(base + kOffRing + (s * kSlotTiles + j) * kTileBytes);
-            const uint64_t db = smem_desc_sw128(bop);
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              mma_bf16(tmem + dcol, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc,
-                       (acc || k > 0) ? 1u : 0u);
-          }
-          mma_commit(smem_u32(&empty[s]));
-          ++it;
-          any = true;
-        }
-        return true;
-      };
+#pragma unroll 1
       for (int b = 0; b < nblk; ++b) {
         const Blk B = blk_of(b, n, h, D, ntiles, nblk);
-        const uint32_t s_prev = base + kOffS + ((b - 1) & 1) * (kDmax / 64) * 2048;
         if (b > 0 && ok) {
           ok = test_or_abort(smem_u32(ready), (uint32_t)((b - 1) & 1), abort, g.err);
           fence_after();
         }
-        // update tiles: index q -> accumulator of unit tile q / nkd, K-chunk q % nkd of block b-1's spins
-        auto upd = [&](int q, uint32_t& dcol, uint32_t& bop, bool& acc) {
-          dcol = (uint32_t)(16 * (q / nkd)), bop = s_prev + (q % nkd) * 2048, acc = true;
-        };
-        if (ok) ok = mma_phase(B.crit0 * nkd, B.crit1 * nkd, upd);
-        const uint32_t zcol = kZCol + 16 * (b & 1);
-        if (ok)
-          ok = mma_phase(B.cor0, B.cor1, [&](int c, uint32_t& dcol, uint32_t& bop, bool& acc) {
-            dcol = zcol, bop = base + kOffHr + (c - B.cor0) * 2048, acc = B.zinit || c > B.cor0;
-          });
-        if (ok && any) mma_commit(smem_u32(zfull));  // also covers the previous block's work
-        else mbar_arrive(smem_u32(zfull));
-        if (ok) ok = mma_phase(B.bulk0 * nkd, ntiles * nkd, upd);
-        if (B.np > 0 && ok) {
-          ok = test_or_abort(smem_u32(merged), (uint32_t)(b & 1), abort, g.err);
-          fence_after();
-          const uint32_t zn = kZCol + 16 * ((b + 1) & 1);
-          if (ok)
-            ok = mma_phase(0, B.np, [&](int c, uint32_t& dcol, uint32_t& bop, bool& acc) {
-              dcol = zn, bop = base + kOffH + c * 2048, acc = c > 0;
-            });
+#pragma unroll 1
+        for (int p = 0; p < 4; ++p) {
+          // the tiles [i0, i1) of phase p in the producer's slots: accumulator
+          // column, B operand and first chunk's accumulation.  Each 128 x 64
+          // weight tile against a 16 x 64 operand is 4 MMAs of K = 16; one
+          // commit releases the slot.
+          const bool upd = p == kPhCrit || p == kPhBulk;
+          int i0, i1;
+          phase_range(B, p, nkd, ntiles, i0, i1);
+          const int sh = upd ? nkd - 1 : 31, msk = upd ? nkd - 1 : -1;
+          const uint32_t dcol = tmem + (uint32_t)(upd ? 0 : kZCol + 16 * ((p == kPhZ ? b + 1 : b) & 1));
+          const uint32_t bop = base + (uint32_t)(upd ? kOffS + ((b - 1) & 1) * (kDmax / 64) * 2048
+                                                     : p == kPhZ ? kOffH : kOffHr - 2048 * i0);
+          const bool acc0 = upd || (p == kPhCor && B.zinit);
+          if (p == kPhZ && B.np > 0 && ok) {
+            ok = test_or_abort(smem_u32(merged), (uint32_t)(b & 1), abort, g.err);
+            fence_after();
+          }
+#pragma unroll 1
+          for (int i = i0; i < i1 && ok; i += kSlotTiles) {
+            const int cnt = min(kSlotTiles, i1 - i);
+            const int s = it % kNSlot;
+            if (!test_or_abort(smem_u32(&full[s]), (uint32_t)((it / kNSlot) & 1), abort, g.err)) {
+              ok = false;
+              break;
+            }
+            fence_after();
+#pragma unroll
+            for (int j = 0; j < kSlotTiles; ++j) {
+              if (j >= cnt) break;
+              const uint32_t dc = dcol + (uint32_t)(16 * ((i + j) >> sh));
+              const uint64_t da = smem_desc_sw128(base + kOffRing + (s * kSlotTiles + j) * kTileBytes);
+              const uint64_t db = smem_desc_sw128(bop + (uint32_t)(((i + j) & msk) * 2048));
+              const uint32_t acc = (acc0 || i + j > i0) ? 1u : 0u;
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                mma_bf16(dc, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc, k > 0 ? 1u : acc);
+            }
+            mma_commit(smem_u32(&empty[s]));
+            ++it;
+            any = true;
+          }
+          if (p == kPhCor) {
+            if (ok && any) mma_commit(smem_u32(zfull));  // also covers the previous block's work
+            else mbar_arrive(smem_u32(zfull));
+          }
         }
       }
       // every MMA has completed before tensor memory is released
@@ -628,26 +624,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int sid = (warp <= 1 ? warp : warp - 4) * 32 + lane;  // solver thread
     const int ht = tid - 64;                                      // helper thread (warps 2-3)
     const int s_me = sid / kLanes, sub = sid % kLanes;
-    float lp = 0.0f;
+    float lp = 0.0f, bias = 0.0f;
     const uint32_t tq = tmem + ((uint32_t)(32 * warp) << 16);
     // logit(u) of block b's steps into LG buffer b & 1; threads t0, t0 + nt, ...
     auto logits = [&](int b, int t0, int nt) {
       float* L = LG + (b & 1) * kDrows * kS;
+#pragma unroll 1
       for (int q = t0; q < kS * (D / 4); q += nt) {
         const int s = q % kS, t = b * D + 4 * (q / kS);
         const int bb = b0 + s;
         float* dst = L + (size_t)(4 * (q / kS)) * kS + s;
+        float x[4];
         if (g.u) {
 #pragma unroll
-          for (int w = 0; w < 4; ++w)
-            dst[w * kS] = (bb < g.B && t + w < n) ? logit(__ldg(g.u + (size_t)bb * n + t + w)) : 0.0f;
+          for (int w = 0; w < 4; ++w) x[w] = (bb < g.B && t + w < n) ? __ldg(g.u + (size_t)bb * n + t + w) : 0.5f;
         } else {
           const uint4 r = philox4x32_10(make_uint4((uint32_t)(t >> 2), (uint32_t)bb + g.boff, it0, it1), g.key0, g.key1);
-          dst[0] = logit(to_unit(r.x));
-          dst[kS] = logit(to_unit(r.y));
-          dst[2 * kS] = logit(to_unit(r.z));
-          dst[3 * kS] = logit(to_unit(r.w));
+          x[0] = to_unit(r.x), x[1] = to_unit(r.y), x[2] = to_unit(r.z), x[3] = to_unit(r.w);
         }
+#pragma unroll
+        for (int w = 0; w < 4; ++w) dst[w * kS] = logit(x[w]);
       }
     };
     // spins of block b (bits in SB buffer b & 1) to the outputs; threads t0,
@@ -660,6 +656,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bf16 one = __float2bfloat16_rn(1.0f), mone = __float2bfloat16_rn(-1.0f);
       // two spins as BF16 (+1 = 0x3F80, -1 = 0xBF80); bit set in dn: spin -1
       auto bf_pair = [](uint32_t dn) { return 0x3F803F80u | (dn & 1u) << 15 | (dn >> 1 & 1u) << 31; };
+#pragma unroll 1
       for (int q = t0; q < kS * (kDmax / 16); q += nt) {
         const int s = q / (kDmax / 16), e0 = 16 * (q % (kDmax / 16));
         const int bb = b0 + s;
@@ -678,6 +675,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           *reinterpret_cast<uint4*>(so) = make_uint4(w[0], w[1], w[2], w[3]);
         } else {
+#pragma unroll 1
           for (int k = 0; k < cnt; ++k) so[k] = (up >> k) & 1u ? (int8_t)1 : (int8_t)-1;
         }
         if (g.sx) {
@@ -688,6 +686,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             d4[0] = make_uint4(bf_pair(dn), bf_pair(dn >> 2), bf_pair(dn >> 4), bf_pair(dn >> 6));
             d4[1] = make_uint4(bf_pair(dn >> 8), bf_pair(dn >> 10), bf_pair(dn >> 12), bf_pair(dn >> 14));
           } else {
+#pragma unroll 1
             for (int k = 0; k < cnt; ++k) dx[k] = (up >> k) & 1u ? one : mone;
           }
         }
@@ -697,7 +696,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       // collects step j's spins) and lane j keeps step j's column
       const uint32_t valid = b0 + kS <= g.B ? 0xFFFFu : (1u << (g.B - b0)) - 1u;  // samples inside B
       if (g.stt || g.sbits)
-        for (int w = t0 >> 5; w < (steps + 31) / 32; w += nt >> 5) {
+#pragma unroll 1
+        for (int w = uniform(t0 >> 5); w < (steps + 31) / 32; w += nt >> 5) {
           const int ln = t0 & 31;
           const uint32_t word = ln < kS ? sb[ln * (kDmax / 32) + w] : 0u;
           uint32_t up = 0;
@@ -716,6 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               d4[0] = make_uint4(bf_pair(dn), bf_pair(dn >> 2), bf_pair(dn >> 4), bf_pair(dn >> 6));
               d4[1] = make_uint4(bf_pair(dn >> 8), bf_pair(dn >> 10), bf_pair(dn >> 12), bf_pair(dn >> 14));
             } else {
+#pragma unroll 1
               for (int s = 0; s < kS; ++s)
                 if (b0 + s < g.B) dt[s] = (dn >> s) & 1u ? mone : one;
             }
@@ -789,22 +790,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     };
-    if (warp < 4) logits(0, tid, 128);
-    if (warp == 2 || warp == 3) {
-      gather_load(0, ht);
-      gather_store(0, ht);
-    }
-    for (int b = 0; b < nblk; ++b) {
-      const Blk B = blk_of(b, n, h, D, ntiles, nblk);
-      const int klo = B.klo, khi = B.khi;
-      const int R = khi - klo;  // <= kRmax (checked by the host)
+    // Turn b: the solver draws block b; warps 2-3 prepare block b + 1 and write
+    // out block b - 1 (so there is one turn before the first block and one
+    // after the last).
+#pragma unroll 1
+    for (int b = -1; b <= nblk; ++b) {
+      const bool draws = b >= 0 && b < nblk;
+      const int* cu = CU + (b & 1) * kBlkInts;
+      const int klo = uniform(cu[kRmax]), R = uniform(cu[kRmax + 1]), zvalid = uniform(cu[kRmax + 2]);
       const int steps = min(D, n - b * D);
-      if (warp < 4) {
-      // (a) the recent units' completion steps (their weights are in Vr / Wr)
-      for (int q = tid; q < (kRmax - R) * kS; q += 128) Pr[R * kS + q] = 0.0f;
-      // TC[r] = the block step whose spin is recent unit r's last input
-      for (int r = tid; r < kRmax; r += 128) CU[r] = r < R ? degree(klo + r, n, h) - 1 - b * D : D;
-      // (b) Z and the recent pre-activations from tensor memory
+      if (warp < 4 && draws) {
+      // Z and the recent pre-activations from tensor memory
       wait_or_abort(smem_u32(zfull), (uint32_t)(b & 1), abort, g.err);
       __syncwarp();
       fence_after();
@@ -812,7 +808,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool live = !__any_sync(0xffffffffu, *abort != 0);
       {
         float v[16];
-        if (B.zvalid && live) {
+        if (zvalid && live) {
           tmem_ld16(tq + kZCol + 16 * (b & 1), v);
         } else {
 #pragma unroll
@@ -820,41 +816,38 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         const int e = 32 * warp + lane;
         if (e < D) {
-          const float c = e < steps ? __ldg(g.b2 + b * D + e) : 0.0f;
 #pragma unroll
-          for (int q = 0; q < 16; ++q) Zs[e * kZld + q] = v[q] + c;  // b2 folded in
+          for (int q = 0; q < 16; ++q) Zs[e * kZld + q] = v[q] + bias;  // b2 folded in
         }
       }
       if (R > 0 && live) {
-        for (int t = klo / 128; t <= (khi - 1) / 128; ++t) {
+#pragma unroll 1
+        for (int t = klo / 128; t <= (klo + R - 1) / 128; ++t) {
           float v[16];
           tmem_ld16(tq + (uint32_t)(16 * t), v);
           const int k = 128 * t + 32 * warp + lane;
-          if (k >= klo && k < khi) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) Pr[(k - klo) * kS + q] = v[q];
-          }
+          for (int q = 0; q < 16; ++q) store_if(k >= klo && k < klo + R, Pr + (k - klo) * kS + q, v[q]);
         }
       }
       fence_before();  // the tensor-memory reads precede the next MMAs into Z (after merged)
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(kBar1Threads) : "memory");
+      if (draws) asm volatile("bar.sync 1, %0;" ::"n"(kBar1Threads) : "memory");
+      {  // b2 of the next block's step, ahead of its use
+        const int i = (b + 1) * D + 32 * warp + lane;
+        bias = warp < 4 && 32 * warp + lane < D && i < n ? __ldg(g.b2 + i) : 0.0f;
+      }
       // (c) the D draws of the block (the solver warps), then the block's
       // spins as the update GEMM's operand; warps 2-3 meanwhile
       if (solver) {
-        const bool relu = g.act == VQMC_ACT_RELU;
-        const float* L = LG + (b & 1) * kDrows * kS;
         uint32_t* sb = SB + (b & 1) * kS * (kDmax / 32);
-        if (g.logp) {
-          if (relu) solve<VQMC_ACT_RELU, true>(Pr, Vr, Wr, Zs, L, CU, sb, PreS, Hr, s_me, sub, klo, R, steps, lp);
-          else solve<VQMC_ACT_SIGMOID, true>(Pr, Vr, Wr, Zs, L, CU, sb, PreS, Hr, s_me, sub, klo, R, steps, lp);
-        } else {
-          if (relu) solve<VQMC_ACT_RELU, false>(Pr, Vr, Wr, Zs, L, CU, sb, PreS, Hr, s_me, sub, klo, R, steps, lp);
-          else solve<VQMC_ACT_SIGMOID, false>(Pr, Vr, Wr, Zs, L, CU, sb, PreS, Hr, s_me, sub, klo, R, steps, lp);
-        }
+        if (draws)
+          solve<ACT, LP>(Pr, Vr, Wr, Zs, LG + (b & 1) * kDrows * kS, cu, sb, PreS, Hr, s_me, sub, klo, R, steps);
         asm volatile("bar.sync 1, %0;" ::"n"(kBar1Threads) : "memory");
+        if (!draws) continue;
         // (d) 8 spins of one sample per 16-byte store (+1 = 0x3F80, -1 = 0xBF80)
         unsigned char* ss = Ss + (b & 1) * (kDmax / 64) * 2048;
+#pragma unroll 1
         for (int q = sid; q < kS * (D / 8); q += kSolverThreads) {
           const int s = q / (D / 8), e = 8 * (q % (D / 8));
           const uint32_t bits = ~(sb[s * (kDmax / 32) + (e >> 5)] >> (e & 31));  // bit set: spin -1
@@ -871,34 +864,69 @@ __global__ void __launch_bounds__(kThreads, 1)
         // block b-1's recent g1 from the staging operand into the GEMM
         // operand (the block's Z GEMM has read Hr: zfull), then release Hr
         // to the solver and the operand to the next Z GEMM
-        if (b > 0) {
-          const int kprev = count_deg_le((b - 1) * D, n, h), cb = kprev >> 6;
-          for (int q = ht; q < (klo - kprev) * kS; q += 64) {
-            const int k = kprev + q / kS, s = q % kS;
-            const uint32_t o = sw128_offset(s, k & 63);
-            bf16* src = reinterpret_cast<bf16*>(Hr + ((k >> 6) - cb) * 2048 + o);
-            *reinterpret_cast<bf16*>(Hs + (k >> 6) * 2048 + o) = *src;
-            *src = __float2bfloat16_rn(0.0f);  // Hr is zero outside the current recent units
+        if (draws) {
+          if (b > 0) {
+            const int kprev = count_deg_le((b - 1) * D, n, h), cb = kprev >> 6;
+#pragma unroll 1
+            for (int q = ht; q < (klo - kprev) * kS; q += 64) {
+              const int k = kprev + q / kS, s = q % kS;
+              const uint32_t o = sw128_offset(s, k & 63);
+              bf16* src = reinterpret_cast<bf16*>(Hr + ((k >> 6) - cb) * 2048 + o);
+              *reinterpret_cast<bf16*>(Hs + (k >> 6) * 2048 + o) = *src;
+              *src = __float2bfloat16_rn(0.0f);  // Hr is zero outside the current recent units
+            }
+          }
+          fence_proxy_async();
+          fence_before();
+          mbar_arrive(smem_u32(merged));
+          asm volatile("bar.arrive 2, %0;" ::"n"(kBar2Threads) : "memory");
+        }
+        if (LP && b > 0) {
+          // log pi of block b - 1: the solver left +-z in place of the logits
+          // of u.  The entries that a thread reads are those that it fills
+          // next for block b + 1.
+          const float* L = LG + ((b - 1) & 1) * kDrows * kS;
+#pragma unroll 1
+          for (int q = ht; q < kS * (D / 4); q += 64) {
+            const int e = 4 * (q / kS), left = n - (b - 1) * D - e;
+            // sum of log sigma(x) = min(x, 0) - log(1 + exp(-|x|)): one
+            // logarithm of the four factors, kept as their product minus 1
+            // (0 for steps past the last, x = 1e30)
+            float lin = 0.0f, prod1 = 0.0f;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              const float x = w < left ? L[(e + w) * kS + q % kS] : 1e30f;
+              lin += fminf(x, 0.0f);
+              prod1 = fmaf(expf(-fabsf(x)), 1.0f + prod1, prod1);
+            }
+            lp += lin - log1pf(prod1);
           }
         }
-        fence_proxy_async();
-        fence_before();
-        mbar_arrive(smem_u32(merged));
-        asm volatile("bar.arrive 2, %0;" ::"n"(kBar2Threads) : "memory");
-        if (b + 1 < nblk) logits(b + 1, ht, 64);
+        if (b + 1 < nblk) {
+          // block b + 1's schedule, out of the way of its solver: TC[r], the
+          // step whose spin is recent unit r's last input, and klo, R, zvalid
+          if (warp == 2) {
+            const Blk N = blk_of(b + 1, n, h, D, ntiles, nblk);
+            int* cn = CU + ((b + 1) & 1) * kBlkInts;
+            const int Rn = N.khi - N.klo;  // <= kRmax (checked by the host)
+            cn[lane] = lane < Rn ? degree(N.klo + lane, n, h) - 1 - (b + 1) * D : D;
+            const int x = lane == 0 ? N.klo : lane == 1 ? Rn : (int)N.zvalid;
+            if (lane < 3) cn[kRmax + lane] = x;
+          }
+          logits(b + 1, ht, 64);
+          gather_load(b + 1, ht);
+        }
         if (b > 0) write_spins(b - 1, ht, 64);
-        if (b + 1 < nblk) gather_load(b + 1, ht);
         asm volatile("bar.sync 1, %0;" ::"n"(kBar1Threads) : "memory");
         if (b + 1 < nblk) gather_store(b + 1, ht);
       }
     }
-    asm volatile("bar.sync 1, %0;" ::"n"(kBar1Threads) : "memory");
-    if (warp < 4) write_spins(nblk - 1, tid, 128);
-    if (solver) {  // the partial sums of log pi of the sample's lanes
-#pragma unroll
-      for (int d = 1; d < kLanes; d <<= 1) lp += __shfl_xor_sync(0xffffffffu, lp, d);
+    if (LP && !solver) {  // the partial sums of log pi of each sample's four threads
+      lp += __shfl_xor_sync(0xffffffffu, lp, 16);
+      if (warp == 3 && lane < kS) LG[lane] = lp;
+      asm volatile("bar.sync 2, 64;" ::: "memory");
+      if (warp == 2 && lane < kS && b0 + lane < g.B && !*abort) g.logp[b0 + lane] = lp + LG[lane];
     }
-    if (solver && sub == 0 && g.logp && b0 + s_me < g.B && !*abort) g.logp[b0 + s_me] = lp;
   }
 
   __syncwarp();
@@ -948,9 +976,16 @@ cudaError_t launch_sampler_tc(const vqmc_ctx* c, int B, const float* d_u, uint64
       !tc_encode_bf16_chunks(&mapV3, c->v_s, sampler_rows(c->n), c->hp, c->hp, 128, 3) ||
       !tc_encode_bf16_chunks(&mapW2, c->w_s, c->h, c->np, c->np, 128, 2))
     return cudaErrorInvalidValue;
+  using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcArgs);
+  constexpr Kernel kernels[2][2] = {
+      {sampler_tc_kernel<VQMC_ACT_RELU, false>, sampler_tc_kernel<VQMC_ACT_RELU, true>},
+      {sampler_tc_kernel<VQMC_ACT_SIGMOID, false>, sampler_tc_kernel<VQMC_ACT_SIGMOID, true>}};
   if (!g_attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(sampler_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
+    for (const auto& row : kernels)
+      for (Kernel k : row) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e != cudaSuccess) return e;
+      }
     g_attr_set = true;
   }
   TcArgs a;
@@ -959,7 +994,6 @@ cudaError_t launch_sampler_tc(const vqmc_ctx* c, int B, const float* d_u, uint64
   a.hp = c->hp;
   a.B = B;
   a.D = D;
-  a.act = c->act;
   a.w = reinterpret_cast<const bf16*>(c->w_s);
   a.np = c->np;
   a.v = reinterpret_cast<const bf16*>(c->v_s);
@@ -980,7 +1014,8 @@ cudaError_t launch_sampler_tc(const vqmc_ctx* c, int B, const float* d_u, uint64
   a.stt = reinterpret_cast<bf16*>(stt);
   a.ldst = c->Bp;
   a.sbits = reinterpret_cast<uint16_t*>(sbits);
-  sampler_tc_kernel<<<(B + kS - 1) / kS, kThreads, kSmemBytes, st>>>(mapV, mapW, mapV2, mapV3, mapW2, a);
+  const Kernel kernel = kernels[c->act == VQMC_ACT_RELU ? 0 : 1][d_logp != nullptr];
+  kernel<<<(B + kS - 1) / kS, kThreads, kSmemBytes, st>>>(mapV, mapW, mapV2, mapV3, mapW2, a);
   return cudaGetLastError();
 }
 

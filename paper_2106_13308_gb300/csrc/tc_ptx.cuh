@@ -12,6 +12,21 @@ namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+// True in one lane of a converged warp.  The issuing threads of tcgen05 and TMA
+// instructions are chosen this way, not by a lane index: the compiler then
+// knows that a single thread runs the branch and issues each instruction once,
+// where for a branch on the lane index it wraps every one in a loop over the
+// lanes that might be active.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -57,6 +72,38 @@ __device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint32_
   for (long long it = 0; it < kSpinLimit; ++it)
     if (mbar_test_wait(bar, parity)) return true;
   if (err) atomicOr(err, kErrTimeout);
+  return false;
+}
+
+// bounded wait that gives up at once after any failure in the CTA; with
+// backoff the polling thread sleeps between tries so that it takes no issue
+// slots from a busy warp on the same sub-partition.
+// test_or_abort is the same wait polling with mbarrier.test_wait, which returns at once: for
+// the MMA issuer's waits on landed tiles, which are usually already complete
+// (a try_wait there costs the issuing thread about 190 cycles even then),
+// and for the single threads of the producer and the MMA issuer on the
+// block hand-offs, where a try_wait's suspension delays the reaction.
+__device__ __forceinline__ bool test_or_abort(uint32_t bar, uint32_t parity, volatile int* abort, uint32_t* err) {
+#pragma unroll 1
+  for (long long it = 0; it < kSpinLimit; ++it) {
+    if (mbar_test_wait(bar, parity)) return true;
+    if ((it & 255) == 255 && *abort) return false;
+  }
+  atomicOr(err, kErrTimeout);
+  *abort = 1;
+  return false;
+}
+__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort, uint32_t* err,
+                                              bool backoff = false) {
+  if (*abort) return false;
+#pragma unroll 1
+  for (long long it = 0; it < kSpinLimit; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 255) == 255 && *abort) return false;
+    if (backoff) __nanosleep(64);
+  }
+  atomicOr(err, kErrTimeout);
+  *abort = 1;
   return false;
 }
 

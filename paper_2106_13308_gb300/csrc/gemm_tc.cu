@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
   float* bias_s = reinterpret_cast<float*>(smem + kOffBias);   // [BN]
   float* rowbuf = reinterpret_cast<float*>(smem + kOffRow);    // [BM]
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int quad = warp & 3, half = warp >> 2;
   constexpr int op = OP;
   constexpr bool kWgrad = op == kOpDV || op == kOpDW;
@@ -298,10 +298,11 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = (uint32_t)uniform((int)*tmem_slot);
   bool ok = true;
 
-  if (warp == 0 && lane == 0) {
+  const bool issuer = warp < 2 && elect_one();
+  if (warp == 0 && issuer) {
     // ---------------------------------------------------------- producer
     for (int it = 0; it < nkt && ok; ++it) {
       const int s = it % NSTAGE;
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && issuer) {
     // --------------------------------------------------------- MMA issuer
     for (int it = 0; it < nkt && ok; ++it) {
       const int s = it % NSTAGE;

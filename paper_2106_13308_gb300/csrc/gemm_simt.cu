@@ -104,6 +104,12 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
   const int m0 = tm * BM, n0 = tn * BN;
   const int m1 = min(m0 + BM, g.M), n1 = min(n0 + BN, g.N);
   constexpr bool wgrad = op == kOpDV || op == kOpDW;
+  // Columns of a thread: 4 tx .. + 3 of each 64, or, where it sums along the
+  // row, 8 tx .. + 7 (eight neighbours summed in order, then a tree over tx: the
+  // energies that enter the gradient keep the sums' order).  The 16-byte pieces
+  // of a B row lie in shared memory in the order in which the threads read them.
+  constexpr bool kRowSum = op == kOpOut || op == kOpEloc;
+  auto column = [&](int q) { return kRowSum ? 8 * tx + 4 * q : 64 * q + 4 * tx; };
   if (wgrad && gemm_tile_masked(op, m0, m1, n0, n1, g.n, g.h)) {
     if (gridDim.z == 1)
       for (int q = tid; q < BM * BN; q += kThreads) {
@@ -145,7 +151,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
       for (int q = 0; q < BK * BN / 4; q += kThreads) {
         const int r = (q + tid) / (BN / 4), c = (q + tid) % (BN / 4) * 4;
         const bool in = k0 + r < khi && n0 + c < g.ldb;  // ldb: N padded to a multiple of 64
-        cp16(dst + 4 * (T::kA + r * BN + c), g.Bm + (in ? (size_t)(k0 + r) * g.ldb + n0 + c : 0), in ? 16 : 0);
+        const int place = kRowSum ? c / 8 * 4 + (c & 4) * 16 : c;
+        cp16(dst + 4 * (T::kA + r * BN + place), g.Bm + (in ? (size_t)(k0 + r) * g.ldb + n0 + c : 0), in ? 16 : 0);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -233,16 +240,9 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
         if (mb + i < g.M) o[i] = x[i];
     }
   };
-  // prod: the logarithms of log sigma(x) = min(x, 0) - log(1 + e), e =
-  // exp(-|x|), are taken of the product of a row's TN factors 1 + e in (1, 2]
-  // (one rounding of 2^-24 each, where each logarithm has an absolute error
-  // of a few 2^-23)
-  float prod[TM];
-#pragma unroll
-  for (int i = 0; i < TM; ++i) prod[i] = 1.0f;
 #pragma unroll
   for (int q = 0; q < TN / 4; ++q) {
-    const int nn = n0 + 64 * q + 4 * tx, valid = g.N - nn;
+    const int nn = n0 + column(q), valid = g.N - nn;
     if (valid <= 0) continue;
     float bias[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if constexpr (op == kOpHidden || op == kOpOut)
@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
           if (g.pre) store4(g.pre + (size_t)m * g.ldpre + nn, a, valid);
           store4(g.out + (size_t)m * g.ldo + nn, x, valid);
         } else if constexpr (op == kOpOut) {
-          // sigma(-x) = (x >= 0 ? e : 1) / (1 + e); hardware exp2 / log2
+          // with e = exp(-|x|): log sigma(x) = min(x, 0) - log(1 + e) and
+          // sigma(-x) = (x >= 0 ? e : 1) / (1 + e), on the hardware exp2 / log2
           // approximations and the approximate division
           float s[4];
           spins4(g.S8 + (size_t)m * g.lds8 + nn, valid, s);
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const float z = s[j] * (acc[i][4 * q + j] + bias[j]), e = __expf(-fabsf(z));
-            if (j < valid) rowsum[i] += fminf(z, 0.0f), prod[i] *= 1.0f + e;
+            if (j < valid) rowsum[i] += fminf(z, 0.0f) - __logf(1.0f + e);
             if (g.coef && j < valid) {
               x[j] = cm * s[j] * __fdividef(z >= 0.0f ? e : 1.0f, 1.0f + e);
               colsum[4 * q + j] += x[j];
@@ -305,9 +306,6 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
 #pragma unroll
         for (int j = 0; j < 4; ++j) store_t(nn + j, t[j]);
   }
-  if constexpr (op == kOpOut)
-#pragma unroll
-    for (int i = 0; i < TM; ++i) rowsum[i] -= __logf(prod[i]);
 
   // row partials: reduce over the 16 tx lanes of each half-warp
   if (g.row_part && (op == kOpOut || op == kOpEloc)) {
@@ -326,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
     __syncthreads();  // the operand stages are consumed
     float(*colbuf)[BN] = reinterpret_cast<float(*)[BN]>(sm);
 #pragma unroll
-    for (int j = 0; j < TN; ++j) colbuf[ty][64 * (j / 4) + 4 * tx + j % 4] = colsum[j];
+    for (int j = 0; j < TN; ++j) colbuf[ty][column(j / 4) + j % 4] = colsum[j];
     __syncthreads();
     if (tid < BN) {
       float v = 0.0f;

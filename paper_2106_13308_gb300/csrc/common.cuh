@@ -151,6 +151,7 @@ struct vqmc_ctx {
   void* tim_H = nullptr;          // [tim_rows][hp] hidden activations of the rows
   float* tim_row_part = nullptr;  // [ceil(n/128)][tim_ld] partial log pi of every row per output tile
   long long tim_ld = 0;           // Bmax (n + 1), rounded up to 4
+  void* tim_part = nullptr;       // tim_tc.cu, in place of the three before: FP64 sums of a block of flips
 
   // workspaces (element type per precision unless noted)
   int8_t* S = nullptr;     // int8 [Bmax][n] samples of vqmc_step
@@ -229,6 +230,12 @@ cudaError_t launch_eloc_dense_finish(const vqmc_ctx* c, int B, const int8_t* d_s
 // (float [B]); *launches (if not null) receives the number of kernels
 cudaError_t launch_tim_offdiag(const vqmc_ctx* c, int B, const int8_t* d_s, float* d_e, cudaStream_t st,
                                int* launches = nullptr);
+// The BF16 model's one-kernel form (tim_tc.cu), after the hidden GEMM: whether
+// it takes a model of hp padded hidden units, its workspace, and the launch
+// (*launches, if not null, grows by its kernels).
+bool tim_tc_applies(int prec, int hp);
+size_t tim_tc_part_bytes(int Bmax, int n);
+cudaError_t launch_tim_tc(const vqmc_ctx* c, int B, const int8_t* d_s, float* d_e, cudaStream_t st, int* launches);
 // rows per chunk of the flipped states for at most Bmax samples (padded
 // sizes hp, np and the activation element size bound its workspace)
 int tim_chunk_rows(int Bmax, int n, int hp, int np, int esize);

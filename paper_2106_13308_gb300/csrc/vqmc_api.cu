@@ -406,13 +406,17 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
     if (cudaMemcpy(c->alpha, inst->alpha, (size_t)n * 4, cudaMemcpyHostToDevice) != cudaSuccess)
       return cleanup_fail(VQMC_ERR_CUDA, "copy of alpha failed");
     hsh = fnv1a(hsh, inst->alpha, (size_t)n * 4);
-    c->tim_rows = tim_chunk_rows(Bmax, n, c->hp, c->np, (int)esize(c));
-    const size_t rows = (size_t)c->tim_rows;
     VQ_ALLOC(c->tim_A, (size_t)Bmax * c->hp * 4);
-    VQ_ALLOC(c->tim_S8, rows * c->np);
-    VQ_ALLOC(c->tim_H, rows * c->hp * esize(c));
-    c->tim_ld = ((long long)Bmax * (n + 1) + 3) / 4 * 4;
-    VQ_ALLOC(c->tim_row_part, (size_t)((n + 127) / 128) * (size_t)c->tim_ld * 4);
+    if (tim_tc_applies(c->prec, c->hp)) {
+      VQ_ALLOC(c->tim_part, tim_tc_part_bytes(Bmax, n));
+    } else {
+      c->tim_rows = tim_chunk_rows(Bmax, n, c->hp, c->np, (int)esize(c));
+      const size_t rows = (size_t)c->tim_rows;
+      VQ_ALLOC(c->tim_S8, rows * c->np);
+      VQ_ALLOC(c->tim_H, rows * c->hp * esize(c));
+      c->tim_ld = ((long long)Bmax * (n + 1) + 3) / 4 * 4;
+      VQ_ALLOC(c->tim_row_part, (size_t)((n + 127) / 128) * (size_t)c->tim_ld * 4);
+    }
   }
   c->inst_hash = hsh;
   if (launch_refresh_weights(c, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
@@ -436,7 +440,7 @@ void vqmc_destroy(vqmc_ctx* c) {
                   c->col, c->w, c->field, c->J, c->J_hi, c->J_lo, c->S, c->E, c->Sx, c->St, c->H, c->Ht,
                   c->D, c->Dt, c->GAt, c->GA, c->logp, c->coef, c->stats, c->row_part, c->col_part, c->err,
                   c->step_stats, c->Sbits, c->eloc_part, c->eloc_slice, c->erow, c->alpha, c->tim_A,
-                  c->tim_S8, c->tim_H, c->tim_row_part, c->sr_A, c->sr_x, c->sr_ones, c->sr_xinv,
+                  c->tim_S8, c->tim_H, c->tim_row_part, c->tim_part, c->sr_A, c->sr_x, c->sr_ones, c->sr_xinv,
                   c->sr_events, c->dstate, c->ones};
   for (void* p : ptrs)
     if (p) cudaFree(p);

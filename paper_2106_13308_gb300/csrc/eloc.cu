@@ -231,103 +231,114 @@ __global__ void eloc_sum_kernel(int B, int nslices, const A* __restrict__ part, 
   E[b] = t;
 }
 
-// E_b = sum over N-tiles of the GEMM's row partials (1/2 s^T J s) + h.s
-__global__ void eloc_dense_finish_kernel(int B, int n, int ntiles, const float* __restrict__ part, int ld,
-                                         const int8_t* __restrict__ S, const float* __restrict__ field,
-                                         float* __restrict__ E) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
+// E_b = sum over N-tiles of the GEMM's row partials (1/2 s^T J s) + h.s, added
+// in the order of the spins.  The chain of n additions bounds it, so nothing
+// else is in it: a CTA takes 32 samples, its warps stage the terms +-h_i of
+// kFinishCols spins in shared memory, and one warp adds the previous ones, a
+// sample per lane.  (One thread per sample reading its spins as it adds took 37
+// us for 1024 samples of 500 spins.)
+constexpr int kFinishCols = 128, kFinishThreads = 288;
+__global__ void __launch_bounds__(kFinishThreads)
+    eloc_dense_finish_kernel(int B, int n, int ntiles, const float* __restrict__ part, int ld,
+                             const int8_t* __restrict__ S, const float* __restrict__ field, float* __restrict__ E) {
+  __shared__ float term[2][32][kFinishCols + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = blockIdx.x * 32 + lane;
   float e = 0.0f;
-  for (int t = 0; t < ntiles; ++t) e += part[(size_t)t * ld + b];
-  if (field) {
-    const int8_t* s = S + (size_t)b * n;
-    for (int i = 0; i < n; ++i) e += s[i] > 0 ? field[i] : -field[i];
+  if (warp == 0 && b < B)
+    for (int t = 0; t < ntiles; ++t) e += part[(size_t)t * ld + b];
+  const int chunks = field ? (n + kFinishCols - 1) / kFinishCols : 0;
+  for (int c = 0; c <= chunks; ++c) {
+    if (warp == 0) {
+      if (c > 0) {
+        const float* x = term[(c - 1) & 1][lane];
+        const int cnt = min(kFinishCols, n - (c - 1) * kFinishCols);
+#pragma unroll 16
+        for (int i = 0; i < cnt; ++i) e += x[i];
+      }
+    } else if (c < chunks) {
+      // warp w: samples 4 (w - 1) .. + 3; lane + 32 q: spins
+#pragma unroll
+      for (int q = 0; q < kFinishCols / 32; ++q) {
+        const int i = c * kFinishCols + 32 * q + lane;
+        const float f = i < n ? field[i] : 0.0f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int s = 4 * (warp - 1) + r, bs = blockIdx.x * 32 + s;
+          if (i < n && bs < B) term[c & 1][s][32 * q + lane] = S[(size_t)bs * n + i] > 0 ? f : -f;
+        }
+      }
+    }
+    __syncthreads();
   }
-  E[b] = e;
+  if (warp == 0 && b < B) E[b] = e;
 }
 
 // FP64 statistics of B energies in one CTA with a fixed reduction order.
-// With ds set, thread 0 also starts the next Adam step (t += 1 and its bias
+// With ds set, one thread also starts the next Adam step (t += 1 and its bias
 // corrections), which the gradient kernels after it read.  Float energies
 // (this kernel); the coefficients (E_b - mean) / B multiply by 1 / B (exact
 // for B a power of two; otherwise within one rounding of the quotient before
 // the conversion to FP32).  Integer energies: stats_int_kernel below.
-template <typename A>
-struct StatAcc;
-template <>
-struct StatAcc<float> {
-  using S = double;
-  using M = double;
-  static __device__ __forceinline__ M lo() { return 1.0 / 0.0; }
-  static __device__ __forceinline__ M hi() { return -1.0 / 0.0; }
-};
-
-template <typename V>
-__device__ __forceinline__ V shfl_down_v(V v, int d) {
-  return __shfl_down_sync(0xffffffffu, v, d);
-}
-
-// Sum, min and max over the CTA (warp shuffles, then one warp over the 32
-// warps' values): the result in every thread.  Fixed order.
-template <typename S, typename M>
-__device__ __forceinline__ void cta_reduce(S& sum, M& mn, M& mx, S* ws, M* wmn, M* wmx) {
+// FP64 runs at 1/64 of the FP32 rate and bounds this kernel, so that only the
+// sums are FP64: the extremes are taken in FP32 and the quotients by one thread
+// (a division is some 30 instructions: computed by every thread, with FP64
+// extremes, 1024 energies took 19 us and 8192 took 41 us).
+__global__ void __launch_bounds__(1024) stats_kernel(int B, const float* __restrict__ E, double* __restrict__ out,
+                                                     float* __restrict__ coef, uint32_t* __restrict__ err,
+                                                     DevState* ds, float beta1, float beta2) {
+  __shared__ double ws[32], quot[2];
+  __shared__ float wmn[32], wmx[32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // sum over the CTA (thread 0 holds it), in a fixed order
+  auto cta_sum = [&](double x) {
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    sum += shfl_down_v(sum, d);
-    const M a = shfl_down_v(mn, d), b = shfl_down_v(mx, d);
-    mn = a < mn ? a : mn;
-    mx = b > mx ? b : mx;
+    for (int d = 16; d > 0; d >>= 1) x += __shfl_down_sync(0xffffffffu, x, d);
+    if (lane == 0) ws[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      x = ws[lane];
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) x += __shfl_down_sync(0xffffffffu, x, d);
+    }
+    return x;
+  };
+  double sum = 0.0;
+  float mn = __int_as_float(0x7f800000), mx = -mn;
+  for (int b = t; b < B; b += 1024) {
+    const float x = E[b];
+    sum += (double)x;
+    mn = x < mn ? x : mn;
+    mx = x > mx ? x : mx;
   }
-  if (lane == 0) ws[warp] = sum, wmn[warp] = mn, wmx[warp] = mx;
-  __syncthreads();
-  if (warp == 0) {
-    sum = ws[lane], mn = wmn[lane], mx = wmx[lane];
+  auto extremes = [&] {
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
-      sum += shfl_down_v(sum, d);
-      const M a = shfl_down_v(mn, d), b = shfl_down_v(mx, d);
+      const float a = __shfl_down_sync(0xffffffffu, mn, d), b = __shfl_down_sync(0xffffffffu, mx, d);
       mn = a < mn ? a : mn;
       mx = b > mx ? b : mx;
     }
-    if (lane == 0) ws[0] = sum, wmn[0] = mn, wmx[0] = mx;
+  };
+  extremes();
+  if (lane == 0) wmn[warp] = mn, wmx[warp] = mx;
+  sum = cta_sum(sum);
+  if (t == 0) quot[0] = sum / (double)B, quot[1] = 1.0 / (double)B;
+  if (warp == 0) {
+    mn = wmn[lane], mx = wmx[lane];
+    extremes();
   }
   __syncthreads();
-  sum = ws[0], mn = wmn[0], mx = wmx[0];
-}
-
-template <typename A>
-__global__ void __launch_bounds__(1024) stats_kernel(int B, const A* __restrict__ E, double* __restrict__ out,
-                                                     float* __restrict__ coef, uint32_t* __restrict__ err,
-                                                     DevState* ds, float beta1, float beta2) {
-  using S = typename StatAcc<A>::S;
-  using M = typename StatAcc<A>::M;
-  __shared__ S ws[32];
-  __shared__ M wmn[32], wmx[32];
-  __shared__ double wv[32];
-  __shared__ M dummy_mn[32], dummy_mx[32];
-  const int t = threadIdx.x;
-  if (ds && t == 0) {
+  const double mean = quot[0], inv = quot[1];
+  double ss = 0.0;
+  for (int b = t; b < B; b += 1024) {
+    const double d = (double)E[b] - mean;
+    ss += d * d;
+    if (coef) coef[b] = (float)(d * inv);
+  }
+  ss = cta_sum(ss);
+  if (ds && t == 1023) {  // beside thread 0's quotients
     ds->adam_t += 1;
     adam_factors(ds, beta1, beta2);
   }
-  S sum = 0;
-  M mn = StatAcc<A>::lo(), mx = StatAcc<A>::hi();
-  for (int b = t; b < B; b += blockDim.x) {
-    const A x = E[b];
-    sum += (S)x;
-    mn = (M)x < mn ? (M)x : mn;
-    mx = (M)x > mx ? (M)x : mx;
-  }
-  cta_reduce(sum, mn, mx, ws, wmn, wmx);
-  const double mean = (double)sum / (double)B;
-  double ss = 0.0;
-  for (int b = t; b < B; b += blockDim.x) {
-    const double d = (double)E[b] - mean;
-    ss += d * d;
-  }
-  M u0 = 0, u1 = 0;
-  cta_reduce(ss, u0, u1, wv, dummy_mn, dummy_mx);
   if (t == 0) {
     const double var = ss / (double)B;
     out[0] = mean;
@@ -335,10 +346,6 @@ __global__ void __launch_bounds__(1024) stats_kernel(int B, const A* __restrict_
     out[2] = (double)mn;
     out[3] = (double)mx;
     if (!isfinite(mean) || !isfinite(var)) atomicOr(err, kErrNonfinite);
-  }
-  if (coef) {
-    const double inv = 1.0 / (double)B;
-    for (int b = t; b < B; b += blockDim.x) coef[b] = (float)(((double)E[b] - mean) * inv);
   }
 }
 
@@ -503,7 +510,7 @@ cudaError_t launch_eloc_sparse(const vqmc_ctx* c, int B, const int8_t* d_s, void
 cudaError_t launch_eloc_dense_finish(const vqmc_ctx* c, int B, const int8_t* d_s, void* d_e, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
   const int ntiles = (c->n + 127) / 128;
-  eloc_dense_finish_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, c->n, ntiles, c->row_part, c->row_part_ld, d_s,
+  eloc_dense_finish_kernel<<<(B + 31) / 32, kFinishThreads, 0, st>>>(B, c->n, ntiles, c->row_part, c->row_part_ld, d_s,
                                                             (const float*)c->field, (float*)d_e);
   return cudaGetLastError();
 }
@@ -516,7 +523,7 @@ cudaError_t launch_stats(const vqmc_ctx* c, int B, const void* d_e, double* d_st
   if (c->ham == VQMC_HAM_SPARSE_I32)
     stats_int_kernel<<<1, 1024, 0, st>>>(B, (const int32_t*)d_e, d_stats, d_coef, c->err, ds, b1, b2);
   else
-    stats_kernel<float><<<1, 1024, 0, st>>>(B, (const float*)d_e, d_stats, d_coef, c->err, ds, b1, b2);
+    stats_kernel<<<1, 1024, 0, st>>>(B, (const float*)d_e, d_stats, d_coef, c->err, ds, b1, b2);
   return cudaGetLastError();
 }
 

@@ -24,11 +24,12 @@
 // an update adds nothing to a complete unit and an incomplete unit (g1 = 0
 // in shared memory until it completes) adds nothing to any logit.
 //
-// CTA = 16 samples, 8 warps: warps 0-3 own TMEM lanes 32w..32w+31 (read Z
+// CTA = 16 samples, 10 warps: warps 0-3 own TMEM lanes 32w..32w+31 (read Z
 // and the recent pre-activations); warps 0, 1, 6 and 7 are the solver (8
 // lanes per sample, each lane owning every 8th step of a segment and partial
 // sums of all the block's recent units) and then write the block's spins as
-// the update GEMM's operand; while they solve, warps 2-3 merge the previous
+// the update GEMM's operand; while they solve, warps 2, 3, 8 and 9 (the
+// helpers) merge the previous
 // block's recent g1 into the Z operand, prepare the next block's schedule,
 // logits and recent-unit weights, write out the previous block's spins and add
 // up its log pi; one thread of warp 4 streams 128 x 64 BF16 weight tiles with
@@ -37,14 +38,14 @@
 // the timeout bit and runs on without waiting, so it still finishes.
 //
 // What bounds it: the chain of the solver's segments, about 550 cycles each,
-// then warps 2-3 (models of few units per block), and some 3,300 cycles from one
+// then the helpers (models of few units per block), and some 3,300 cycles from one
 // block's last draw to the next one's first.  Measured (GB300, n = 10000, h =
-// 2000, 1024 samples with log pi): 1264 -> 742 us; n = 500, h = 193: 138 -> 92
-// us.  What that took, the arithmetic unchanged: warp-uniform control flow made
+// 2000, 1024 samples with log pi): 1264 -> 726 us; n = 500, h = 193: 138 -> 85
+// us; n = 10000, h = 424: 804 -> 505 us.  What that took, the arithmetic unchanged: warp-uniform control flow made
 // known to the compiler (the warp index, the segment bounds) and one elected
 // thread per issuing warp; one copy of each piece of code (280 -> 90 KB; the
 // instruction cache holds 32); predicated stores in place of branches; log pi
-// and the next block's schedule moved to warps 2-3.
+// and the next block's schedule moved to the helpers.
 #include <algorithm>
 #include <type_traits>
 
@@ -72,15 +73,20 @@ constexpr int kMaxHp = 2048;               // hidden units (padded) in TMEM
 constexpr int kDmax = 128;
 constexpr int kTmemCols = 512;             // A: 16 per 128 units (<= 256), Z at 256
 constexpr int kZCol = 256;
-constexpr int kThreads = 256;
+constexpr int kThreads = 320;
 // The solver: kLanes lanes per sample on warps 0, 1, 6 and 7 (one warp on
 // each SM sub-partition).
 constexpr int kLanes = 8;
 constexpr int kSolverThreads = kS * kLanes;
-// named barriers: 1 = warps 0-3 and the solver warps, 2 = warps 2-3 (arrive)
-// with the solver warps (sync)
-constexpr int kBar1Threads = 128 + 64;
-constexpr int kBar2Threads = 64 + kSolverThreads;
+// The helpers: warps 2, 3, 8 and 9, also one on each sub-partition (two on the
+// sub-partitions of warps 6 and 7 slowed those: 14,300 against 12,000 cycles a
+// block for the solver without them, and with few units per block the helpers'
+// work was the longer one: n = 10000, h = 424 599 -> 505 us with four).
+constexpr int kHelpers = 128;
+// named barriers: 1 = helpers and solver, 2 = helpers (arrive) with the solver
+// (sync)
+constexpr int kBar1Threads = kHelpers + kSolverThreads;
+constexpr int kBar2Threads = kHelpers + kSolverThreads;
 constexpr int kZld = kS + 1;               // padded row of the Z buffer
 constexpr uint32_t kIdesc = idesc_bf16(128, kS);
 
@@ -363,7 +369,7 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
   }
   if (q < kDmax / 32) SB[s_me * (kDmax / 32) + q] = q == 0 ? wd[0] : q == 1 ? wd[1] : q == 2 ? wd[2] : wd[3];
   // every recent unit is complete: its g1 goes to the staging operand Hr
-  // (2 chunks of 64 units from chunk klo / 64), once warps 2-3 have moved
+  // (2 chunks of 64 units from chunk klo / 64), once the helpers have moved
   // the previous block's recent g1 out of it
   asm volatile("bar.sync 2, %0;" ::"n"(kBar2Threads) : "memory");
 #pragma unroll
@@ -455,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     mbar_init(smem_u32(zfull), 1);
     mbar_init(smem_u32(ready), kSolverThreads);
-    mbar_init(smem_u32(merged), 64);
+    mbar_init(smem_u32(merged), kHelpers);
     mbar_init(smem_u32(drain), 1);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -618,11 +624,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Warps 0, 1, 6 and 7 are the solver, one warp on each SM sub-partition
     // (warp w runs on w % 4): the solver is issue-bound, and the producer and
     // MMA warps that share sub-partitions 0 and 1 with it issue little.
-    // Warps 0-3 read tensor memory; warps 2-3 meanwhile prepare the next
+    // Warps 0-3 read tensor memory; the helpers meanwhile prepare the next
     // block's logits and write out the previous block's spins.
-    const bool solver = warp <= 1 || warp >= 6;
+    const bool solver = warp <= 1 || warp == 6 || warp == 7;
     const int sid = (warp <= 1 ? warp : warp - 4) * 32 + lane;  // solver thread
-    const int ht = tid - 64;                                      // helper thread (warps 2-3)
+    const int ht = warp < 4 ? tid - 64 : tid - 192;               // helper thread
     const int s_me = sid / kLanes, sub = sid % kLanes;
     float lp = 0.0f, bias = 0.0f;
     const uint32_t tq = tmem + ((uint32_t)(32 * warp) << 16);
@@ -725,28 +731,23 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     };
     // The recent units' weights of block bb (W2 rows of its steps, W1 of its
-    // recent units), loaded by warps 2-3 (helper thread t < 64) into registers
-    // during the previous block's solver and stored into Vr / Wr once the
-    // solver is done.  Vr: thread t owns steps t and t + 64, 5 aligned
-    // 16-byte pieces of W2 from unit klo & ~7; Wr: pieces (unit q % 32,
-    // inputs 8 (q / 32) ..) for q = t + 64 j, so that a warp's transposing
-    // stores hit 32 different units.
-    uint4 gv[2][5], gw[8];
+    // recent units), loaded by the helpers (thread t) into registers during the
+    // previous block's solver and stored into Vr / Wr once the solver is done.
+    // Vr: thread t owns step t, 5 aligned 16-byte pieces of W2 from unit klo &
+    // ~7; Wr: pieces (unit q % 32, inputs 8 (q / 32) ..) for q = t + 128 j, so
+    // that a warp's transposing stores hit 32 different units.
+    uint4 gv[5], gw[4];
     auto gather_load = [&](int bb, int t) {
       const int klo = count_deg_le(bb * D, n, h), R = count_deg_le(bb * D + D, n, h) - klo;
       const int steps = min(D, n - bb * D), k8 = klo & ~7;
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int e = t + 64 * i;
+      for (int c = 0; c < 5; ++c)
+        gv[c] = (t < steps && k8 + 8 * c < g.hp)
+                    ? __ldg(reinterpret_cast<const uint4*>(g.v + (size_t)(bb * D + t) * g.hp + k8) + c)
+                    : make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int c = 0; c < 5; ++c)
-          gv[i][c] = (e < steps && k8 + 8 * c < g.hp)
-                         ? __ldg(reinterpret_cast<const uint4*>(g.v + (size_t)(bb * D + e) * g.hp + k8) + c)
-                         : make_uint4(0, 0, 0, 0);
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int q = t + 64 * j, r = q & 31, c = q >> 5;
+      for (int j = 0; j < 4; ++j) {
+        const int q = t + kHelpers * j, r = q & 31, c = q >> 5;
         gw[j] = (8 * c < steps && r < R)  // pieces past the last step stay in [0, np)
                     ? __ldg(reinterpret_cast<const uint4*>(g.w + (size_t)(klo + r) * g.np + (size_t)bb * D) + c)
                     : make_uint4(0, 0, 0, 0);
@@ -757,30 +758,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int steps = min(D, n - bb * D), off = klo & 7;
       // Vr[e][r] = W2 of step e, unit klo + r (r < 32; zero for units past the
       // block's recent ones: they complete after the block, masked in W2)
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int e = t + 64 * i;
-        if (e >= D) continue;
+      if (t < D) {
         uint32_t w[20];
 #pragma unroll
-        for (int c = 0; c < 5; ++c) w[4 * c] = gv[i][c].x, w[4 * c + 1] = gv[i][c].y, w[4 * c + 2] = gv[i][c].z,
-                                    w[4 * c + 3] = gv[i][c].w;
+        for (int c = 0; c < 5; ++c) w[4 * c] = gv[c].x, w[4 * c + 1] = gv[c].y, w[4 * c + 2] = gv[c].z, w[4 * c + 3] = gv[c].w;
+        // the 32 weights from element off on: a shift by off / 2 words (bits 1
+        // and 2 of off in turn), then by half a word
+#pragma unroll
+        for (int i = 0; i < 18; ++i) w[i] = (off & 4) ? w[i + 2] : w[i];
+#pragma unroll
+        for (int i = 0; i < 17; ++i) w[i] = (off & 2) ? w[i + 1] : w[i];
         uint32_t d[16];
 #pragma unroll
-        for (int sh = 0; sh < 4; ++sh)
-          if ((off >> 1) == sh) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) d[j] = (off & 1) ? __byte_perm(w[sh + j], w[sh + j + 1], 0x5432) : w[sh + j];
-          }
-        uint4* dst = reinterpret_cast<uint4*>(Vr + e * kLdW);
+        for (int i = 0; i < 16; ++i) d[i] = __byte_perm(w[i], w[i + 1], (off & 1) ? 0x5432 : 0x3210);
+        uint4* dst = reinterpret_cast<uint4*>(Vr + t * kLdW);
 #pragma unroll
         for (int j = 0; j < 4; ++j) dst[j] = make_uint4(d[4 * j], d[4 * j + 1], d[4 * j + 2], d[4 * j + 3]);
       }
       // Wr[e][r] = W1 of unit klo + r, input of step e (zero for r >= R)
       unsigned short* sw = reinterpret_cast<unsigned short*>(Wr);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int q = t + 64 * j, r = q & 31, c = q >> 5;
+      for (int j = 0; j < 4; ++j) {
+        const int q = t + kHelpers * j, r = q & 31, c = q >> 5;
         if (8 * c >= D) continue;
         const uint32_t w[4] = {gw[j].x, gw[j].y, gw[j].z, gw[j].w};
 #pragma unroll
@@ -790,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     };
-    // Turn b: the solver draws block b; warps 2-3 prepare block b + 1 and write
+    // Turn b: the solver draws block b; the helpers prepare block b + 1 and write
     // out block b - 1 (so there is one turn before the first block and one
     // after the last).
 #pragma unroll 1
@@ -838,7 +837,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         bias = warp < 4 && 32 * warp + lane < D && i < n ? __ldg(g.b2 + i) : 0.0f;
       }
       // (c) the D draws of the block (the solver warps), then the block's
-      // spins as the update GEMM's operand; warps 2-3 meanwhile
+      // spins as the update GEMM's operand; the helpers meanwhile
       if (solver) {
         uint32_t* sb = SB + (b & 1) * kS * (kDmax / 32);
         if (draws)
@@ -868,7 +867,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (b > 0) {
             const int kprev = count_deg_le((b - 1) * D, n, h), cb = kprev >> 6;
 #pragma unroll 1
-            for (int q = ht; q < (klo - kprev) * kS; q += 64) {
+            for (int q = ht; q < (klo - kprev) * kS; q += kHelpers) {
               const int k = kprev + q / kS, s = q % kS;
               const uint32_t o = sw128_offset(s, k & 63);
               bf16* src = reinterpret_cast<bf16*>(Hr + ((k >> 6) - cb) * 2048 + o);
@@ -887,7 +886,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           // next for block b + 1.
           const float* L = LG + ((b - 1) & 1) * kDrows * kS;
 #pragma unroll 1
-          for (int q = ht; q < kS * (D / 4); q += 64) {
+          for (int q = ht; q < kS * (D / 4); q += kHelpers) {
             const int e = 4 * (q / kS), left = n - (b - 1) * D - e;
             // sum of log sigma(x) = min(x, 0) - log(1 + exp(-|x|)): one
             // logarithm of the four factors, kept as their product minus 1
@@ -913,19 +912,20 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int x = lane == 0 ? N.klo : lane == 1 ? Rn : (int)N.zvalid;
             if (lane < 3) cn[kRmax + lane] = x;
           }
-          logits(b + 1, ht, 64);
+          logits(b + 1, ht, kHelpers);
           gather_load(b + 1, ht);
         }
-        if (b > 0) write_spins(b - 1, ht, 64);
+        if (b > 0) write_spins(b - 1, ht, kHelpers);
         asm volatile("bar.sync 1, %0;" ::"n"(kBar1Threads) : "memory");
         if (b + 1 < nblk) gather_store(b + 1, ht);
       }
     }
-    if (LP && !solver) {  // the partial sums of log pi of each sample's four threads
+    if (LP && !solver) {  // the partial sums of log pi of each sample's eight threads
       lp += __shfl_xor_sync(0xffffffffu, lp, 16);
-      if (warp == 3 && lane < kS) LG[lane] = lp;
-      asm volatile("bar.sync 2, 64;" ::: "memory");
-      if (warp == 2 && lane < kS && b0 + lane < g.B && !*abort) g.logp[b0 + lane] = lp + LG[lane];
+      if (lane < kS) LG[(ht >> 5) * kS + lane] = lp;
+      asm volatile("bar.sync 2, %0;" ::"n"(kHelpers) : "memory");
+      if (warp == 2 && lane < kS && b0 + lane < g.B && !*abort)
+        g.logp[b0 + lane] = (LG[lane] + LG[kS + lane]) + (LG[2 * kS + lane] + LG[3 * kS + lane]);
     }
   }
 

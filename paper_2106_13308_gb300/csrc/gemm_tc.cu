@@ -29,6 +29,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "gemm.cuh"
@@ -57,6 +58,15 @@ constexpr int kNumOps = 6;
 // output adjoint, the fused Adam steps) lose 20-30% without a second CTA
 // beside them (dW2 119 -> 144 us, dW1 113 -> 140 us, kOpOut 92 -> 122 us).
 constexpr int kStageChunks[kNumOps] = {2, 1, 1, 2, 1, 1};
+// With at most one tile per SM there is no second CTA to lose: every op takes
+// the larger copies (the weight gradients of n = h = 1000, 4096 samples: 36
+// tiles of 64 K chunks).  About half of a weight gradient's tiles lie outside
+// the mask and end at once.
+bool one_per_sm(int op, dim3 grid, int sms) {
+  const long long tiles = (long long)grid.x * grid.y;
+  const bool masked = op == kOpDV || op == kOpDW;
+  return (masked ? (tiles + std::max(grid.x, grid.y)) / 2 : tiles) <= sms;
+}
 template <int KC>
 struct Stages {
   static constexpr int kStage = KC * (TILE_A_BYTES + TILE_B_BYTES);
@@ -605,7 +615,7 @@ cudaError_t launch_gemm_tc_bf16(const GemmArgs<bf16>& a, cudaStream_t st) {
   // K chunks per stage: the chunked views cover the floor(K / 64) whole
   // chunks (the partial last chunk goes through the 2D maps' zero fill)
   const int kfull = a.K / BK;
-  const int kc = kfull >= 2 ? kStageChunks[a.op] : 1;
+  const int kc = kfull < 2 ? 1 : one_per_sm(a.op, grid, a.sms) ? 2 : kStageChunks[a.op];
   CUtensorMap mac = ma, mbc = mb, mb2c = mb2;
   if (kc == 2 && (!tc_encode_bf16_chunks(&mac, a.A, a.M, kfull * BK, a.lda, BM, 2) ||
                   !tc_encode_bf16_chunks(&mbc, a.Bm, a.N, kfull * BK, a.ldb, BN, 2) ||

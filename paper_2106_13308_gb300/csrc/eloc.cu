@@ -232,39 +232,43 @@ __global__ void eloc_sum_kernel(int B, int nslices, const A* __restrict__ part, 
 }
 
 // E_b = sum over N-tiles of the GEMM's row partials (1/2 s^T J s) + h.s, added
-// in the order of the spins.  The chain of n additions bounds it, so nothing
-// else is in it: a CTA takes 32 samples, its warps stage the terms +-h_i of
-// kFinishCols spins in shared memory, and one warp adds the previous ones, a
-// sample per lane.  (One thread per sample reading its spins as it adds took 37
-// us for 1024 samples of 500 spins.)
-constexpr int kFinishCols = 128, kFinishThreads = 288;
+// in the order of the spins.  The chain of n additions bounds it, so little
+// else is in it: a CTA takes 32 samples, its warps turn the spins of up to
+// kFinishCols columns into sign words (a ballot per sample and 32 columns, many
+// loads in flight), and one warp adds +-h_i, a sample per lane.  (One thread per
+// sample reading its spins as it adds took 37 us for 1024 samples of 500 spins.)
+constexpr int kFinishCols = 2048, kFinishThreads = 512;
 __global__ void __launch_bounds__(kFinishThreads)
     eloc_dense_finish_kernel(int B, int n, int ntiles, const float* __restrict__ part, int ld,
                              const int8_t* __restrict__ S, const float* __restrict__ field, float* __restrict__ E) {
-  __shared__ float term[2][32][kFinishCols + 1];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = blockIdx.x * 32 + lane;
+  __shared__ uint32_t down[32][kFinishCols / 32 + 1];  // bit q of word w: spin 32 w + q is not +1
+  __shared__ __align__(16) float h[kFinishCols];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, b0 = blockIdx.x * 32, b = b0 + lane;
   float e = 0.0f;
   if (warp == 0 && b < B)
     for (int t = 0; t < ntiles; ++t) e += part[(size_t)t * ld + b];
-  const int chunks = field ? (n + kFinishCols - 1) / kFinishCols : 0;
-  for (int c = 0; c <= chunks; ++c) {
+  for (int c0 = 0; field && c0 < n; c0 += kFinishCols) {
+    const int cols = min(kFinishCols, n - c0), words = (cols + 31) / 32;
+    for (int i = tid; i < cols; i += kFinishThreads) h[i] = field[c0 + i];
+    // warp w: words of samples w and w + 16 in turn
+#pragma unroll 8
+    for (int q = 0; q < 2 * words; ++q) {
+      const int s = warp + 16 * (q & 1), i = 32 * (q >> 1) + lane;
+      const bool in = i < cols & b0 + s < B;
+      const int8_t v = S[in ? (size_t)(b0 + s) * n + c0 + i : 0];
+      const uint32_t m = __ballot_sync(0xffffffffu, in & v <= 0);
+      if (lane == 0) down[s][q >> 1] = m;
+    }
+    __syncthreads();
     if (warp == 0) {
-      if (c > 0) {
-        const float* x = term[(c - 1) & 1][lane];
-        const int cnt = min(kFinishCols, n - (c - 1) * kFinishCols);
-#pragma unroll 16
-        for (int i = 0; i < cnt; ++i) e += x[i];
-      }
-    } else if (c < chunks) {
-      // warp w: samples 4 (w - 1) .. + 3; lane + 32 q: spins
+      for (int w = 0; w < words; ++w) {
+        const uint32_t m = down[lane][w];
+        const int cnt = min(32, cols - 32 * w);
+        if (cnt == 32) {
 #pragma unroll
-      for (int q = 0; q < kFinishCols / 32; ++q) {
-        const int i = c * kFinishCols + 32 * q + lane;
-        const float f = i < n ? field[i] : 0.0f;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int s = 4 * (warp - 1) + r, bs = blockIdx.x * 32 + s;
-          if (i < n && bs < B) term[c & 1][s][32 * q + lane] = S[(size_t)bs * n + i] > 0 ? f : -f;
+          for (int i = 0; i < 32; ++i) e += (m >> i) & 1u ? -h[32 * w + i] : h[32 * w + i];
+        } else {
+          for (int i = 0; i < cnt; ++i) e += (m >> i) & 1u ? -h[32 * w + i] : h[32 * w + i];
         }
       }
     }

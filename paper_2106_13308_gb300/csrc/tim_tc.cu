@@ -20,14 +20,15 @@
 // 64 (w / 4) .. of each 128-column output tile); warp 8 streams W2 tiles
 // (128 outputs x 64 units) with TMA; warp 9 issues the MMAs into two
 // accumulators, so that one output tile's epilogue runs beside the next
-// one's MMAs.  Every wait is bounded: after a failed one the CTA raises the
+// one's MMAs.  They wait with try_wait, which suspends: polling took a fifth of
+// the epilogue's issue slots.  Every wait is bounded: after a failed one the CTA raises the
 // timeout bit and runs on without waiting.
 //
-// What bounds it: the epilogue, one exponential, one logarithm and some 14 more
+// What bounds it: the epilogue, one exponential, one logarithm and some 11 more
 // instructions for each of the B n n / 2 outputs that do not cancel (164 M of
-// them at n = 500, B = 1024: 70 us of issue slots).  Measured there, h = 193
+// them at n = 500, B = 1024: 60 us of issue slots).  Measured there, h = 193
 // (GB300), a training step: 1141 us with the rows and their spins written to
-// memory and read back by the general GEMM, 483 us with this kernel.
+// memory and read back by the general GEMM, 467 us with this kernel.
 #include <algorithm>
 
 #include "gemm.cuh"
@@ -65,6 +66,15 @@ struct TimArgs {
   double* part;         // [blocks of flips][B]
   uint32_t* err;
 };
+
+// log sigma(x) = min(x, 0) - ln 2 log2(1 + 2^(-|x| log2 e)) on the hardware's
+// exp2 and log2; subnormals are flushed, which 1 + .. absorbs
+__device__ __forceinline__ float log_sigmoid_fast(float x) {
+  float e, l;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fabsf(x) * -1.44269504f));
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(1.0f + e));
+  return fmaf(l, -0.69314718f, fminf(x, 0.0f));
+}
 
 template <int ACT>
 __device__ __forceinline__ float act1(float a) {
@@ -137,7 +147,7 @@ __global__ void __launch_bounds__(kThreads, 2)
           for (int c = 0; c < nk; ++c, ++it) {
             const int s = it % g.stages;
             if (it >= g.stages &&
-                !test_or_abort(smem_u32(&empty[s]), (uint32_t)((it / g.stages - 1) & 1), abort, g.err)) {
+                !wait_or_abort(smem_u32(&empty[s]), (uint32_t)((it / g.stages - 1) & 1), abort, g.err)) {
               ok = false;
               break;
             }
@@ -157,17 +167,17 @@ __global__ void __launch_bounds__(kThreads, 2)
       bool ok = true;
       for (long long q = blockIdx.x; q < g.tiles && ok; q += gridDim.x, ++turn) {
         const int j = (int)(q / g.sblocks);
-        ok = test_or_abort(smem_u32(aready), (uint32_t)(turn & 1), abort, g.err);
+        ok = wait_or_abort(smem_u32(aready), (uint32_t)(turn & 1), abort, g.err);
         fence_after();
         for (int t = j * g.seg / kRows; t < ntiles && ok; ++t, ++acc) {
           const int nk = chunks(t), buf = acc & 1;
           if (acc >= 2) {
-            ok = test_or_abort(smem_u32(&accempty[buf]), (uint32_t)((acc / 2 - 1) & 1), abort, g.err);
+            ok = wait_or_abort(smem_u32(&accempty[buf]), (uint32_t)((acc / 2 - 1) & 1), abort, g.err);
             fence_after();
           }
           for (int c = 0; c < nk && ok; ++c, ++it) {
             const int s = it % g.stages;
-            ok = test_or_abort(smem_u32(&full[s]), (uint32_t)((it / g.stages) & 1), abort, g.err);
+            ok = wait_or_abort(smem_u32(&full[s]), (uint32_t)((it / g.stages) & 1), abort, g.err);
             if (!ok) break;
             fence_after();
             const uint64_t da = smem_desc_sw128(base + (uint32_t)(c * kTileBytes));
@@ -297,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             for (int e = 0; e < 4; ++e) {
               const float z = v[4 * e4 + e] + bq[e];
               const float x = __int_as_float(__float_as_int(z) ^ (int)((neg << (31 - 4 * e4 - e)) & 0x80000000u));
-              rs += fminf(x, 0.0f) - __logf(1.0f + __expf(-fabsf(z)));
+              rs += log_sigmoid_fast(x);
             }
           }
         }

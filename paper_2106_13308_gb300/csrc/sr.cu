@@ -249,10 +249,21 @@ __global__ void __launch_bounds__(256) chol_update_kernel(float* __restrict__ A,
   tri_index(blockIdx.x, &ii, &jj);
   const size_t i0 = (size_t)(k + 1 + ii) * kNB, j0 = (size_t)(k + 1 + jj) * kNB, k0 = (size_t)k * kNB;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  for (int idx = tid; idx < kNB * kNB; idx += 256) {
-    const int r = idx >> 6, l = idx & 63;
-    si[l][r] = A[(i0 + r) * ld + k0 + l];
-    sj[l][r] = A[(j0 + r) * ld + k0 + l];
+  // every load at once (ld and the block offsets are multiples of 64): the
+  // launch is one memory latency and 64 steps long
+  float4 x[4], y[4], old[4];
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const int r = ty + 16 * w, l = 4 * tx;
+    x[w] = *reinterpret_cast<const float4*>(A + (i0 + r) * ld + k0 + l);
+    y[w] = *reinterpret_cast<const float4*>(A + (j0 + r) * ld + k0 + l);
+    old[w] = *reinterpret_cast<const float4*>(A + (i0 + 4 * ty + w) * ld + j0 + 4 * tx);
+  }
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const int r = ty + 16 * w, l = 4 * tx;
+    si[l][r] = x[w].x, si[l + 1][r] = x[w].y, si[l + 2][r] = x[w].z, si[l + 3][r] = x[w].w;
+    sj[l][r] = y[w].x, sj[l + 1][r] = y[w].y, sj[l + 2][r] = y[w].z, sj[l + 3][r] = y[w].w;
   }
   __syncthreads();
   float acc[4][4] = {};
@@ -268,8 +279,30 @@ __global__ void __launch_bounds__(256) chol_update_kernel(float* __restrict__ A,
   }
 #pragma unroll
   for (int r = 0; r < 4; ++r)
+    *reinterpret_cast<float4*>(A + (i0 + 4 * ty + r) * ld + j0 + 4 * tx) =
+        make_float4(old[r].x - acc[r][0], old[r].y - acc[r][1], old[r].z - acc[r][2], old[r].w - acc[r][3]);
+}
+
+// s = fmaf(a[i stride], y[16 i], s) for i = 0 .. 4 blocks - 1 in order, sixteen
+// loads of a in flight: their latency bounds the solve's sweeps
+__device__ __forceinline__ void sweep(const float* a, size_t stride, const float* y, int blocks, float& s) {
+  int k = 0;
+#pragma unroll 1
+  for (; k + 4 <= blocks; k += 4) {
+    float x[16];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) A[(i0 + 4 * ty + r) * ld + j0 + 4 * tx + q] -= acc[r][q];
+    for (int i = 0; i < 16; ++i) x[i] = __ldg(a + (size_t)(4 * k + i) * stride);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s = fmaf(x[i], y[16 * (4 * k + i)], s);
+  }
+#pragma unroll 1
+  for (; k < blocks; ++k) {
+    float x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = __ldg(a + (size_t)(4 * k + i) * stride);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s = fmaf(x[i], y[16 * (4 * k + i)], s);
+  }
 }
 
 // L L^T x = rhs with the factor from the kernels above (T blocks of 64; rows
@@ -295,7 +328,7 @@ __global__ void __launch_bounds__(1024) chol_solve_kernel(const float* __restric
       const int r = tid >> 4, p = tid & 15;
       const float* row = A + (r0 + r) * ld;
       float s = 0.0f;
-      for (int l = p; l < (int)r0; l += 16) s = fmaf(row[l], y[l], s);
+      sweep(row + p, 16, y + p, kb, s);
 #pragma unroll
       for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
       if (p == 0) rv[r] = y[r0 + r] - s;
@@ -324,7 +357,7 @@ __global__ void __launch_bounds__(1024) chol_solve_kernel(const float* __restric
     {
       const int r = tid & 63, p = tid >> 6;
       float s = 0.0f;
-      for (int l = (int)r0 + kNB + p; l < N; l += 16) s = fmaf(A[(size_t)l * ld + r0 + r], y[l], s);
+      sweep(A + (r0 + kNB + p) * ld + r0 + r, (size_t)16 * ld, y + r0 + kNB + p, T - 1 - kb, s);
       part[p * kNB + r] = s;
     }
     __syncthreads();

@@ -39,8 +39,12 @@ namespace vqmc {
 namespace {
 
 constexpr int BM = 128, BN = 128, BK = 64, NSTAGE = 3;
-constexpr int kThreads = 256;
-constexpr int kHalf = BN / 2;  // columns per epilogue thread
+constexpr bool is_wgrad(int op) { return op == kOpDV || op == kOpDW; }
+// Threads, and columns per epilogue thread.  The weight gradients' epilogue is a
+// chain of a load, a root and a division per entry that a warp can't overlap
+// with the next entry's (both have a branch for unusual operands): sixteen warps.
+constexpr int threads_of(int op) { return is_wgrad(op) ? 512 : 256; }
+constexpr int cols_of(int op) { return BN / (threads_of(op) / 128); }
 constexpr int TILE_A_BYTES = BM * BK * 2;  // 16 KB
 constexpr int TILE_B_BYTES = BN * BK * 2;  // 16 KB
 constexpr int TMEM_COLS = BN;  // FP32 accumulator: 128 lanes x BN columns
@@ -59,7 +63,7 @@ constexpr int kNumOps = 6;
 // beside them (dW2 119 -> 144 us, dW1 113 -> 140 us, kOpOut 92 -> 122 us).
 constexpr int kStageChunks[kNumOps] = {2, 1, 1, 2, 1, 1};
 // With at most one tile per SM there is no second CTA to lose: every op takes
-// the larger copies (the weight gradients of n = h = 1000, 4096 samples: 36
+// the larger copies (weight gradients of n = h = 1000, 4096 samples: 43.5 -> 36.2 us; 36
 // tiles of 64 K chunks).  About half of a weight gradient's tiles lie outside
 // the mask and end at once.
 bool one_per_sm(int op, dim3 grid, int sms) {
@@ -133,6 +137,20 @@ __device__ __forceinline__ void logsig_pair(float x, float& ls, float& sm) {
   sm = __fdividef(x >= 0.0f ? e : 1.0f, 1.0f + e);
 }
 
+// *p = x where ok holds, as a predicated store: a warp serialises the branch
+// around a conditional store (some 70 cycles where lanes differ), and the
+// compiler can't move the next element's arithmetic across it
+__device__ __forceinline__ void store_if(bool ok, bf16* p, float x) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t@p st.global.b16 [%1], %2;\n\t}" ::"r"((int)ok), "l"(p),
+               "h"(__bfloat16_as_ushort(__float2bfloat16_rn(x)))
+               : "memory");
+}
+__device__ __forceinline__ void store_if_cs(bool ok, float* p, float x) {  // evict-first, as __stcs
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t@p st.global.cs.f32 [%1], %2;\n\t}" ::"r"((int)ok),
+               "l"(p), "f"(x)
+               : "memory");
+}
+
 // 16 consecutive BF16 values as two 16-byte stores
 __device__ __forceinline__ void store16_bf16(bf16* dst, const float (&x)[16]) {
   uint32_t w[8];
@@ -167,11 +185,11 @@ __device__ __forceinline__ uint32_t neg_bits16(const int8_t* src, int valid) {
 }
 
 // Row stride (floats) of a warp's staging block in shared memory: 32 rows x
-// 64 columns, padded so that both row- and column-wise accesses are free of
+// 32 columns, padded so that both row- and column-wise accesses are free of
 // bank conflicts.
-constexpr int kStageLd = kHalf + 1;
+constexpr int kStageCols = cols_of(kOpDV), kStageLd = kStageCols + 1;
 
-// The weight-gradient epilogue of one warp after its 32 x 64 block of the
+// The weight-gradient epilogue of one warp after its 32 x 32 block of the
 // gradient (rows m0w.., columns c0..) was staged in G: row r of the block
 // keeps columns [kl, kh) of lane r's (kl_me, kh_me).  Lanes run along the
 // columns for the row-major arrays (theta, moments, gradient, row copy: one
@@ -181,59 +199,57 @@ constexpr int kStageLd = kHalf + 1;
 // is stored, zero outside the mask.
 __device__ __forceinline__ void wgrad_block(const GemmArgs<bf16>& g, bool fused, float* G, int m0w, int c0,
                                             int lane, int kl_me, int kh_me) {
-  const float ibc1 = fused ? __ldg(g.ibc) : 0.0f, ibc2 = fused ? __ldg(g.ibc + 1) : 0.0f;
-  for (int r0 = 0; r0 < 32; r0 += 4) {
-    float gq[8], mq[8], vq[8], tq[8];
-    bool keep[8], in[8];
+  const int k = c0 + lane;
+  if (!fused) {
+    for (int r = 0; r < 32; ++r) {
+      const int kl = __shfl_sync(0xffffffffu, kl_me, r), kh = __shfl_sync(0xffffffffu, kh_me, r), m = m0w + r;
+      if (m < g.M && k < g.N) g.gout[(size_t)m * g.ldg + k] = k >= kl && k < kh ? G[r * kStageLd + lane] : 0.0f;
+    }
+    return;
+  }
+  const float ibc1 = __ldg(g.ibc), ibc2 = __ldg(g.ibc + 1);
+  // No branches: every lane loads (entries outside the matrix from its last row
+  // or column) and computes, the stores are predicated.
+  constexpr int kRowsAtOnce = 8;
+#pragma unroll 1
+  for (int r0 = 0; r0 < 32; r0 += kRowsAtOnce) {
+    float mq[kRowsAtOnce], vq[kRowsAtOnce], tq[kRowsAtOnce];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int r = r0 + (j >> 1), col = lane + 32 * (j & 1);
-      const int kl = __shfl_sync(0xffffffffu, kl_me, r), kh = __shfl_sync(0xffffffffu, kh_me, r);
-      const int m = m0w + r, k = c0 + col;
-      in[j] = m < g.M && k < g.N;
-      keep[j] = in[j] && k >= kl && k < kh;
-      gq[j] = G[r * kStageLd + col];
-      if (fused && keep[j]) {
-        const size_t q = (size_t)m * g.ldg + k;
-        mq[j] = __ldcs(g.adam_m + q);
-        vq[j] = __ldcs(g.adam_v + q);
-        tq[j] = __ldcs(g.theta + q);
-      }
+    for (int j = 0; j < kRowsAtOnce; ++j) {
+      const size_t q = (size_t)min(m0w + r0 + j, g.M - 1) * g.ldg + min(k, g.N - 1);
+      mq[j] = __ldcs(g.adam_m + q);
+      vq[j] = __ldcs(g.adam_v + q);
+      tq[j] = __ldcs(g.theta + q);
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int r = r0 + (j >> 1), col = lane + 32 * (j & 1);
-      const int m = m0w + r, k = c0 + col;
+    for (int j = 0; j < kRowsAtOnce; ++j) {
+      const int r = r0 + j, m = m0w + r;
+      const int kl = __shfl_sync(0xffffffffu, kl_me, r), kh = __shfl_sync(0xffffffffu, kh_me, r);
+      const bool keep = m < g.M && k < g.N && k >= kl && k < kh;
       const size_t q = (size_t)m * g.ldg + k;
-      if (!fused) {
-        if (in[j]) g.gout[q] = keep[j] ? gq[j] : 0.0f;
-        continue;
-      }
-      float t = 0.0f;
-      if (keep[j]) {
-        const float mn = g.beta1 * mq[j] + (1.0f - g.beta1) * gq[j];
-        const float vn = g.beta2 * vq[j] + (1.0f - g.beta2) * gq[j] * gq[j];
-        t = tq[j] - g.lr * (mn * ibc1) / (sqrtf(vn * ibc2) + g.eps);
-        __stcs(g.adam_m + q, mn);
-        __stcs(g.adam_v + q, vn);
-        __stcs(g.theta + q, t);
-        if (g.cp_row) g.cp_row[(size_t)(m + g.cp_shift) * g.ld_cp_row + k] = __float2bfloat16_rn(t);
-      }
-      G[r * kStageLd + col] = t;
+      const float gq = G[r * kStageLd + lane];
+      const float mn = g.beta1 * mq[j] + (1.0f - g.beta1) * gq;
+      const float vn = g.beta2 * vq[j] + (1.0f - g.beta2) * gq * gq;
+      const float x = keep ? vn * ibc2 : 1.0f;  // (a masked entry's 0 would take the root's slow path)
+      const float t = tq[j] - g.lr * (mn * ibc1) / (sqrtf(x) + g.eps);
+      store_if_cs(keep, g.adam_m + q, mn);
+      store_if_cs(keep, g.adam_v + q, vn);
+      store_if_cs(keep, g.theta + q, t);
+      if (g.cp_row) store_if(keep, g.cp_row + (size_t)(m + g.cp_shift) * g.ld_cp_row + k, t);
+      G[r * kStageLd + lane] = t;  // (masked entries are not read)
     }
   }
-  if (!fused) return;
   __syncwarp();
   const int m = m0w + lane;
-  if (m < g.M)
-    for (int col = 0; col < kHalf; ++col) {
-      const int k = c0 + col;
-      if (k >= kl_me && k < kh_me && k < g.N) g.cp_t[(size_t)k * g.ld_cp_t + m] = __float2bfloat16_rn(G[lane * kStageLd + col]);
-    }
+#pragma unroll 4
+  for (int col = 0; col < kStageCols; ++col) {
+    const int kc = c0 + col;
+    store_if(m < g.M && kc >= kl_me && kc < kh_me && kc < g.N, g.cp_t + (size_t)kc * g.ld_cp_t + m, G[lane * kStageLd + col]);
+  }
 }
 
 template <int OP, int KC>
-__global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
+__global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                    const __grid_constant__ CUtensorMap mapB2, const __grid_constant__ CUtensorMap mapAc,
                    const __grid_constant__ CUtensorMap mapBc, const __grid_constant__ CUtensorMap mapB2c,
@@ -257,7 +273,8 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
   const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int quad = warp & 3, half = warp >> 2;
   constexpr int op = OP;
-  constexpr bool kWgrad = op == kOpDV || op == kOpDW;
+  constexpr bool kWgrad = is_wgrad(op);
+  constexpr int kThreads = threads_of(OP), kCols = cols_of(OP);
   const bool fused = kWgrad && g.theta != nullptr;
   // Tiles in launch order, heaviest K range first where the masks make the
   // ranges uneven (the hidden GEMM and the output GEMM: K grows with the
@@ -363,20 +380,20 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
   // ------------------------------------ epilogue operands, during the main loop
   const int m = m0 + quad * 32 + lane;  // this thread's tile row
   const bool mvalid = m < g.M;
-  const int c0 = n0 + kHalf * half;     // this thread's first column
+  const int c0 = n0 + kCols * half;     // this thread's first column
   if (tid < BN) bias_s[tid] = ((op == kOpHidden || op == kOpOut) && n0 + tid < g.N) ? g.bias[n0 + tid] : 0.0f;
-  uint32_t neg[kHalf / 16];  // kOpOut / kOpEloc: bit q of neg[c]: spin of column c0 + 16c + q is -1
-  uint4 hpre[kHalf / 8];     // kOpGA: stored activations H[m][c0 .. c0 + 63]
+  uint32_t neg[kCols / 16];  // kOpOut / kOpEloc: bit q of neg[c]: spin of column c0 + 16c + q is -1
+  uint4 hpre[kCols / 8];     // kOpGA: stored activations H[m][c0 .. c0 + 63]
   if constexpr (op == kOpOut || op == kOpEloc) {
 #pragma unroll
-    for (int c = 0; c < kHalf / 16; ++c)
+    for (int c = 0; c < kCols / 16; ++c)
       neg[c] = mvalid ? neg_bits16(g.S8 + (size_t)m * g.lds8 + c0 + 16 * c, g.N - (c0 + 16 * c)) : 0u;
   }
   if constexpr (op == kOpGA) {
     const bf16* hrow = g.aux + (size_t)m * g.ldaux + c0;
-    const bool vec = mvalid && c0 + kHalf <= g.N && (reinterpret_cast<uintptr_t>(hrow) & 15) == 0;
+    const bool vec = mvalid && c0 + kCols <= g.N && (reinterpret_cast<uintptr_t>(hrow) & 15) == 0;
 #pragma unroll
-    for (int c = 0; c < kHalf / 8; ++c) {
+    for (int c = 0; c < kCols / 8; ++c) {
       if (vec) {
         hpre[c] = __ldg(reinterpret_cast<const uint4*>(hrow) + c);
       } else {
@@ -405,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
   __syncwarp();
   fence_after();
   __syncthreads();  // bias_s
-  const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(kHalf * half);
+  const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(kCols * half);
   // warp-uniform: tcgen05.ld is executed by all lanes of a warp or none
   const bool acc_valid = __all_sync(0xffffffffu, nkt > 0 && done_ok);
   float rowsum = 0.0f;
@@ -413,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
   const float cm = (op == kOpOut && g.coef && mvalid) ? g.coef[m] : 0.0f;
 
 #pragma unroll
-  for (int c = 0; c < kHalf / 16; ++c) {
+  for (int c = 0; c < kCols / 16; ++c) {
     float v[16];
     if (acc_valid) {
       tmem_ld16(trow + (uint32_t)(16 * c), v);
@@ -456,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
           const float sgn = (neg[c] >> q) & 1u ? -1.0f : 1.0f;
           float ls, sm;
           logsig_pair(sgn * z, ls, sm);
-          if (in) rowsum += ls;
+          rowsum += in ? ls : 0.0f;
           d[q] = in ? cm * sgn * sm : 0.0f;
           cs[q] = d[q];
         }
@@ -464,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
           const float x = ((neg[c] >> q) & 1u ? -1.0f : 1.0f) * (v[q] + bias_s[lb + q]);
-          if (mvalid && nb + q < g.N) rowsum += fminf(x, 0.0f) - log_one_plus(__expf(-fabsf(x)));
+          rowsum += mvalid && nb + q < g.N ? fminf(x, 0.0f) - log_one_plus(__expf(-fabsf(x))) : 0.0f;
         }
       }
       if (g.coef) {
@@ -477,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
         }
 #pragma unroll
         for (int q = 0; q < 16; ++q)
-          if (mvalid && nb + q < g.N) g.out_t[(size_t)(nb + q) * g.ldt + m] = __float2bfloat16_rn(d[q]);
+          store_if(mvalid && nb + q < g.N, g.out_t + (size_t)(nb + q) * g.ldt + m, d[q]);
       }
     } else if constexpr (op == kOpGA) {
       // the adjoint of the pre-activation: (D V)[m][k] * act'(a), act' from H
@@ -489,7 +506,7 @@ __global__ void __launch_bounds__(kThreads, Stages<KC>::kMinBlocks)
         const bool in = mvalid && nb + q < g.N;
         const float da = g.act == VQMC_ACT_RELU ? (hv > 0.0f ? 1.0f : 0.0f) : hv * (1.0f - hv);
         const float x = in ? v[q] * da : 0.0f;
-        if (in) g.out_t[(size_t)(nb + q) * g.ldt + m] = __float2bfloat16_rn(x);
+        store_if(in, g.out_t + (size_t)(nb + q) * g.ldt + m, x);
         cs[q] = x;
       }
     } else if constexpr (kWgrad) {
@@ -625,9 +642,9 @@ cudaError_t launch_gemm_tc_bf16(const GemmArgs<bf16>& a, cudaStream_t st) {
 #define VQMC_GEMM_LAUNCH(OP)                                                                                   \
   case OP:                                                                                                     \
     if (kc == 2)                                                                                               \
-      gemm_tc_kernel<OP, 2><<<grid, kThreads, Stages<2>::kSmem, st>>>(ma, mb, mb2, mac, mbc, mb2c, a, two, kfull); \
+      gemm_tc_kernel<OP, 2><<<grid, threads_of(OP), Stages<2>::kSmem, st>>>(ma, mb, mb2, mac, mbc, mb2c, a, two, kfull); \
     else                                                                                                       \
-      gemm_tc_kernel<OP, 1><<<grid, kThreads, Stages<1>::kSmem, st>>>(ma, mb, mb2, mac, mbc, mb2c, a, two, kfull); \
+      gemm_tc_kernel<OP, 1><<<grid, threads_of(OP), Stages<1>::kSmem, st>>>(ma, mb, mb2, mac, mbc, mb2c, a, two, kfull); \
     break;
   switch (a.op) {
     VQMC_GEMM_LAUNCH(kOpHidden)

@@ -4,7 +4,8 @@
 // the log-prob forward (Sec. 2.3), its adjoint (gradient of Sec. 2.1) and the
 // dense local energy.
 //
-// One CTA computes one 128 x 128 output tile with 8 warps:
+// One CTA computes one 128 x 128 output tile with 8 warps (16 in the weight
+// gradients):
 //   warp 0 allocates 128 TMEM columns; its lane 0 streams K-tiles of A
 //          (128 x 64) and B (128 x 64) into a 3-stage shared-memory ring with
 //          TMA (cp.async.bulk.tensor, 128-byte swizzle, zero fill beyond the
@@ -12,8 +13,9 @@
 //   warp 1 lane 0 issues tcgen05.mma (M = 128, N = 128, K = 16, four per
 //          K-tile) into the TMEM accumulator and tcgen05.commit-s each stage
 //          back to the producer and, after the last K-tile, to the epilogue;
-//   all 8 warps run the op's epilogue: warp w reads TMEM lanes
-//          32 (w % 4) .. + 31 (its tile rows), columns 64 (w / 4) .. + 63,
+//   all warps run the op's epilogue: warp w reads TMEM lanes 32 (w % 4) .. +
+//          31 (its tile rows), columns 64 (w / 4) .. + 63 (32 (w / 4) .. + 31 in
+//          the weight gradients),
 //          with tcgen05.ld.  The epilogue operands that do not depend on the
 //          accumulator (spins, stored activations, bias; the optimiser state
 //          of the fused Adam step) are requested while the main loop runs.

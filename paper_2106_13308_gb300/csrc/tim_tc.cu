@@ -28,7 +28,8 @@
 // instructions for each of the B n n / 2 outputs that do not cancel (164 M of
 // them at n = 500, B = 1024: 60 us of issue slots).  Measured there, h = 193
 // (GB300), a training step: 1141 us with the rows and their spins written to
-// memory and read back by the general GEMM, 467 us with this kernel.
+// memory and read back by the general GEMM, 446 us with this kernel (0.21 ms
+// of it; 156 M warp instructions, 64% of the issue slots).
 #include <algorithm>
 
 #include "gemm.cuh"
@@ -237,18 +238,16 @@ __global__ void __launch_bounds__(kThreads, 2)
               w[p].x = k < h ? __bfloat162float(__float2bfloat16_rn(__ldg(wrow + 64 * p))) : 0.0f;
               w[p].y = k + 1 < h ? __bfloat162float(__float2bfloat16_rn(__ldg(wrow + 64 * p + 1))) : 0.0f;
             }
+            // units past h: activation of the zero padding of A, times zero weights
+            unsigned char* row = sm + (size_t)(k0 / 64) * kTileBytes + sw128_offset(s * per + f, 2 * lane);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const float two_s = flip && b[u] < g.B ? 2.0f * (float)__ldg(g.S + (size_t)b[u] * n + i) : 0.0f;
-              const int r = 32 * u + s * per + f;
 #pragma unroll
               for (int p = 0; p < 4; ++p) {
                 if (p >= np) break;
-                const int k = k0 + 64 * p + 2 * lane;
-                const float x0 = k < h ? act1<ACT>(a[u][p].x - two_s * w[p].x) : 0.0f;
-                const float x1 = k + 1 < h ? act1<ACT>(a[u][p].y - two_s * w[p].y) : 0.0f;
-                *reinterpret_cast<__nv_bfloat162*>(sm + (size_t)(k0 / 64 + p) * kTileBytes + sw128_offset(r, 2 * lane)) =
-                    __floats2bfloat162_rn(x0, x1);
+                *reinterpret_cast<__nv_bfloat162*>(row + p * kTileBytes + u * 4096) =
+                    __floats2bfloat162_rn(act1<ACT>(a[u][p].x - two_s * w[p].x), act1<ACT>(a[u][p].y - two_s * w[p].y));
               }
             }
           }

@@ -47,28 +47,12 @@ __device__ __forceinline__ float weight<bf16>(float w) { return __bfloat162float
 // Rows [g0, g0 + rows) of the expansion, one warp per row: the hidden
 // activations act(a(x) - 2 s_i W1_:,i) (the output GEMM's operand, padding
 // zero; the BF16 model rounds them to BF16 like every hidden activation) and
-// the row's spins as int8 for the output epilogue's signs, 8 activations and
-// 16 spins per lane and 16-byte store.  A: a(x) [B][hp] FP32; W1t: the
-// master W1^T [n][h] (FP32; rounded to BF16 for the BF16 model).  hp and np
-// are multiples of 64.
-template <typename T>
-__device__ __forceinline__ void store8(T* p, const float (&x)[8]);
-template <>
-__device__ __forceinline__ void store8<float>(float* p, const float (&x)[8]) {
-  reinterpret_cast<float4*>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
-  reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
-}
-template <>
-__device__ __forceinline__ void store8<bf16>(bf16* p, const float (&x)[8]) {
-  uint32_t w[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(x[2 * q], x[2 * q + 1]);
-    w[q] = *reinterpret_cast<const uint32_t*>(&v);
-  }
-  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
+// the row's spins as int8 for the output epilogue's signs.  Lanes run along the
+// row in every access: the rows of W1 and of the spins have no alignment, so
+// that wider pieces per lane only spread a warp's access over more lines (8
+// activations and 16 spins per lane took 80 us for 131,072 FP32 rows of 256 +
+// 512).  A: a(x) [B][hp] FP32; W1t: the master W1^T [n][h] (FP32; rounded to
+// BF16 for the BF16 model).  hp and np are multiples of 64.
 template <typename T>
 __global__ void tim_rows_kernel(int n, int h, int hp, int np, int act, long long g0, int rows,
                                 const int8_t* __restrict__ S, const float* __restrict__ A,
@@ -83,32 +67,34 @@ __global__ void tim_rows_kernel(int n, int h, int hp, int np, int act, long long
   const float two_s = i < n ? 2.0f * (float)src[i] : 0.0f;
   const float* wrow = W1t + (size_t)(i < n ? i : 0) * h;
   T* dh = H + (size_t)r * hp;
-  for (int k0 = 8 * lane; k0 < hp; k0 += 256) {
-    const float4 p0 = reinterpret_cast<const float4*>(a0 + k0)[0], p1 = reinterpret_cast<const float4*>(a0 + k0)[1];
-    const float av[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-    float x[8];
+  for (int k0 = 0; k0 < hp; k0 += 256) {
+    float av[8], wv[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int k = k0 + e;
-      x[e] = 0.0f;
-      if (k < h) {
-        const float a = i < n ? av[e] - two_s * weight<T>(wrow[k]) : av[e];
-        x[e] = act == VQMC_ACT_RELU ? fmaxf(a, 0.0f) : 1.0f / (1.0f + expf(-a));
-      }
+      const int k = k0 + 32 * e + lane;
+      av[e] = k < h ? a0[k] : 0.0f;
+      wv[e] = k < h && i < n ? wrow[k] : 0.0f;
     }
-    store8<T>(dh + k0, x);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int k = k0 + 32 * e + lane;
+      const float a = i < n ? av[e] - two_s * weight<T>(wv[e]) : av[e];
+      const float x = act == VQMC_ACT_RELU ? fmaxf(a, 0.0f) : 1.0f / (1.0f + expf(-a));
+      if (k < hp) dh[k] = to_t<T>(k < h ? x : 0.0f);
+    }
   }
   int8_t* d8 = S8 + (size_t)r * np;
-  for (int k0 = 16 * lane; k0 < np; k0 += 512) {
-    uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll 4
+  for (int k0 = 4 * lane; k0 < np; k0 += 128) {
+    uint32_t w = 0;
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
+    for (int e = 0; e < 4; ++e) {
       const int k = k0 + e;
       int v = k < n ? src[k] : 0;
       if (k == i) v = -v;
-      w[e >> 2] |= (uint32_t)(uint8_t)(int8_t)v << (8 * (e & 3));
+      w |= (uint32_t)(uint8_t)(int8_t)v << (8 * e);
     }
-    *reinterpret_cast<uint4*>(d8 + k0) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint32_t*>(d8 + k0) = w;
   }
 }
 

@@ -35,6 +35,11 @@ __host__ __device__ inline int count_deg_le(int x, int n, int h) {
   return c > h ? h : (int)c;
 }
 
+// lane 0's value, which the compiler then knows to be the same in all lanes: it
+// keeps the control flow that depends on it free of the reconvergence code
+// that a shuffle behind a possibly divergent branch costs (some 8 instructions)
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 // The samplers read rows in groups: their weight copies have zero rows past the
 // model's (wt_s row j = input j with row 0 zero, v_s row i = output i+1), up to
 // three rows past the last one they need, in multiples of 8.

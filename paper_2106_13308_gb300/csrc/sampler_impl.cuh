@@ -91,11 +91,6 @@ __device__ __forceinline__ void cp_wait() {  // all but the last N groups have l
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// lane 0's value, which the compiler then knows to be the same in all lanes: it
-// keeps the control flow that depends on it free of the reconvergence code
-// that a shuffle behind a possibly divergent branch costs (some 8 instructions)
-__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
-
 // 16 bytes to shared memory if in: one predicated store (a divergent branch
 // around it costs about 70 cycles)
 __device__ __forceinline__ void st16_if(uint32_t dst, uint64_t x, uint64_t y, bool in) {

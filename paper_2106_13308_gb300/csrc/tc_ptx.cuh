@@ -12,7 +12,6 @@ namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 // True in one lane of a converged warp.  The issuing threads of tcgen05 and TMA
 // instructions are chosen this way, not by a lane index: the compiler then
 // knows that a single thread runs the branch and issues each instruction once,

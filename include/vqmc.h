@@ -213,8 +213,8 @@ vqmc_status vqmc_sample(vqmc_ctx* ctx, int32_t B, const float* d_u, uint64_t ite
  * in FP32 otherwise (|E - E_exact| <= n^2 2^-23 max|J_ij|).  With a transverse field
  * alpha, also -sum_i alpha_i sqrt(pi(s^(i)) / pi(s)) (s^(i): spin i flipped,
  * Eq. (e:tim)): the n flipped states of every sample and the sample itself
- * go through the model's log-prob GEMMs in chunks of rows, so this costs
- * about n + 1 log-prob evaluations per sample. */
+ * go through the model's output layer, so this costs about n + 1 log-prob
+ * evaluations per sample. */
 vqmc_status vqmc_local_energy(vqmc_ctx* ctx, int32_t B, const int8_t* d_s, void* d_e, vqmc_stream stream);
 
 /* log pi(s_b) (Sec. 2.3) of B configurations by the full masked forward

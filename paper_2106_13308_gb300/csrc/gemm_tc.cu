@@ -431,8 +431,16 @@ __global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
   const bool want_col = g.col_part && ((op == kOpOut && g.coef) || op == kOpGA);
   const float cm = (op == kOpOut && g.coef && mvalid) ? g.coef[m] : 0.0f;
 
-#pragma unroll
+  // The epilogues with exponentials stay rolled: unrolled they are 90 KB (output)
+  // and 70 KB (hidden) of code, beyond the instruction cache's 32.
+  constexpr int kUnroll = op == kOpOut || op == kOpHidden ? 1 : kCols / 16;
+#pragma unroll kUnroll
   for (int c = 0; c < kCols / 16; ++c) {
+    uint32_t neg_c = 0;
+    if constexpr (op == kOpOut || op == kOpEloc) {
+#pragma unroll
+      for (int e = 0; e < kCols / 16; ++e) neg_c = c == e ? neg[e] : neg_c;
+    }
     float v[16];
     if (acc_valid) {
       tmem_ld16(trow + (uint32_t)(16 * c), v);
@@ -472,7 +480,7 @@ __global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
         for (int q = 0; q < 16; ++q) {
           const bool in = mvalid && nb + q < g.N;
           const float z = v[q] + bias_s[lb + q];
-          const float sgn = (neg[c] >> q) & 1u ? -1.0f : 1.0f;
+          const float sgn = (neg_c >> q) & 1u ? -1.0f : 1.0f;
           float ls, sm;
           logsig_pair(sgn * z, ls, sm);
           rowsum += in ? ls : 0.0f;
@@ -482,7 +490,7 @@ __global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
       } else {  // log pi only
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
-          const float x = ((neg[c] >> q) & 1u ? -1.0f : 1.0f) * (v[q] + bias_s[lb + q]);
+          const float x = ((neg_c >> q) & 1u ? -1.0f : 1.0f) * (v[q] + bias_s[lb + q]);
           rowsum += mvalid && nb + q < g.N ? fminf(x, 0.0f) - log_one_plus(__expf(-fabsf(x))) : 0.0f;
         }
       }
@@ -519,7 +527,7 @@ __global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
     } else if constexpr (op == kOpEloc) {
 #pragma unroll
       for (int q = 0; q < 16; ++q)
-        if (mvalid && nb + q < g.N) rowsum = fmaf((neg[c] >> q) & 1u ? -0.5f : 0.5f, v[q], rowsum);
+        if (mvalid && nb + q < g.N) rowsum = fmaf((neg_c >> q) & 1u ? -0.5f : 0.5f, v[q], rowsum);
     }
     if (want_col) {
       const float w = colsum16(cs, lane);

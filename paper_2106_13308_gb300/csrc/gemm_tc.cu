@@ -458,9 +458,19 @@ __global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
       float x[16];
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
-        const float a = v[q] + bias_s[lb + q];
-        if (g.pre && mvalid && nb + q < g.N) g.pre[(size_t)m * g.ldpre + nb + q] = a;
-        x[q] = g.act == VQMC_ACT_RELU ? fmaxf(a, 0.0f) : sigmoidf_(a);
+        v[q] += bias_s[lb + q];
+        x[q] = g.act == VQMC_ACT_RELU ? fmaxf(v[q], 0.0f) : sigmoidf_(v[q]);
+      }
+      if (g.pre) {
+        float* p = g.pre + (size_t)m * g.ldpre + nb;
+        if (full && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) reinterpret_cast<float4*>(p)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        } else if (mvalid) {
+#pragma unroll
+          for (int q = 0; q < 16; ++q)
+            if (nb + q < g.N) p[q] = v[q];
+        }
       }
       if (full) {
         store16_bf16(g.out + (size_t)m * g.ldo + nb, x);

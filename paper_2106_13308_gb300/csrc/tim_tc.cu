@@ -28,8 +28,8 @@
 // instructions for each of the B n n / 2 outputs that do not cancel (164 M of
 // them at n = 500, B = 1024: 60 us of issue slots).  Measured there, h = 193
 // (GB300), a training step: 1141 us with the rows and their spins written to
-// memory and read back by the general GEMM, 446 us with this kernel (0.21 ms
-// of it; 156 M warp instructions, 64% of the issue slots).
+// memory and read back by the general GEMM, 430 us with this kernel (0.21 ms
+// of it; 145 M warp instructions, 61% of the issue slots).
 #include <algorithm>
 
 #include "gemm.cuh"

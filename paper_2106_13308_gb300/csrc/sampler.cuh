@@ -57,6 +57,7 @@ __device__ __forceinline__ float to_unit(uint32_t x) { return (float)(x >> 8) * 
 // logit(u) = log(u / (1 - u)); -inf at u = 0.  u < sigma(z) iff z > logit(u).
 __device__ __forceinline__ float logit(float u) { return logf(u) - log1pf(-u); }
 
+// log sigma(x) without overflow.
 __device__ __forceinline__ float log_sigmoid(float x) {
   return x >= 0.0f ? -log1pf(expf(-x)) : x - log1pf(expf(x));
 }

@@ -25,8 +25,8 @@
 // timeout bit and runs on without waiting.
 //
 // What bounds it: the epilogue, one exponential, one logarithm and some 11 more
-// instructions for each of the B n n / 2 outputs that do not cancel (164 M of
-// them at n = 500, B = 1024: 60 us of issue slots).  Measured there, h = 193
+// instructions for each of the B n n / 2 outputs that do not cancel (185 M of
+// them at n = 500, B = 1024: 65 us of issue slots).  Measured there, h = 193
 // (GB300), a training step: 1141 us with the rows and their spins written to
 // memory and read back by the general GEMM, 430 us with this kernel (0.21 ms
 // of it; 145 M warp instructions, 61% of the issue slots).

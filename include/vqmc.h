@@ -78,9 +78,10 @@ enum { VQMC_PREC_FP32 = 0, VQMC_PREC_BF16 = 1 };
 /* Sampler implementation (vqmc_config.sampler).  All draw the same exact
  * samples of the model (Algorithm 1) from the same uniforms.
  *   AUTO: TENSOR_CORE where it applies, else CUDA_CORE.
- *   CUDA_CORE: FP32 FMAs on the CUDA cores, in blocks of up to 16 steps; any
- *     model with h <= 5120 (BF16 weights) or h <= 2816 (FP32 weights).  A CTA
- *     carries 8 samples.
+ *   CUDA_CORE: FP32 FMAs on the CUDA cores, any model with h <= 5120 (BF16
+ *     weights) or h <= 2816 (FP32 weights), in blocks of up to 16 steps or, where
+ *     many units complete at a step or a small model has a large batch, step by
+ *     step: the two differ in speed alone, not in any bit.
  *   CUDA_CORE_WIDE: the CUDA-core sampler with the summation order it uses
  *     beyond h = 2048 (four runs of 64 units instead of two or one: the FP32
  *     rounding of a logit differs) at any h; the batch autotuner chooses

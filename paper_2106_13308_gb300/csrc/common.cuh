@@ -202,12 +202,15 @@ struct vqmc_ctx {
 
 namespace vqmc {
 
-// ---- sampler_bf16.cu / sampler_f32.cu: whether the CUDA-core sampler runs
-// models with hp padded hidden units and weights of type WT, in its default
-// or wide summation order
+// ---- sampler_bf16.cu / sampler_f32.cu: whether the CUDA-core samplers run
+// models with hp padded hidden units and weights of type WT
 template <typename WT>
-bool sampler_wt_supports(int hp, bool wide);
+bool sampler_wt_supports(int hp);
 // ---- sampler.cu
+// Whether launch_sampler takes the CUDA-core sampler that goes step by step
+// (sampler_steps.cuh), not the blocked one (sampler_impl.cuh): both give the same
+// bits, so this is a matter of speed alone.
+bool sampler_stepwise(int prec, int act, int n, int h, int B, bool wide, int sms);
 // boff: index of sample 0 in the Philox counter
 cudaError_t launch_uniforms(int B, int n, uint64_t seed, uint64_t iteration, float* d_u, cudaStream_t st,
                             uint32_t boff = 0);

@@ -9,6 +9,7 @@ namespace vqmc {
 struct SamplerArgs {
   int n, h, hp, B;
   int act;          // VQMC_ACT_*
+  int nst;          // ring stages of the step-at-a-time sampler
   int wide;         // 1: the summation order of hp > 2048 at any hp
   const void* wt;   // [n][hp]
   const void* v;    // [n][hp]
@@ -20,14 +21,15 @@ struct SamplerArgs {
   const unsigned long long* it_dev;  // if not null: the Philox iteration, read on the device
   int8_t* s_out;    // [B][n]
   float* logp;      // [B] or null
-  uint32_t* err;
+  uint32_t* err;    // device error word (bounded waits of the step-at-a-time sampler)
 };
 
-// Launches the sampler for weights of type WT (float or bf16).
+// Launch the samplers for weights of type WT (float or bf16): in blocks of
+// steps (sampler_impl.cuh) and step by step (sampler_steps.cuh).
 template <typename WT>
 cudaError_t launch_sampler_wt(const SamplerArgs& a, cudaStream_t st);
-
-
+template <typename WT>
+cudaError_t launch_sampler_steps_wt(const SamplerArgs& a, cudaStream_t st);
 
 namespace {
 

@@ -46,6 +46,7 @@
 
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "sampler.cuh"
 
 namespace vqmc {
@@ -62,24 +63,10 @@ constexpr int kSolvers = 2;      // warps that draw, 4 samples each: the last on
 constexpr int kThreads = 32 * kWarps;
 constexpr int kChunk = 64;       // units per chunk of the state
 
-// ---- packed FP32 pairs (fma.rn.f32x2: two IEEE FP32 FMAs in one instruction)
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
 __device__ __forceinline__ float sum2(uint64_t v) {
   float lo, hi;
   unpack2(v, lo, hi);
   return lo + hi;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
 }
 // 16 bytes from global to shared memory, asynchronously
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
@@ -701,16 +688,17 @@ cudaError_t launch_cfg(const SamplerArgs& a, cudaStream_t st) {
 // The summation order (GW) by hp; `wide` asks for the order of hp > 2048 at any hp.
 template <typename WT>
 cudaError_t launch_sampler_wt(const SamplerArgs& a, cudaStream_t st) {
-  if (!sampler_wt_supports<WT>(a.hp, a.wide)) return cudaErrorNotSupported;
+  if (!sampler_wt_supports<WT>(a.hp)) return cudaErrorNotSupported;
   if (a.wide || a.hp > 2048) return launch_cfg<WT, 4>(a, st);
   if (a.hp <= 64) return launch_cfg<WT, 1>(a, st);
   return launch_cfg<WT, 2>(a, st);
 }
 
-// Whether launch_sampler_wt<WT> runs models with hp padded hidden units.
+// Whether the CUDA-core samplers run models with hp padded hidden units: two
+// stages of the step-at-a-time sampler's weight ring have to fit the shared
+// memory.
 template <typename WT>
-bool sampler_wt_supports(int hp, bool wide) {
-  (void)wide;
+bool sampler_wt_supports(int hp) {
   return hp <= (sizeof(WT) == 2 ? 5120 : 2816);
 }
 

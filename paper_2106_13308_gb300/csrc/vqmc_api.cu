@@ -246,8 +246,7 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
   }
   if (cfg->sampler > VQMC_SAMPLER_CUDA_CORE_WIDE) return fail(VQMC_ERR_INVALID_ARG, "bad sampler");
   const bool wide = cfg->sampler == VQMC_SAMPLER_CUDA_CORE_WIDE;
-  if (!(cfg->precision == VQMC_PREC_BF16 ? sampler_wt_supports<bf16>(pad_up(h), wide)
-                                         : sampler_wt_supports<float>(pad_up(h), wide)))
+  if (!(cfg->precision == VQMC_PREC_BF16 ? sampler_wt_supports<bf16>(pad_up(h)) : sampler_wt_supports<float>(pad_up(h))))
     return fail(VQMC_ERR_UNSUPPORTED,
                 "the CUDA-core sampler supports h <= 5120 with BF16 weights and h <= 2816 with FP32 weights");
 
@@ -1190,9 +1189,7 @@ vqmc_status vqmc_batch_autotune(vqmc_batch* b, const int32_t* B, vqmc_stream str
       float f = 0.0f;
       time_alone(i, &f);
       cost[i] = f;
-      const bool other = c->sampler == VQMC_SAMPLER_CUDA_CORE && c->hp <= 2048 &&
-                         (c->prec == VQMC_PREC_BF16 ? sampler_wt_supports<bf16>(c->hp, !c->sampler_wide)
-                                                    : sampler_wt_supports<float>(c->hp, !c->sampler_wide));
+      const bool other = c->sampler == VQMC_SAMPLER_CUDA_CORE && c->hp <= 2048;
       if (s == VQMC_OK && other) {
         c->sampler_wide ^= 1;
         time_alone(i, &f);

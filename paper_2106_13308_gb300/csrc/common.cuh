@@ -175,6 +175,7 @@ struct vqmc_ctx {
   void* Dt = nullptr;      // [n][Bp]
   void* GAt = nullptr;     // [h][Bp] hidden pre-activation adjoint, transposed
   float* GA = nullptr;     // FP32: the same, [Bmax][hp]
+  float* wg_part = nullptr;  // FP32: parts of the weight gradients' split batch
   float* logp = nullptr;   // [Bmax]
   float* coef = nullptr;   // [Bmax]
   double* stats = nullptr; // [4]

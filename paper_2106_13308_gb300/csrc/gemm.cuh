@@ -53,8 +53,7 @@ struct GemmArgs {
   int ldc;
   uint32_t* err;       // device error word (bounded waits)
   int sms;             // SMs of the device (FP32: choice of the tile)
-  float* part;         // FP32 weight gradients, optional: scratch for the parts
-  size_t part_cap;     // of a split K, part_cap floats
+  float* part;         // FP32 weight gradients: scratch for the parts of a split K
   // Adam step fused into the weight-gradient epilogue (tensor-core path,
   // kOpDV / kOpDW with theta set; gout unused): theta, adam_m and adam_v
   // point at the weight block, [M][ldg]; the refreshed weights also go to
@@ -100,6 +99,10 @@ __host__ __device__ inline bool gemm_tile_masked(int op, int m0, int m1, int n0,
 cudaError_t launch_gemm_simt_f32(const GemmArgs<float>& a, cudaStream_t st);
 // rows per tile (and per column partial) of that launch
 int gemm_simt_rows(int op, int M, int N, int sms);
+// parts that the weight gradients split K into (1: none), *kpart of K in each, and
+// floats of scratch for every K up to Kmax
+int gemm_simt_parts(int M, int N, int K, int sms, int* kpart);
+size_t gemm_simt_part_floats(int M, int N, int Kmax, int sms);
 // tcgen05 path (BF16 operands, FP32 accumulation in tensor memory).
 cudaError_t launch_gemm_tc_bf16(const GemmArgs<bf16>& a, cudaStream_t st);
 bool gemm_tc_available();

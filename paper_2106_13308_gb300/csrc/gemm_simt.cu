@@ -390,20 +390,40 @@ int gemm_simt_rows(int op, int M, int N, int sms) {
   return tiles(M, N, 128, 128) >= 3ll * sms ? 128 : 64;
 }
 
+namespace {
+
+// 64 x 128 tiles: the choice between them and 64 x 64
+bool wide_tiles(int M, int N, int sms) { return 2 * tiles(M, N, 64, 128) >= 3ll * sms; }
+
+}  // namespace
+
+// The weight gradients of few tiles split K, the batch: as many parts as give four
+// CTAs per SM, of at least 64 samples each (n = 301, h = 203, 777 samples: 20 tiles,
+// 10 parts).  Sizes and the device alone decide, so that the same call gives the same
+// bits in every context; the parts take at most 16 KB for each of the four CTAs.
+int gemm_simt_parts(int M, int N, int K, int sms, int* kpart) {
+  *kpart = 0;
+  if (gemm_simt_rows(kOpDV, M, N, sms) == 128 || wide_tiles(M, N, sms)) return 1;
+  const long long want = std::min(4ll * sms / tiles(M, N, 64, 64), (long long)K / 64);
+  if (want <= 1) return 1;
+  *kpart = ((K + (int)want - 1) / (int)want + BK - 1) / BK * BK;
+  return (K + *kpart - 1) / *kpart;
+}
+
+size_t gemm_simt_part_floats(int M, int N, int Kmax, int sms) {
+  int kpart;
+  if (gemm_simt_parts(M, N, Kmax, sms, &kpart) <= 1) return 0;
+  // rounding the parts up to steps of K only lowers their number
+  return (size_t)std::min(4ll * sms / tiles(M, N, 64, 64), (long long)Kmax / 64) * M * N;
+}
+
 cudaError_t launch_gemm_simt_f32(const GemmArgs<float>& a, cudaStream_t st) {
   if (a.M <= 0 || a.N <= 0) return cudaSuccess;
   const int sms = a.sms > 0 ? a.sms : 1;
   if (gemm_simt_rows(a.op, a.M, a.N, sms) == 128) return launch_tile<8, 8>(a, 1, 0, st);
-  if (a.op == kOpOut || a.op == kOpEloc || 2 * tiles(a.M, a.N, 64, 128) >= 3ll * sms) return launch_tile<4, 8>(a, 1, 0, st);
-  // few tiles: the weight gradients (K = the batch) also split K, as far as
-  // the scratch for the parts goes and with at least 64 samples each
+  if (a.op == kOpOut || a.op == kOpEloc || wide_tiles(a.M, a.N, sms)) return launch_tile<4, 8>(a, 1, 0, st);
   int parts = 1, kpart = 0;
-  if ((a.op == kOpDV || a.op == kOpDW) && a.part) {
-    const long long want = 4ll * sms / tiles(a.M, a.N, 64, 64), cap = (long long)(a.part_cap / ((size_t)a.M * a.N));
-    parts = (int)std::max(1ll, std::min({want, cap, (long long)a.K / 64}));
-    kpart = ((a.K + parts - 1) / parts + BK - 1) / BK * BK;
-    parts = (a.K + kpart - 1) / kpart;
-  }
+  if (a.op == kOpDV || a.op == kOpDW) parts = gemm_simt_parts(a.M, a.N, a.K, sms, &kpart);
   return launch_tile<4, 4>(a, parts, kpart, st);
 }
 

@@ -78,9 +78,7 @@ GemmArgs<T> make_args(const vqmc_ctx* c, GemmOp op, int B, const int8_t* d_s, co
   a.ldc = c->col_part_ld;
   a.err = c->err;
   a.sms = c->num_sms;
-  // FP32: the output adjoint's row-major copy D is read by the hidden adjoint
-  // alone, so the weight gradients after it have it for the parts of a split K
-  if (c->prec == VQMC_PREC_FP32) a.part = (float*)c->D, a.part_cap = (size_t)c->Bmax * c->np;
+  a.part = c->wg_part;
   const int n = c->n, h = c->h;
   switch (op) {
     case kOpHidden:
@@ -302,7 +300,10 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
   VQ_ALLOC(c->D, (size_t)Bmax * c->np * es);
   VQ_ALLOC(c->Dt, (size_t)n * c->Bp * es);
   VQ_ALLOC(c->GAt, (size_t)h * c->Bp * es);
-  if (c->prec == VQMC_PREC_FP32) VQ_ALLOC(c->GA, (size_t)Bmax * c->hp * es);
+  if (c->prec == VQMC_PREC_FP32) {
+    VQ_ALLOC(c->GA, (size_t)Bmax * c->hp * es);
+    VQ_ALLOC(c->wg_part, gemm_simt_part_floats(n, h, Bmax, c->num_sms) * 4);
+  }
   VQ_ALLOC(c->logp, (size_t)Bmax * 4);
   VQ_ALLOC(c->coef, (size_t)Bmax * 4);
   VQ_ALLOC(c->ones, (size_t)Bmax * 4);
@@ -437,7 +438,7 @@ void vqmc_destroy(vqmc_ctx* c) {
   }
   void* ptrs[] = {c->theta, c->adam_m, c->adam_v, c->grad, c->wt_s, c->v_s, c->w_s, c->vt_s, c->row_ptr,
                   c->col, c->w, c->field, c->J, c->J_hi, c->J_lo, c->S, c->E, c->Sx, c->St, c->H, c->Ht,
-                  c->D, c->Dt, c->GAt, c->GA, c->logp, c->coef, c->stats, c->row_part, c->col_part, c->err,
+                  c->D, c->Dt, c->GAt, c->GA, c->wg_part, c->logp, c->coef, c->stats, c->row_part, c->col_part, c->err,
                   c->step_stats, c->Sbits, c->eloc_part, c->eloc_slice, c->erow, c->alpha, c->tim_A,
                   c->tim_S8, c->tim_H, c->tim_row_part, c->tim_part, c->sr_A, c->sr_x, c->sr_ones, c->sr_xinv,
                   c->sr_events, c->dstate, c->ones};

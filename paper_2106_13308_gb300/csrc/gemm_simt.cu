@@ -353,7 +353,8 @@ template <int OP, int TM, int TN>
 cudaError_t launch_op(const GemmArgs<float>& a, int parts, int kpart, cudaStream_t st) {
   using T = Tile<TM, TN>;
   auto kern = gemm_simt_kernel<OP, TM, TN>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmem);
+  static OncePerDevice smem;
+  const cudaError_t e = allow_smem(smem, std::initializer_list<decltype(kern)>{kern}, T::kSmem);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.N + T::BN - 1) / T::BN, (a.M + T::BM - 1) / T::BM, parts);
   kern<<<grid, kThreads, T::kSmem, st>>>(a, kpart);

@@ -568,32 +568,40 @@ __global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 std::once_flag g_once;
-bool g_have_tc = false;
+OncePerDevice g_device;
 
-void init_once() {
-  cudaDriverEntryPointQueryResult q;
-  void* fn = nullptr;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-      q == cudaDriverEntryPointSuccess && fn) {
-    g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  }
-  int dev = 0, major = 0, minor = 0;
-  cudaGetDevice(&dev);
+bool have_encode() {
+  std::call_once(g_once, [] {
+    cudaDriverEntryPointQueryResult q;
+    void* fn = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess && fn)
+      g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+  });
+  return g_encode != nullptr;
+}
+
+// Whether `dev` runs the tcgen05 kernels, with their shared-memory limits set.
+cudaError_t set_up_device(int dev) {
+  int major = 0, minor = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
-  g_have_tc = g_encode != nullptr && major == 10 && minor == 3;
+  if (major != 10 || minor != 3) return cudaErrorNotSupported;
   const void* k1[] = {(const void*)gemm_tc_kernel<kOpHidden, 1>, (const void*)gemm_tc_kernel<kOpOut, 1>,
                       (const void*)gemm_tc_kernel<kOpDV, 1>,     (const void*)gemm_tc_kernel<kOpGA, 1>,
                       (const void*)gemm_tc_kernel<kOpDW, 1>,     (const void*)gemm_tc_kernel<kOpEloc, 1>};
   const void* k2[] = {(const void*)gemm_tc_kernel<kOpHidden, 2>, (const void*)gemm_tc_kernel<kOpOut, 2>,
                       (const void*)gemm_tc_kernel<kOpDV, 2>,     (const void*)gemm_tc_kernel<kOpGA, 2>,
                       (const void*)gemm_tc_kernel<kOpDW, 2>,     (const void*)gemm_tc_kernel<kOpEloc, 2>};
-  for (const void* k : k1)
-    if (g_have_tc && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Stages<1>::kSmem) != cudaSuccess)
-      g_have_tc = false;
-  for (const void* k : k2)
-    if (g_have_tc && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Stages<2>::kSmem) != cudaSuccess)
-      g_have_tc = false;
+  for (const void* k : k1) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Stages<1>::kSmem);
+    if (e != cudaSuccess) return e;
+  }
+  for (const void* k : k2) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Stages<2>::kSmem);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 bool encode(CUtensorMap* map, const void* ptr, int rows, int cols, int ld) {
@@ -603,7 +611,7 @@ bool encode(CUtensorMap* map, const void* ptr, int rows, int cols, int ld) {
 }  // namespace
 
 bool tc_encode_bf16(CUtensorMap* map, const void* ptr, int rows, int cols, int ld, int box_rows) {
-  if (!gemm_tc_available()) return false;
+  if (!have_encode()) return false;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
   cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
@@ -616,7 +624,7 @@ bool tc_encode_bf16(CUtensorMap* map, const void* ptr, int rows, int cols, int l
 
 bool tc_encode_bf16_chunks(CUtensorMap* map, const void* ptr, int rows, int cols, int ld, int box_rows,
                            int box_chunks) {
-  if (!gemm_tc_available() || cols % BK || box_chunks < 1 || box_chunks > 8) return false;
+  if (!have_encode() || cols % BK || box_chunks < 1 || box_chunks > 8) return false;
   // chunk c of row r starts at element r * ld + 64 c: the view covers
   // exactly the rows x cols elements of the 2D matrix
   cuuint64_t dims[3] = {(cuuint64_t)BK, (cuuint64_t)rows, (cuuint64_t)(cols / BK)};
@@ -630,8 +638,8 @@ bool tc_encode_bf16_chunks(CUtensorMap* map, const void* ptr, int rows, int cols
 }
 
 bool gemm_tc_available() {
-  std::call_once(g_once, init_once);
-  return g_have_tc;
+  int dev = -1;
+  return have_encode() && cudaGetDevice(&dev) == cudaSuccess && g_device(dev, [&] { return set_up_device(dev); }) == cudaSuccess;
 }
 
 cudaError_t launch_gemm_tc_bf16(const GemmArgs<bf16>& a, cudaStream_t st) {

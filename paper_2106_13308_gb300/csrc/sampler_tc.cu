@@ -939,7 +939,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-bool g_attr_set = false;
+OncePerDevice g_smem;
 
 // largest number of units completing inside one block of D steps
 int max_recent(int n, int h, int D) {
@@ -977,17 +977,10 @@ cudaError_t launch_sampler_tc(const vqmc_ctx* c, int B, const float* d_u, uint64
       !tc_encode_bf16_chunks(&mapW2, c->w_s, c->h, c->np, c->np, 128, 2))
     return cudaErrorInvalidValue;
   using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcArgs);
-  constexpr Kernel kernels[2][2] = {
-      {sampler_tc_kernel<VQMC_ACT_RELU, false>, sampler_tc_kernel<VQMC_ACT_RELU, true>},
-      {sampler_tc_kernel<VQMC_ACT_SIGMOID, false>, sampler_tc_kernel<VQMC_ACT_SIGMOID, true>}};
-  if (!g_attr_set) {
-    for (const auto& row : kernels)
-      for (Kernel k : row) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-      }
-    g_attr_set = true;
-  }
+  constexpr Kernel kernels[] = {sampler_tc_kernel<VQMC_ACT_RELU, false>, sampler_tc_kernel<VQMC_ACT_RELU, true>,
+                                sampler_tc_kernel<VQMC_ACT_SIGMOID, false>, sampler_tc_kernel<VQMC_ACT_SIGMOID, true>};
+  const cudaError_t e = allow_smem(g_smem, kernels, kSmemBytes);
+  if (e != cudaSuccess) return e;
   TcArgs a;
   a.n = c->n;
   a.h = c->h;
@@ -1014,7 +1007,7 @@ cudaError_t launch_sampler_tc(const vqmc_ctx* c, int B, const float* d_u, uint64
   a.stt = reinterpret_cast<bf16*>(stt);
   a.ldst = c->Bp;
   a.sbits = reinterpret_cast<uint16_t*>(sbits);
-  const Kernel kernel = kernels[c->act == VQMC_ACT_RELU ? 0 : 1][d_logp != nullptr];
+  const Kernel kernel = kernels[(c->act == VQMC_ACT_RELU ? 0 : 2) + (d_logp != nullptr)];
   kernel<<<(B + kS - 1) / kS, kThreads, kSmemBytes, st>>>(mapV, mapW, mapV2, mapV3, mapW2, a);
   return cudaGetLastError();
 }

@@ -365,7 +365,7 @@ int stages_of(int hp) {
   return std::min(kMaxStages, a < 113 * 1024 && two >= 2 ? two : one);
 }
 
-bool g_attr_set = false;
+OncePerDevice g_smem;
 
 }  // namespace
 
@@ -389,18 +389,14 @@ cudaError_t launch_tim_tc(const vqmc_ctx* c, int B, const int8_t* d_s, float* d_
   a.part = (double*)c->tim_part;
   a.err = c->err;
   const int smem = 1024 + (c->hp / 64 + a.stages) * kTileBytes + kMisc;
-  if (!g_attr_set) {
-    for (auto k : {tim_fused_kernel<VQMC_ACT_RELU>, tim_fused_kernel<VQMC_ACT_SIGMOID>}) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      if (e != cudaSuccess) return e;
-    }
-    g_attr_set = true;
-  }
+  const auto kernels = {tim_fused_kernel<VQMC_ACT_RELU>, tim_fused_kernel<VQMC_ACT_SIGMOID>};
+  cudaError_t e = allow_smem(g_smem, kernels, 227 * 1024);
+  if (e != cudaSuccess) return e;
   const long long resident = (long long)c->num_sms * (smem <= 113 * 1024 ? 2 : 1);
   const int grid = (int)std::min(a.tiles, resident);
   if (c->act == VQMC_ACT_RELU) tim_fused_kernel<VQMC_ACT_RELU><<<grid, kThreads, smem, st>>>(mapV, a);
   else tim_fused_kernel<VQMC_ACT_SIGMOID><<<grid, kThreads, smem, st>>>(mapV, a);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   tim_finish_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, blocks, a.part, d_e);
   if (launches) *launches += 2;

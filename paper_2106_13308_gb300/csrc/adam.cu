@@ -83,7 +83,7 @@ __device__ __forceinline__ bool tile_masked(int z, int r0, int nr, int k0, int n
 // kernel-side copies.  Grid (h/32, n/32, 2): z = 0 for W1^T, z = 1 for W2;
 // each 32 x 32 tile is updated with coalesced accesses along k, written to
 // the row copy (wt_s shifted by one row, v_s), and through shared memory to
-// the transposed copy (w_s, vt_s).  Only entries inside the MADE masks are
+// the transposed copy (w_s, vt_s), each where the context has it.  Only entries inside the MADE masks are
 // updated (fully masked tiles return at once), so the masked weights stay
 // zero whatever the gradient holds there.  Padding of the copies is never
 // written (zero since allocation).
@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(256) adam_refresh_kernel(int n, int h, int hp,
   }
   __syncthreads();
   T* dst = z == 0 ? w_s : vt_s;
+  if (!dst) return;
   for (int kk = ty; kk < 32; kk += 8) {
     const int k = k0 + kk, r = r0 + tx;
     if (k < h && r < n && kept(z, r, k, n, h)) dst[(long long)k * np + r] = cvt<T>(tile[tx][kk]);
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(256) adam_refresh4_kernel(int n, int h, int hp
   }
   __syncthreads();
   T* dst = z == 0 ? w_s : vt_s;
+  if (!dst) return;
   for (int kk = ty; kk < 128; kk += 8) {
     const int kq = k0 + kk, r = r0 + tx;
     if (kq < h && r < n && kept(z, r, kq, n, h)) dst[(long long)kq * np + r] = cvt<T>(tile[tx][kk]);
@@ -269,7 +271,7 @@ cudaError_t refresh(vqmc_ctx* c, cudaStream_t st) {
   rows_kernel<T><<<grid_for(c, (long long)rows * c->hp), 256, 0, st>>>(c->n, c->h, c->hp, rows, c->theta, (T*)c->wt_s,
                                                                     (T*)c->v_s);
   dim3 grid((c->np + 31) / 32, (c->h + 31) / 32), block(32, 8);
-  transpose_kernel<T><<<grid, block, 0, st>>>(c->n, c->h, c->np, c->theta, (T*)c->w_s);
+  if (c->w_s) transpose_kernel<T><<<grid, block, 0, st>>>(c->n, c->h, c->np, c->theta, (T*)c->w_s);
   transpose_kernel<T><<<grid, block, 0, st>>>(c->n, c->h, c->np, c->theta + (long long)c->n * c->h + c->h,
                                                (T*)c->vt_s);
   return cudaGetLastError();

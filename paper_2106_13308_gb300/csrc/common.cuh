@@ -146,8 +146,10 @@ struct vqmc_ctx {
   //                               row 0 and rows > n zero; sampler
   //   v_s  [sampler_rows(n)][hp]  row i = row i of W2 (output i+1), rows >= n
   //                               zero; sampler and Z GEMM
-  //   w_s  [h][np]  rows of W1 (unit k <- all inputs), hidden GEMM
-  //   vt_s [h][np]  rows of W2^T (unit k -> all outputs), backward GEMM
+  //   w_s  [h][np]  rows of W1 (unit k <- all inputs): BF16 only, hidden GEMM and
+  //                 tensor-core sampler (the FP32 hidden GEMM reads wt_s)
+  //   vt_s [h][np]  rows of W2^T (unit k -> all outputs): BF16 hidden adjoint,
+  //                 FP32 output GEMM (BF16: v_s, which the FP32 adjoint reads)
   void* wt_s = nullptr;
   void* v_s = nullptr;
   void* w_s = nullptr;
@@ -188,10 +190,10 @@ struct vqmc_ctx {
   void* Sx = nullptr;      // [Bmax][np] spins as GEMM operand
   void* St = nullptr;      // [n][Bp] spins transposed
   void* H = nullptr;       // [Bmax][hp] hidden activations
-  void* Ht = nullptr;      // [h][Bp]
+  void* Ht = nullptr;      // [h][Bp]; FP32: with the SR workspace
   void* D = nullptr;       // [Bmax][np] output adjoint delta
   void* Dt = nullptr;      // [n][Bp]
-  void* GAt = nullptr;     // [h][Bp] hidden pre-activation adjoint, transposed
+  void* GAt = nullptr;     // [h][Bp] hidden pre-activation adjoint, transposed; FP32: with the SR workspace
   float* GA = nullptr;     // FP32: the same, [Bmax][hp]
   float* wg_part = nullptr;  // FP32: parts of the weight gradients' split batch
   float* logp = nullptr;   // [Bmax]
@@ -211,7 +213,7 @@ struct vqmc_ctx {
   // Cholesky workspace [sr_ld][sr_ld] (lower triangle), its solution, a
   // vector of ones [sr_ld] (unit coefficients of the per-sample pass), the
   // inverse-transposed diagonal blocks of the factor [sr_ld / 64][64][64],
-  // and the Gram kernel's event order [n + h]
+  // and the Gram kernel's event order [n + h]; with them Ht and GAt
   float* sr_A = nullptr;
   float* sr_x = nullptr;
   float* sr_ones = nullptr;
@@ -281,19 +283,20 @@ cudaError_t launch_col_sum(const vqmc_ctx* c, int N, int mtiles, float* out, cud
 enum GemmOp {
   kOpHidden = 0,  // H = act(S W1^T + b1); writes H, Ht
   kOpOut = 1,     // Z = H W2^T + b2; logp row partials; if coef: delta, Dt, dc partials
-  kOpDV = 2,      // dW2 = Dt . Ht^T  (masked) -> grad, or the Adam step on W2
-  kOpGA = 3,      // G = D . W2 ; GA = G * act'(H) -> GAt ; db1 partials
-  kOpDW = 4,      // dW1^T = St . GAt^T (masked) -> grad, or the Adam step on W1^T
+  kOpDV = 2,      // dW2 = Dt . H  (masked) -> grad, or the Adam step on W2; BF16 reads Ht, FP32 H
+  kOpGA = 3,      // G = D . W2 ; GA = G * act'(H) -> GAt, FP32 GA ; db1 partials
+  kOpDW = 4,      // dW1^T = St . GA (masked) -> grad, or the Adam step on W1^T; BF16 reads GAt, FP32 GA
   kOpEloc = 5     // T = S J (hi/lo) ; row partials 1/2 s.T
 };
 // Adam factors of one step for the weight-gradient GEMMs that apply the step
 // in their epilogue: device pointer to {1 / (1 - beta1^t), 1 / (1 - beta2^t)}
-// (the context's DevState).
+// (the context's DevState).  transposed: an FP32 hidden GEMM or adjoint also
+// writes Ht or GAt, which the Gram kernel alone reads there (BF16: always).
 struct AdamStep {
   const float* ibc;
 };
 cudaError_t launch_gemm(const vqmc_ctx* c, GemmOp op, int B, const int8_t* d_s, const float* coef,
-                        float* grad, cudaStream_t st, const AdamStep* fuse = nullptr);
+                        float* grad, cudaStream_t st, const AdamStep* fuse = nullptr, bool transposed = false);
 
 // ---- vqmc_api.cu: sets the thread-local message of vqmc_last_error
 vqmc_status set_last_error(vqmc_status s, const std::string& msg);

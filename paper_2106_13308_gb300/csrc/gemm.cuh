@@ -32,7 +32,7 @@ struct GemmArgs {
   const float* coef;   // [M] or null
   T* out;              // row-major [M][ldo]
   int ldo;
-  T* out_t;            // transposed [N][ldt] (kOpHidden: optional)
+  T* out_t;            // transposed [N][ldt] (kOpHidden, FP32 also kOpGA: optional)
   int ldt;
   float* pre;          // kOpHidden, optional: FP32 pre-activations a = S W1^T + b1, [M][ldpre]
   int ldpre;

@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
       for (int j = 0; j < 4; ++j) t[j][i] = x[j];
     }
     if constexpr (op == kOpHidden || op == kOpOut || op == kOpGA)
-      if (op == kOpGA || (op == kOpHidden && g.out_t) || (op == kOpOut && g.coef))
+      if (g.out_t && (op != kOpOut || g.coef))
 #pragma unroll
         for (int j = 0; j < 4; ++j) store_t(nn + j, t[j]);
   }

@@ -415,6 +415,9 @@ cudaError_t sr_workspace(vqmc_ctx* c) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->sr_x, N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->sr_ones, N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->sr_xinv, N * kNB * sizeof(float));
+  const size_t ht = (size_t)c->h * c->Bp * sizeof(float);
+  if (e == cudaSuccess) e = cudaMalloc(&c->Ht, ht);
+  if (e == cudaSuccess) e = cudaMalloc(&c->GAt, ht);
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->sr_events, ev.size() * sizeof(int));
   if (e == cudaSuccess) e = cudaMemcpy(c->sr_events, ev.data(), ev.size() * sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
@@ -427,8 +430,10 @@ cudaError_t sr_workspace(vqmc_ctx* c) {
                              (int)solve_smem(sr_blocks(kSrMaxBatch)));
   if (e != cudaSuccess) {
     cudaFree(c->sr_A), cudaFree(c->sr_x), cudaFree(c->sr_ones), cudaFree(c->sr_xinv), cudaFree(c->sr_events);
+    cudaFree(c->Ht), cudaFree(c->GAt);
     c->sr_A = c->sr_x = c->sr_ones = c->sr_xinv = nullptr;
     c->sr_events = nullptr;
+    c->Ht = c->GAt = nullptr;
   }
   return e;
 }

@@ -139,7 +139,7 @@ namespace vqmc {
 vqmc_status set_last_error(vqmc_status s, const std::string& msg) { return fail(s, msg); }
 
 cudaError_t launch_gemm(const vqmc_ctx* c, GemmOp op, int B, const int8_t* d_s, const float* coef, float* grad,
-                        cudaStream_t st, const AdamStep* fuse) {
+                        cudaStream_t st, const AdamStep* fuse, bool transposed) {
   if (c->prec == VQMC_PREC_BF16) {
     GemmArgs<bf16> a = make_args<bf16>(c, op, B, d_s, coef, grad);
     if (op == kOpEloc) a.Bm = (const bf16*)c->J_hi, a.Bm2 = (const bf16*)c->J_lo;
@@ -163,10 +163,16 @@ cudaError_t launch_gemm(const vqmc_ctx* c, GemmOp op, int B, const int8_t* d_s, 
   GemmArgs<float> a = make_args<float>(c, op, B, d_s, coef, grad);
   // the CUDA-core GEMM reads its second operand in [K][N] form
   switch (op) {
-    case kOpHidden: a.Bm = (const float*)c->wt_s + c->hp, a.ldb = c->hp; break;  // row j = input j
+    case kOpHidden:  // row j = input j
+      a.Bm = (const float*)c->wt_s + c->hp, a.ldb = c->hp;
+      if (!transposed) a.out_t = nullptr;
+      break;
     case kOpOut: a.Bm = (const float*)c->vt_s, a.ldb = c->np; break;
     case kOpDV: a.Bm = (const float*)c->H, a.ldb = c->hp; break;
-    case kOpGA: a.Bm = (const float*)c->v_s, a.ldb = c->hp, a.out = c->GA, a.ldo = c->hp; break;
+    case kOpGA:
+      a.Bm = (const float*)c->v_s, a.ldb = c->hp, a.out = c->GA, a.ldo = c->hp;
+      if (!transposed) a.out_t = nullptr;
+      break;
     case kOpDW: a.Bm = c->GA, a.ldb = c->hp; break;
     case kOpEloc: a.Bm = c->J; break;  // symmetric
   }
@@ -183,7 +189,7 @@ namespace {
 // With fuse set (BF16), the two weight-gradient GEMMs apply that Adam step
 // to W2 and W1^T in their epilogues instead of writing dW2 and dW1^T; both
 // run after every GEMM that reads the old weights (hidden adjoint: W2).
-// With hidden_done, H and Ht already hold this batch's hidden activations.
+// With hidden_done, H (and Ht) already hold this batch's hidden activations.
 vqmc_status backward_from_operands(vqmc_ctx* c, int B, const int8_t* d_s, const float* gout, float* grad,
                                    cudaStream_t st, const AdamStep* fuse = nullptr, bool hidden_done = false) {
   const int n = c->n, h = c->h;
@@ -288,7 +294,7 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
   c->b2 = c->theta + (size_t)2 * n * h + h;
   VQ_ALLOC(c->wt_s, (size_t)sampler_rows(n) * c->hp * es);
   VQ_ALLOC(c->v_s, (size_t)sampler_rows(n) * c->hp * es);
-  VQ_ALLOC(c->w_s, (size_t)h * c->np * es);
+  if (c->prec == VQMC_PREC_BF16) VQ_ALLOC(c->w_s, (size_t)h * c->np * es);
   VQ_ALLOC(c->vt_s, (size_t)h * c->np * es);
 
   VQ_ALLOC(c->S, (size_t)Bmax * n);
@@ -296,11 +302,12 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
   VQ_ALLOC(c->Sx, (size_t)Bmax * c->np * es);
   VQ_ALLOC(c->St, (size_t)n * c->Bp * es);
   VQ_ALLOC(c->H, (size_t)Bmax * c->hp * es);
-  VQ_ALLOC(c->Ht, (size_t)h * c->Bp * es);
   VQ_ALLOC(c->D, (size_t)Bmax * c->np * es);
   VQ_ALLOC(c->Dt, (size_t)n * c->Bp * es);
-  VQ_ALLOC(c->GAt, (size_t)h * c->Bp * es);
-  if (c->prec == VQMC_PREC_FP32) {
+  if (c->prec == VQMC_PREC_BF16) {
+    VQ_ALLOC(c->Ht, (size_t)h * c->Bp * es);
+    VQ_ALLOC(c->GAt, (size_t)h * c->Bp * es);
+  } else {
     VQ_ALLOC(c->GA, (size_t)Bmax * c->hp * es);
     VQ_ALLOC(c->wg_part, gemm_simt_part_floats(n, h, Bmax, c->num_sms) * 4);
   }
@@ -826,9 +833,9 @@ vqmc_status sr_check(vqmc_ctx* c, int B) {
 // each sample's s, delta, H and GA (Sec. 2.3 chain rule).
 vqmc_status sr_operands(vqmc_ctx* c, int B, const int8_t* d_s, cudaStream_t st) {
   VQ_CUDA(launch_spins_to_operands(c, B, d_s, c->Sx, c->St, st));
-  VQ_CUDA(launch_gemm(c, kOpHidden, B, d_s, nullptr, nullptr, st));
+  VQ_CUDA(launch_gemm(c, kOpHidden, B, d_s, nullptr, nullptr, st, nullptr, /*transposed=*/true));
   VQ_CUDA(launch_gemm(c, kOpOut, B, d_s, c->sr_ones, nullptr, st));
-  VQ_CUDA(launch_gemm(c, kOpGA, B, d_s, nullptr, nullptr, st));
+  VQ_CUDA(launch_gemm(c, kOpGA, B, d_s, nullptr, nullptr, st, nullptr, /*transposed=*/true));
   return VQMC_OK;
 }
 

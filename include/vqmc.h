@@ -84,8 +84,8 @@ enum { VQMC_PREC_FP32 = 0, VQMC_PREC_BF16 = 1 };
  *     step: the two differ in speed alone, not in any bit.
  *   CUDA_CORE_WIDE: the CUDA-core sampler with the summation order it uses
  *     beyond h = 2048 (four runs of 64 units instead of two or one: the FP32
- *     rounding of a logit differs) at any h; the batch autotuner chooses
- *     between the two per member.
+ *     rounding of a logit differs) at any h; the batch autotuner takes it for
+ *     a member where it goes step by step and is the faster one.
  *   TENSOR_CORE: blocks of 64 or 128 steps whose bulk work (the logits from
  *     hidden units completed before the block, and the update of hidden
  *     units by the block's spins) runs as tcgen05 GEMMs, with a sequential
@@ -413,8 +413,8 @@ vqmc_status vqmc_batch_graph_launch(vqmc_batch* batch, vqmc_stream stream, vqmc_
 
 /* Autotuner of the batch's schedule.  First it measures one iteration of
  * each member alone; a member on the CUDA-core sampler with at most 2048
- * hidden units is timed in both of its summation orders (its own, and that of
- * VQMC_SAMPLER_CUDA_CORE_WIDE) and keeps the faster.  Then it
+ * hidden units takes the order of VQMC_SAMPLER_CUDA_CORE, or, where that of
+ * VQMC_SAMPLER_CUDA_CORE_WIDE goes step by step, the faster of the two.  Then it
  * times one captured batched iteration (graph replays) under each candidate
  * schedule -- 1, 2, 4, ... up to the batch's internal streams, with members
  * assigned round-robin in index order or longest first onto the

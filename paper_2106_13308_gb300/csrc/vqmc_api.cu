@@ -1174,9 +1174,12 @@ vqmc_status vqmc_batch_autotune(vqmc_batch* b, const int32_t* B, vqmc_stream str
   if (!stream) return fail(VQMC_ERR_INVALID_ARG, "autotuning captures graphs: pass a non-default stream");
   cudaStream_t st = S(stream);
   const size_t m = b->members.size();
-  // 1. cost of one iteration of each member alone (after one warm-up step),
-  // and for a member on the CUDA-core sampler up to 2048 hidden units the
-  // faster of its two summation orders
+  // 1. cost of one iteration of each member alone (after one warm-up step).  For a
+  // member on the CUDA-core sampler up to 2048 hidden units also the choice of its
+  // summation order: its own, unless the wide one is a kernel of another shape (it
+  // goes step by step) and is the faster of the two.  In blocks of steps the wide
+  // order is the slower one (1.15 times in the median of 1,676 sizes, nowhere faster by
+  // 1%), and a timing of near-equal forms would let noise choose the rounding.
   std::vector<double> cost(m, 0.0);
   {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1194,10 +1197,12 @@ vqmc_status vqmc_batch_autotune(vqmc_batch* b, const int32_t* B, vqmc_stream str
     };
     for (size_t i = 0; i < m && s == VQMC_OK; ++i) {
       vqmc_ctx* c = b->members[i];
+      const bool two = c->sampler == VQMC_SAMPLER_CUDA_CORE && c->hp <= 2048;
+      const bool other = two && sampler_stepwise(c->prec, c->act, c->n, c->h, B[i], /*wide=*/true, c->num_sms);
+      if (two && !other) c->sampler_wide = 0;
       float f = 0.0f;
       time_alone(i, &f);
       cost[i] = f;
-      const bool other = c->sampler == VQMC_SAMPLER_CUDA_CORE && c->hp <= 2048;
       if (s == VQMC_OK && other) {
         c->sampler_wide ^= 1;
         time_alone(i, &f);

@@ -578,8 +578,9 @@ class VQMCBatch:
         _check(_lib.vqmc_batch_graph_launch(self.handle, _stream(stream), out))
 
     def autotune(self, B, stream=None):
-        """Chooses each member's sampler layout (timed alone) and the schedule
-        (streams, member assignment) by timing graph replays; returns
+        """Chooses each member's order of the CUDA-core sampler's sums (timed alone
+        where the wide one goes step by step) and the schedule (streams, member
+        assignment) by timing graph replays; returns
         (streams, ms per batched iteration)."""
         s, ms = ctypes.c_int32(), ctypes.c_double()
         _check(_lib.vqmc_batch_autotune(self.handle, self._bs(B), _stream(stream), ctypes.byref(s), ctypes.byref(ms)))

@@ -175,7 +175,7 @@ struct vqmc_ctx {
   int8_t* tim_S8 = nullptr;       // [tim_rows][np] spins of the rows
   void* tim_H = nullptr;          // [tim_rows][hp] hidden activations of the rows
   float* tim_row_part = nullptr;  // [ceil(n/128)][tim_ld] partial log pi of every row per output tile
-  long long tim_ld = 0;           // Bmax (n + 1), rounded up to 4
+  long long tim_ld = 0;           // samples of the general form's largest batch times (n + 1), rounded up to 4
   void* tim_part = nullptr;       // tim_tc.cu, in place of the three before: FP64 sums of a block of flips
 
   // workspaces (element type per precision unless noted)
@@ -260,9 +260,11 @@ cudaError_t launch_eloc_dense_finish(const vqmc_ctx* c, int B, const int8_t* d_s
 cudaError_t launch_tim_offdiag(const vqmc_ctx* c, int B, const int8_t* d_s, float* d_e, cudaStream_t st,
                                int* launches = nullptr);
 // The BF16 model's one-kernel form (tim_tc.cu), after the hidden GEMM: whether
-// it takes a model of hp padded hidden units, its workspace, and the launch
+// it takes a batch of a model of hp padded hidden units, the largest batch up to
+// Bmax that it leaves to the general form (0: none), its workspace, and the launch
 // (*launches, if not null, grows by its kernels).
-bool tim_tc_applies(int prec, int hp);
+bool tim_tc_applies(int prec, int act, int n, int hp, int B, int sms);
+int tim_general_batch(int prec, int act, int n, int hp, int Bmax, int sms);
 size_t tim_tc_part_bytes(int Bmax, int n);
 cudaError_t launch_tim_tc(const vqmc_ctx* c, int B, const int8_t* d_s, float* d_e, cudaStream_t st, int* launches);
 // rows per chunk of the flipped states for at most Bmax samples (padded

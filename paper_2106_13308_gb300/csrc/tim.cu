@@ -17,8 +17,8 @@
 // flipped spin of all its rows, and the log-ratio is summed from the partials
 // of the remaining tiles (one warp per sample).
 //
-// This is the path of the FP32 model and of BF16 models too wide for the one
-// kernel of tim_tc.cu, which starts from the same a(x).
+// This is the path of the FP32 model and, where it is the faster one, of the BF16
+// model; the one kernel of tim_tc.cu starts from the same a(x).
 #include "gemm.cuh"
 
 namespace vqmc {
@@ -178,7 +178,7 @@ cudaError_t offdiag(const vqmc_ctx* c, int B, const int8_t* d_s, float* d_e, cud
   cudaError_t e = launch_spins_to_operands(c, B, d_s, c->Sx, nullptr, st);
   if (e == cudaSuccess) e = chunk_gemm<T>(c, kOpHidden, B, 0, st);
   if (e != cudaSuccess) return e;
-  if (tim_tc_applies(c->prec, c->hp)) {
+  if (tim_tc_applies(c->prec, c->act, n, c->hp, B, c->num_sms)) {
     if (launches) *launches = 2;
     return launch_tim_tc(c, B, d_s, d_e, st, launches);
   }

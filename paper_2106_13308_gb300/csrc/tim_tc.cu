@@ -367,11 +367,54 @@ int stages_of(int hp) {
 
 OncePerDevice g_smem;
 
+
+// Estimated time in us of both forms of an energy call, without what they share (the
+// model's constants, fitted on a GB300 to 5,662 sizes: n = 1 to 500, h = 10 to 640,
+// 1 to 4096 samples).  Here: rounds of resident CTAs, each with the operand of one
+// tile (a sigmoid costs three times a relu) and the average of its output tiles.
+// tim.cu: rows through memory, on the whole chip even where this kernel has few tiles,
+// and a fixed cost for its launches.
+struct Times {
+  double tile;       // us of one round
+  long long blocks;  // of flips
+  int spw, per_sm;
+  double rows;       // us per row of the general form
+};
+Times times_of(int act, int n, int hp) {
+  const int seg = seg_of(n), nt = (n + kRows - 1) / kRows, blocks = blocks_of(n);
+  double tiles = 0.0;
+  for (int j = 0; j < blocks; ++j) tiles += nt - j * seg / kRows;
+  const bool sig = act == VQMC_ACT_SIGMOID;
+  return {hp / 64 * (sig ? 3.25 : 1.12) + 5.3 * tiles / blocks, blocks, 32 / (seg + 1),
+          hp / 64 * kTileBytes + kMisc + 1024 + 2 * kTileBytes <= 113 * 1024 ? 2 : 1,
+          1e-6 * (hp * (sig ? 1.9 : 1.2) + 445.0 * nt - 0.84 * n)};
+}
+bool faster(const Times& t, int n, int B, int sms) {
+  if (n <= 2) return false;  // 1 or 2 flips for the 32 rows of a warp
+  const long long tiles = t.blocks * ((B + 4 * t.spw - 1) / (4 * t.spw)), round = (long long)t.per_sm * sms;
+  const double here = 21.2 + 0.0087 * n + t.tile * (double)((tiles + round - 1) / round);
+  return here <= 28.9 + 0.069 * n + t.rows * (double)B * (n + 1);
+}
+
 }  // namespace
 
-// The operand of hp units has to fit shared memory beside the ring; wider
-// models go through tim.cu's row workspace and the general GEMM.
-bool tim_tc_applies(int prec, int hp) { return prec == VQMC_PREC_BF16 && hp <= kMaxHp; }
+// The operand of hp units has to fit shared memory beside the ring, and the call has
+// to be faster here than through tim.cu's row workspace and the general GEMM.  The
+// estimate names the slower form, by more than 5% and 1 us, at 147 of 5,662 measured
+// sizes, by at most 23%.  What the line is for (us, here | there): n = 64, h = 640, sigmoid,
+// 1024 samples 242 | 130; n = 8, h = 640, sigmoid, 128 samples 74 | 38; n = 500, h = 192,
+// relu, 1024 samples 236 | 761.
+bool tim_tc_applies(int prec, int act, int n, int hp, int B, int sms) {
+  return prec == VQMC_PREC_BF16 && hp <= kMaxHp && faster(times_of(act, n, hp), n, B, sms);
+}
+
+int tim_general_batch(int prec, int act, int n, int hp, int Bmax, int sms) {
+  if (prec != VQMC_PREC_BF16 || hp > kMaxHp) return Bmax;
+  const Times t = times_of(act, n, hp);
+  int B = Bmax;
+  while (B > 0 && faster(t, n, B, sms)) --B;
+  return B;
+}
 
 size_t tim_tc_part_bytes(int Bmax, int n) { return (size_t)blocks_of(n) * (size_t)Bmax * sizeof(double); }
 

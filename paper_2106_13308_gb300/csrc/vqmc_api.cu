@@ -414,14 +414,15 @@ vqmc_status vqmc_create(const vqmc_config* cfg, const vqmc_instance* inst, vqmc_
       return cleanup_fail(VQMC_ERR_CUDA, "copy of alpha failed");
     hsh = fnv1a(hsh, inst->alpha, (size_t)n * 4);
     VQ_ALLOC(c->tim_A, (size_t)Bmax * c->hp * 4);
-    if (tim_tc_applies(c->prec, c->hp)) {
-      VQ_ALLOC(c->tim_part, tim_tc_part_bytes(Bmax, n));
-    } else {
-      c->tim_rows = tim_chunk_rows(Bmax, n, c->hp, c->np, (int)esize(c));
+    // rows of the general form for the batches that go there (all in FP32)
+    const int general = tim_general_batch(c->prec, c->act, n, c->hp, Bmax, c->num_sms);
+    if (c->prec == VQMC_PREC_BF16) VQ_ALLOC(c->tim_part, tim_tc_part_bytes(Bmax, n));
+    if (general > 0) {
+      c->tim_rows = tim_chunk_rows(general, n, c->hp, c->np, (int)esize(c));
       const size_t rows = (size_t)c->tim_rows;
       VQ_ALLOC(c->tim_S8, rows * c->np);
       VQ_ALLOC(c->tim_H, rows * c->hp * esize(c));
-      c->tim_ld = ((long long)Bmax * (n + 1) + 3) / 4 * 4;
+      c->tim_ld = ((long long)general * (n + 1) + 3) / 4 * 4;
       VQ_ALLOC(c->tim_row_part, (size_t)((n + 127) / 128) * (size_t)c->tim_ld * 4);
     }
   }

@@ -431,29 +431,35 @@ __device__ __forceinline__ float spin_val<float>(int8_t s) { return s > 0 ? 1.0f
 template <>
 __device__ __forceinline__ bf16 spin_val<bf16>(int8_t s) { return __float2bfloat16_rn(s > 0 ? 1.0f : -1.0f); }
 
-// 16 spins as T, with 16-byte stores where p allows it and all `cnt` are inside
+// the first cnt of 16 spins as T in 16-byte stores, zeros after the last: rows are
+// padded to multiples of 64 and start on 16-byte boundaries
+template <bool ALL, typename T>
+__device__ __forceinline__ void store_spins16(T* p, const uint32_t (&w)[4], int cnt) {
+  constexpr int kPer = 16 / sizeof(T);
+#pragma unroll
+  for (int v = 0; v < 16 / kPer; ++v) {
+    if (!ALL && kPer * v >= cnt) break;
+    __align__(16) T x[kPer];
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      const int q = kPer * v + e;
+      x[e] = ALL || q < cnt ? spin_val<T>((int8_t)(w[q >> 2] >> (8 * (q & 3)))) : T(0.0f);
+    }
+    reinterpret_cast<uint4*>(p)[v] = *reinterpret_cast<const uint4*>(x);
+  }
+}
 template <typename T>
 __device__ __forceinline__ void store_spins(T* p, const uint32_t (&w)[4], int cnt) {
-  auto spin = [&](int q) { return spin_val<T>((int8_t)(w[q >> 2] >> (8 * (q & 3)))); };
-  if (cnt >= 16 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
-    constexpr int kPer = 16 / sizeof(T);
-#pragma unroll
-    for (int v = 0; v < 16 / kPer; ++v) {
-      __align__(16) T x[kPer];
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) x[q] = spin(kPer * v + q);
-      reinterpret_cast<uint4*>(p)[v] = *reinterpret_cast<const uint4*>(x);
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-      if (q < cnt) p[q] = spin(q);
-  }
+  if (cnt >= 16) store_spins16<true>(p, w, cnt);
+  else store_spins16<false>(p, w, cnt);
 }
 
 // int8 [B][n] -> T [B][ldx] and T [n][ldt] (transposed through a 64 x 64 tile).
 // Bound by its writes; a thread moves 16 spins with 16-byte accesses (one spin
-// and 2-byte stores per thread took 13 us for 4096 x 1000 in BF16, this 9).
+// and 2-byte stores per thread took 13 us for 4096 x 1000 in BF16, this 9).  Rows
+// that don't start on such a boundary are cut from aligned words, and every piece
+// is stored whole (with single bytes for these and for the last piece of a row 8192 x
+// 301 spins took 8.1 us, so 3.8).
 constexpr int kCvt = 64, kCvtLd = kCvt + 4;
 template <typename T>
 __global__ void __launch_bounds__(256) spins_convert_kernel(int B, int n, const int8_t* __restrict__ S,
@@ -465,9 +471,17 @@ __global__ void __launch_bounds__(256) spins_convert_kernel(int B, int n, const 
   if (b0 + r < B && i0 + c < n) {
     const int8_t* src = S + (size_t)(b0 + r) * n + i0 + c;
     const int cnt = min(16, n - i0 - c);
-    if (cnt == 16 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(src), word = at & ~(uintptr_t)3;
+    const uintptr_t first = reinterpret_cast<uintptr_t>(S), end = first + (size_t)B * n;
+    if ((at & 15) == 0 && at + 16 <= end) {
       const uint4 v = __ldg(reinterpret_cast<const uint4*>(src));
       w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+    } else if (word >= first && word + 20 <= end) {  // the five words lie inside the array
+      uint32_t x[5];
+#pragma unroll
+      for (int q = 0; q < 5; ++q) x[q] = __ldg(reinterpret_cast<const uint32_t*>(word) + q);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w[q] = __funnelshift_r(x[q], x[q + 1], 8 * (int)(at & 3));
     } else {
 #pragma unroll
       for (int q = 0; q < 16; ++q)

@@ -90,8 +90,6 @@ using namespace tc;
 // Instruction descriptor of the 128 x 128 tile.
 constexpr uint32_t kIdesc = idesc_bf16(BM, BN);
 
-__device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + expf(-x)); }
-
 // Sum of v over the 32 lanes for 16 columns by recursive halving: afterwards
 // lane l holds the warp's sum of column colsum16_col(l) (lanes 2c and 2c+1
 // hold the same value).
@@ -459,7 +457,15 @@ __global__ void __launch_bounds__(threads_of(OP), Stages<KC>::kMinBlocks)
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
         v[q] += bias_s[lb + q];
-        x[q] = g.act == VQMC_ACT_RELU ? fmaxf(v[q], 0.0f) : sigmoidf_(v[q]);
+      }
+      if (g.act == VQMC_ACT_RELU) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) x[q] = fmaxf(v[q], 0.0f);
+      } else {  // 1 / (1 + exp(-a)), the sixteen exponentials first (one by one the op took 10.5 us for 301 x 130 x 64, so 9.5)
+#pragma unroll
+        for (int q = 0; q < 16; ++q) x[q] = 1.0f + expf(-v[q]);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) x[q] = 1.0f / x[q];
       }
       if (g.pre) {
         float* p = g.pre + (size_t)m * g.ldpre + nb;

@@ -53,9 +53,9 @@ inline cudaError_t allow_smem(OncePerDevice& once, const Kernels& set, int bytes
   });
 }
 
-// lane 0's value, which the compiler then knows to be the same in all lanes: it
-// keeps the control flow that depends on it free of the reconvergence code
-// that a shuffle behind a possibly divergent branch costs (some 8 instructions)
+// lane 0's value, for control flow that is the same in all lanes of a warp: the
+// samplers and GEMMs are faster where warp indexes and loop bounds are passed through
+// it (figures in sampler_tc.cu, with its other changes)
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 // The samplers read rows in groups: their weight copies have zero rows past the

@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(kFinishThreads)
 // the conversion to FP32).  Integer energies: stats_int_kernel below.
 // FP64 runs at 1/64 of the FP32 rate and bounds this kernel, so that only the
 // sums are FP64: the extremes are taken in FP32 and the quotients by one thread
-// (a division is some 30 instructions: computed by every thread, with FP64
-// extremes, 1024 energies took 19 us and 8192 took 41 us).
+// (computed by every thread, with FP64 extremes, 1024 energies took 19 us and 8192
+// took 41; now 10 and 24).
 __global__ void __launch_bounds__(1024) stats_kernel(int B, const float* __restrict__ E, double* __restrict__ out,
                                                      float* __restrict__ coef, uint32_t* __restrict__ err,
                                                      DevState* ds, float beta1, float beta2) {

@@ -23,6 +23,7 @@
 // 144 -> 12 us with the batch split.
 #include <algorithm>
 
+#include "f32x2.cuh"
 #include "gemm.cuh"
 
 namespace vqmc {
@@ -41,21 +42,8 @@ struct Tile {
   static constexpr int kSmem = kStages * kStage * 4;
 };
 
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + expf(-x)); }
 
-__device__ __forceinline__ uint64_t dup2(float x) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
-  return r;
-}
 // 16 bytes to shared memory, the first `bytes` of them from src, zeros beyond
 __device__ __forceinline__ void cp16(uint32_t dst, const float* src, int bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
@@ -186,7 +174,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
         }
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
-          const uint64_t ai = dup2(kk == 0 ? a[i].x : kk == 1 ? a[i].y : kk == 2 ? a[i].z : a[i].w);
+          const float av = kk == 0 ? a[i].x : kk == 1 ? a[i].y : kk == 2 ? a[i].z : a[i].w;
+          const uint64_t ai = pack2(av, av);
 #pragma unroll
           for (int j = 0; j < TN / 2; ++j) acc2[i][j] = fma2(ai, b[j], acc2[i][j]);
         }
@@ -195,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_simt_kernel(const GemmArgs<f
   }
 
   // ---------------------------------------------------------------- epilogue
-  // columns in groups of four: group q starts at n0 + 64 q + 4 tx
+  // columns in groups of four: group q starts at n0 + column(q)
   const int mb = m0 + ty * TM;
   float acc[TM][TN];
 #pragma unroll

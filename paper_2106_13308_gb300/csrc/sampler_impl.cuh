@@ -29,19 +29,23 @@
 // neighbouring pairs (one octet) of one virtual warp, so the solver finishes
 // the tree from its 8 leaves and the partial sums of the other octets.
 //
-// What bounds it: the chain from one draw to the next (about 220 cycles, on two
-// of the CTA's eight warps) up to about 1000 hidden units, beyond it the issue
-// slots and shared-memory reads of the Z and U phases (2 bytes per multiply-add;
+// What bounds it: up to about 1000 hidden units the chain from one draw to the next
+// (about 220 cycles, on two of the CTA's eight warps) with the Z and U phases before
+// and after a block's draws (at n = h = 1000 some 350 cycles a draw), beyond it the
+// issue slots and shared-memory reads of these phases (2 bytes per multiply-add;
 // at n = h = 2000 55% of the issue slots and 60% of the load/store pipe are busy);
 // two CTAs on an SM overlap one's draws with the other's GEMMs.  Measured
 // (GB300), against one step at a time with a reduction over the CTA's lanes for
 // every draw: a sampling and energy pass at n = h = 1000, 1024 samples (BF16)
 // 1457 -> 293 us; a training step at n = h = 2000, 8192 samples (BF16) 9194 ->
-// 4118 us; the draws alone at n = 10000, h = 2000, 2048 samples (FP32) 7780 ->
-// 5250 us (16 TFLOP/s).  The code stays near the instruction cache's 32 KB: at
-// 47 KB (loops peeled, branches not known to be uniform) it ran at 2.7 cycles per
-// instruction.  No per-step store in the solver (25 cycles each, 70 behind a
-// divergent branch): the spins are written after a block.
+// 4013 us; the draws alone at n = 10000, h = 2000, 2048 samples (FP32) 7800 ->
+// 5040 us (16 TFLOP/s).  Loops are rolled and branches uniform: peeled and with
+// branches on lane values it ran at 2.7 cycles per instruction.  No per-step store in
+// the solver (25 cycles each, 70 behind a divergent branch): the spins are written
+// after a block.
+//
+// Where it is not the faster one (many units completing at a step, or a small model's
+// large batch), sampler.cu takes the sampler of sampler_steps.cuh: the same bits.
 #pragma once
 
 #include <type_traits>
@@ -153,8 +157,8 @@ struct Block {
   int e0, e1, grp, pad;
 };
 
-// count_deg_le and degree in 32 bits: n h < 2^32 for every model whose
-// weights fit the GPU (h <= 5120).
+// count_deg_le and degree in 32 bits: n h < 2^31 for every model (h <= 5120; a sparse
+// instance has n <= 51,200, a dense one n^2 FP32 couplings in device memory).
 __device__ __forceinline__ int complete_before(int e, int n, int h) {  // units with m(k) <= e
   if (e < 1) return 0;
   if (n <= 1) return h;
@@ -324,7 +328,7 @@ struct BlockSampler {
   // l of a sample holds leaf l of the group's octet.  The chain from one draw
   // to the next (the newest unit's pre-activation and act, its leaf's FMA, four
   // levels of sums, three shuffles, b2, the other virtual warps' trees, the
-  // compare) is about 200 cycles; a spin has two values, so both logits of step
+  // compare) is about 220 cycles; a spin has two values, so both logits of step
   // t + 1 are begun before spin t is known, and each iteration finishes the two
   // logits of step t beside the first half of step t + 1's.  Only the units
   // that complete with spin t differ between the two.  Nothing is stored per
@@ -514,9 +518,8 @@ __device__ __forceinline__ void write_block(const SamplerArgs& g, const Block& b
   }
 }
 
-// The steady state of the kernel has to fit the instruction cache (the phases
-// alternate every few thousand cycles, and a miss costs several hundred): the
-// activation is a template parameter, and loops are unrolled no further than
+// The phases alternate every few thousand cycles, so the kernel's code is kept small:
+// the activation is a template parameter, and loops are unrolled no further than
 // their operands' latency asks for.
 template <typename WT, int GW, bool RELU>
 __global__ void __launch_bounds__(kThreads, 2) sampler_kernel(const SamplerArgs g) {

@@ -41,15 +41,15 @@
 // then the helpers (models of few units per block), and some 3,300 cycles from one
 // block's last draw to the next one's first.  Measured (GB300, n = 10000, h =
 // 2000, 1024 samples with log pi): 1264 -> 726 us; n = 500, h = 193: 138 -> 85
-// us; n = 10000, h = 424: 804 -> 505 us.  What that took, the arithmetic unchanged: warp-uniform control flow made
-// known to the compiler (the warp index, the segment bounds) and one elected
-// thread per issuing warp; one copy of each piece of code (280 -> 90 KB; the
-// instruction cache holds 32); predicated stores in place of branches; log pi
-// and the next block's schedule moved to the helpers.
+// us; n = 10000, h = 424: 804 -> 505 us.  What that took, the arithmetic unchanged:
+// warp-uniform values for the warp index and the segment bounds and one elected
+// thread per issuing warp; one copy of each piece of code; predicated stores in
+// place of branches; log pi and the next block's schedule moved to the helpers.
 #include <algorithm>
 #include <type_traits>
 
 #include "gemm.cuh"
+#include "f32x2.cuh"
 #include "sampler.cuh"
 #include "tc_ptx.cuh"
 
@@ -142,20 +142,8 @@ struct TcArgs {
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-// FP32 pairs for fma.rn.f32x2 (two IEEE FP32 FMAs per instruction)
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
 // the two BF16 weights of a word, widened (exactly) to an FP32 pair
-__device__ __forceinline__ uint64_t bf2(uint32_t w) { return pk2(bf_lo(w), bf_hi(w)); }
+__device__ __forceinline__ uint64_t bf2(uint32_t w) { return pack2(bf_lo(w), bf_hi(w)); }
 
 // *p = x where ok holds, as a predicated store (a branch around one costs the
 // warp some 70 cycles)
@@ -224,35 +212,35 @@ __device__ __forceinline__ void solve(const float* Pr, const bf16* Vr, const bf1
     const uint4* vr = reinterpret_cast<const uint4*>(Vr + e * kLdW);
     const float4* hv = reinterpret_cast<const float4*>(hh);
     // four FP32 accumulators a0..a3 as the pairs (a0, a1), (a2, a3)
-    uint64_t a01 = pk2(Zs[e * kZld + s_me], 0.0f), a23 = pk2(0.0f, 0.0f);
+    uint64_t a01 = pack2(Zs[e * kZld + s_me], 0.0f), a23 = pack2(0.0f, 0.0f);
 #pragma unroll
     for (int c = 0; c <= PH; ++c) {
       const uint4 v = vr[c];
       const float4 x = hv[2 * c], y = hv[2 * c + 1];
-      a01 = fma2(bf2(v.x), pk2(x.x, x.y), a01);
-      a23 = fma2(bf2(v.y), pk2(x.z, x.w), a23);
-      a01 = fma2(bf2(v.z), pk2(y.x, y.y), a01);
-      a23 = fma2(bf2(v.w), pk2(y.z, y.w), a23);
+      a01 = fma2(bf2(v.x), pack2(x.x, x.y), a01);
+      a23 = fma2(bf2(v.y), pack2(x.z, x.w), a23);
+      a01 = fma2(bf2(v.z), pack2(y.x, y.y), a01);
+      a23 = fma2(bf2(v.w), pack2(y.z, y.w), a23);
     }
     float a0, a1, a2, a3;
-    upk2(a01, a0, a1);
-    upk2(a23, a2, a3);
+    unpack2(a01, a0, a1);
+    unpack2(a23, a2, a3);
     return (a0 + a1) + (a2 + a3);
   };
   // this lane's partial sums of the recent units of chunks PH .. 3 += sv * W1 of step row el
   auto wrow = [&](auto ph, int el, float sv) {
     constexpr int PH = decltype(ph)::value;
     const uint4* wr = reinterpret_cast<const uint4*>(Wr + el * kLdW);
-    const uint64_t s2 = pk2(sv, sv);
+    const uint64_t s2 = pack2(sv, sv);
 #pragma unroll
     for (int c = PH; c < 4; ++c) {
       const uint4 w = wr[c];
       const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        uint64_t pp = pk2(P[8 * c + 2 * j], P[8 * c + 2 * j + 1]);
+        uint64_t pp = pack2(P[8 * c + 2 * j], P[8 * c + 2 * j + 1]);
         pp = fma2(bf2(ww[j]), s2, pp);
-        upk2(pp, P[8 * c + 2 * j], P[8 * c + 2 * j + 1]);
+        unpack2(pp, P[8 * c + 2 * j], P[8 * c + 2 * j + 1]);
       }
     }
   };
@@ -620,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_wait(smem_u32(drain), 0u, g.err);
     }
   } else {
-    // ---------------------------- warps 0-3 and 6-7: blocks, solver
+    // ---------------- warps 0-3 and 6-9: tensor-memory reads, solver, helpers
     // Warps 0, 1, 6 and 7 are the solver, one warp on each SM sub-partition
     // (warp w runs on w % 4): the solver is issue-bound, and the producer and
     // MMA warps that share sub-partitions 0 and 1 with it issue little.

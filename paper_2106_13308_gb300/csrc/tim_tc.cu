@@ -21,14 +21,14 @@
 // (128 outputs x 64 units) with TMA; warp 9 issues the MMAs into two
 // accumulators, so that one output tile's epilogue runs beside the next
 // one's MMAs.  They wait with try_wait, which suspends: polling took a fifth of
-// the epilogue's issue slots.  Every wait is bounded: after a failed one the CTA raises the
-// timeout bit and runs on without waiting.
+// the epilogue's issue slots.  Every wait is bounded: after a failed one the CTA
+// raises the timeout bit and runs on without waiting.
 //
-// What bounds it: the epilogue, one exponential, one logarithm and some 11 more
-// instructions for each of the B n n / 2 outputs that do not cancel (185 M of
-// them at n = 500, B = 1024: 65 us of issue slots).  Measured there, h = 193
+// What bounds it: the issue slots of the epilogue, an exponential and a logarithm for
+// every output of the tiles that are not skipped (185 M at n = 500, B = 1024, of which
+// the B n n / 2 = 128 M that do not cancel are wanted).  Measured there, h = 193
 // (GB300), a training step: 1141 us with the rows and their spins written to
-// memory and read back by the general GEMM, 430 us with this kernel (0.21 ms
+// memory and read back by the general GEMM, 432 us with this kernel (0.21 ms
 // of it; 145 M warp instructions, 61% of the issue slots).
 #include <algorithm>
 

@@ -35,7 +35,7 @@ iterations over 5 seeds.
 A fourth, many independent instances trained together: 64 Max-Cut instances of
 uneven size (n ~ U{100..5000}, G(n, 6/(n-1)), weights +-1, hidden units h = n,
 512 samples each), BF16, stepped as one CUDA graph launch per batched
-iteration under the schedule and sampler layouts the library's autotuner
+iteration under the schedule and summation orders the library's autotuner
 picked; reported under "batched" beside the same batch stepped call by call,
 with the lower bound of the longest member's iteration alone.
 

@@ -333,16 +333,14 @@ __global__ void wgrad_sum_kernel(int op, int M, int N, int parts, const float* _
   float s = 0.0f;
   if ((nn < count_deg_le(m, n, h)) == (op == kOpDV)) {
     const float* p = part + (size_t)m * N + nn;
-    int z = 0;
 #pragma unroll 1
-    for (; z + 8 <= parts; z += 8) {  // eight loads in flight: their latency bounds the sum
+    for (int z = 0; z < parts; z += 8) {  // eight loads in flight: their latency bounds the sum
       float x[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) x[q] = p[(size_t)(z + q) * M * N];
+      for (int q = 0; q < 8; ++q) x[q] = z + q < parts ? p[(size_t)(z + q) * M * N] : 0.0f;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) s += x[q];
+      for (int q = 0; q < 8; ++q) s += x[q];  // (a zero past the last part changes nothing: s is never -0)
     }
-    for (; z < parts; ++z) s += p[(size_t)z * M * N];
   }
   gout[(size_t)m * ldg + nn] = s;
 }
